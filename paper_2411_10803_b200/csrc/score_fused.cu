@@ -389,7 +389,7 @@ struct __align__(8) Barriers {
   uint64_t eready[kMaxBufs];     // exp -> add warps: exponentials of a head are in tensor memory
   uint64_t tempty[kMaxBufs];     // add warps -> MMA: tensor-memory buffer free
   uint64_t sfull[kMaxSlots];    // all CTAs' (max, sum) pairs of a head have arrived
-  uint64_t fin;                  // add warps meet before / after staging the head sums
+  uint64_t fin;                  // add warps meet before staging the head sums
   uint64_t ph;                   // add warps meet once per head (per-head maxima of Eq. 10)
   uint64_t gsent[kMaxBufs];      // grid plans: exp warps -> publishing thread: this CTA's pairs of a head are in global memory
   uint64_t gfull[kMaxGatherSlots];   // filter tail: a gathered row has landed in its slot
@@ -596,14 +596,16 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
 
   // End of the score part, executed by every thread: tensor memory freed, and no CTA goes on
   // while a peer may still write into its shared memory.  The cluster barrier also orders every
-  // CTA's g_out / i_out stores before what the filter tail loads.  (In the filter kernel each
-  // warp role calls this from its own branch and continues there with its part of the tail, so
-  // every role keeps the register count setmaxnreg gave it; no second setmaxnreg is needed.)
+  // CTA's g_out / i_out stores before what the filter tail loads.  (Each warp role
+  // calls this from its own branch - in the filter kernel it continues there with its part of the
+  // tail - so every role keeps the register count setmaxnreg gave it; no second setmaxnreg is needed.)
   __shared__ int32_t kept_total_s;
-  auto common_exit = [&]() {
+  auto common_exit = [&](auto&& finish) {
     __syncwarp();   // a warp whose lane 0 had a role of its own is whole again before the aligned instructions below
     tc_fence_before();
     cta_sync();
+    finish();       // (exp warps: the scores from the staged head sums)
+    if (p.gx) cta_sync();   // every score of this CTA is stored before the request's CTAs meet below
     if (p.gx) {
       // grid plan: the request's CTAs are no cluster.  In the filter kernel they meet through a
       // counter in global memory: every CTA's scores are stored before any CTA selects.  (A CTA
@@ -902,10 +904,12 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     }
     if constexpr (FILTER) {
       // filter tail, TMA / MMA warps: nothing to do but to meet the others
-      common_exit();
+      common_exit([] {});
       if (cluster_gave_up()) { leave_after_give_up(ft.sel.kept_cnt); return; }
       cta_sync();   // pairs with the barrier after the selection
       return;
+    } else {
+      common_exit([] {});
     }
   } else if (warp < kExpWarps) {
     // ---------------- exp warps ----------------
@@ -1078,19 +1082,70 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       if (lane == 0) mbar_arrive(smem_u32(&bars.eready[buf]));
       if (threadIdx.x == 0) MD_TRACE(h, 4);
     }
+    // Head mean -> column sum (Eq. 8) and column max (Eq. 10) over the text rows, by the eight exp
+    // warps once the add warps have staged the head sums: a warp takes 32 keys and an eighth of the
+    // rows at a time, and the eighths of a key meet in shared memory.  (By the four add warps alone,
+    // a key per thread and all rows one after the other, it took 3.8 us at 320 keys per CTA.)
+    auto finish_scores = [&]() {
+      if (*abort_flag != 0) return;   // (the same answer in every thread: nothing raises it any more)
+      constexpr int kParts = 8;
+      const float* const mat = reinterpret_cast<const float*>(stage_ptr);
+      const int ld = p.tk | 1;
+      float2* const parts = reinterpret_cast<float2*>(stage_ptr + ((static_cast<size_t>(NROWS) * ld * 4 + 15) & ~static_cast<size_t>(15)));
+      const int per_part = (p.N + kParts - 1) / kParts, n_groups = (p.tk + 31) / 32;
+      for (int x = warp; x < n_groups * kParts; x += kExpWarps) {
+        const int c = (x / kParts) * 32 + lane, part = x % kParts;
+        const int r1 = min(p.N, (part + 1) * per_part);
+        if (c < p.tk) {
+          float sum = 0.0f, mx = -INFINITY;
+#pragma unroll 8
+          for (int r = part * per_part; r < r1; ++r) {
+            const float v = mat[r * ld + c];
+            sum += v;
+            mx = fmaxf(mx, v);
+          }
+          parts[part * p.tk + c] = make_float2(sum, mx);
+        }
+      }
+      pdl_wait();
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      for (int c = threadIdx.x; c < p.tk; c += kExpThreads) {
+        const int j = static_cast<int>(rank) * p.tk + c - p.vis_start;   // vision-relative index
+        if (j < 0 || j >= p.M) continue;
+        float sum = 0.0f, mx = -INFINITY;
+#pragma unroll
+        for (int x = 0; x < kParts; ++x) {
+          const float2 v = parts[x * p.tk + c];
+          sum += v.x;
+          mx = fmaxf(mx, v.y);
+        }
+        if constexpr (PH) mx = ph_stage[c] * (1.0f / kPhScale);
+        const bool present = j < Mb;    // beyond the request's own tokens: zeros
+        float gv = present ? sum * p.inv_heads : 0.0f, iv = present ? mx * p.inv_heads : 0.0f;
+        if (p.combine) {                // the text rows before row0 were scored by the launch before this one
+          gv += p.g_out[static_cast<size_t>(b) * p.M + j];
+          iv = fmaxf(iv, p.i_out[static_cast<size_t>(b) * p.M + j]);
+        }
+        p.g_out[static_cast<size_t>(b) * p.M + j] = gv;
+        p.i_out[static_cast<size_t>(b) * p.M + j] = iv;
+      }
+      if (threadIdx.x == 0) MD_TRACE(0, 10);   // scores stored
+    };
     if constexpr (FILTER) {
       // filter tail, exp warps: selection of this request.  Dynamic shared memory is free by now:
       // all copies have landed, all MMAs have read them and every statistics pair sent to this CTA
       // has been consumed.  Each CTA of the cluster runs the same selection on its own (identical
       // inputs, fixed order: identical lists); rank 0 stores the list.
       __shared__ SelectShared sel_sh;
-      common_exit();
+      common_exit(finish_scores);
       if (cluster_gave_up()) { leave_after_give_up(ft.sel.kept_cnt); return; }
       pdl_wait();   // the outputs written below may still be read by an earlier kernel in the stream
       filter_select(ft.sel, sel_sh, b, threadIdx.x, rank == 0, kept_list, &kept_total_s);
       if (threadIdx.x == 0) MD_TRACE(0, 12);   // selection done
       cta_sync();   // the list is complete: the copy thread may start
       return;
+    } else {
+      common_exit(finish_scores);
     }
   } else {
     // ---------------- add warps ----------------
@@ -1123,31 +1178,27 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       float f;                                 // factor of this CTA's exponentials of the row
       if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.sfull[slot]), sph, abort_flag, wait_limit))) break;
       if (tid_a == 0) MD_TRACE(h, 5);
-      if (p.gx) {
-        // grid plan: one merged pair per CTA in the slot; this CTA's own stabilisers are still in
-        // its shared memory (until the buffer is released below)
-        const float2* srow = stats + slot * slot_pairs + row;
-        float m = -INFINITY;
-        for (int c = 0; c < p.cluster; ++c) m = fmaxf(m, srow[c * NROWS].x);
-        float l = 0.0f;
-        for (int c = 0; c < p.cluster; ++c) {
-          const float2 v = srow[c * NROWS];
-          l = fmaf(v.y, ex2(v.x - m), l);
+      {
+        // Statistics of this row over the whole key range, relative to this CTA's own stabiliser:
+        // f = 1 / sum over CTAs of l_c 2^(m_c - m_own).  Independent terms, four loads in flight: the
+        // loop is on every head's serial path (as a maximum first and a sum over the CTAs second it
+        // took 0.5 us with 2 CTAs and 0.8 us with 16).  A sum that overflows means that this CTA's
+        // share is below 2^-127: f = 0.  Grid plans: one merged pair per CTA in the slot; this CTA's own
+        // stabilisers are still in its shared memory (until the buffer is released below).
+        const float2* const srow = stats + slot * slot_pairs + row;
+        const float own = p.gx ? own_pairs[buf * NROWS + row].x : srow[rank * NROWS].x;
+        float l0 = 0.0f, l1 = 0.0f;
+#pragma unroll 1
+        for (int c = 0; c < p.cluster; c += 4) {
+          float2 v[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) v[e] = c + e < p.cluster ? srow[(c + e) * NROWS] : make_float2(-INFINITY, 0.0f);
+          l0 = fmaf(v[0].y, ex2(v[0].x - own), l0);     // an empty pair is (-inf, 0): contributes 0
+          l1 = fmaf(v[1].y, ex2(v[1].x - own), l1);
+          l0 = fmaf(v[2].y, ex2(v[2].x - own), l0);
+          l1 = fmaf(v[3].y, ex2(v[3].x - own), l1);
         }
-        const float inv_l = 1.0f / l;
-        f = ex2(own_pairs[buf * NROWS + row].x - m) * inv_l;
-      } else {
-        // statistics of this row over the whole key range: every CTA's pairs
-        const float2* srow = stats + slot * slot_pairs + row;
-        float m = -INFINITY;
-        for (int c = 0; c < p.cluster; ++c) m = fmaxf(m, srow[c * NROWS].x);
-        float l = 0.0f;
-        for (int c = 0; c < p.cluster; ++c) {
-          const float2 v = srow[c * NROWS];
-          l = fmaf(v.y, ex2(v.x - m), l);     // an empty pair is (-inf, 0): contributes 0
-        }
-        const float inv_l = 1.0f / l;
-        f = ex2(srow[rank * NROWS].x - m) * inv_l;
+        f = own == -INFINITY ? 0.0f : 1.0f / (l0 + l1);   // (own = -inf: the row sees none of this CTA's keys)
       }
       if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.eready[buf]), bph, abort_flag, wait_limit))) break;
       if (tid_a == 0) MD_TRACE(h, 6);
@@ -1236,11 +1287,11 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       if (tid_a == 0) MD_TRACE(h, 7);
     }
 
-    // head mean -> column sum (Eq. 8) and column max (Eq. 10) over the text rows
+    // the head sums go to shared memory, where the exp warps reduce them over the text rows
     mbar_arrive(smem_u32(&bars.fin));
     if (__all_sync(0xffffffffu, h == p.H && mbar_wait(smem_u32(&bars.fin), 0u, abort_flag, wait_limit))) {
       // all TMA copies have landed and all MMAs have read them: the staging area is free
-      float* mat = reinterpret_cast<float*>(stage_ptr);
+      float* const mat = reinterpret_cast<float*>(stage_ptr);
       const int ld = p.tk | 1;
       if (row < p.N) {
 #pragma unroll
@@ -1252,38 +1303,15 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           }
         }
       }
-      mbar_arrive(smem_u32(&bars.fin));
-      const bool staged = mbar_wait(smem_u32(&bars.fin), 1u, abort_flag, wait_limit);
-      pdl_wait();
-      for (int c = tid_a, x = 0; staged && c < p.tk; c += kAddThreads, ++x) {
-        const int j = static_cast<int>(rank) * p.tk + c - p.vis_start;   // vision-relative index
-        if (j < 0 || j >= p.M) continue;
-        float s = 0.0f, mx = -INFINITY;
-        for (int r = 0; r < p.N; ++r) {
-          const float v = mat[r * ld + c];
-          s += v;
-          mx = fmaxf(mx, v);
-        }
-        if constexpr (PH) {
-          mx = 0.0f;   // (x < PHK always; a compile-time unrolled pick keeps ph_acc in registers)
+      if constexpr (PH) {
 #pragma unroll
-          for (int y = 0; y < PHK; ++y) mx = (y == x) ? ph_acc[y] : mx;
-          mx *= 1.0f / kPhScale;
-        }
-        const bool present = j < Mb;    // beyond the request's own tokens: zeros
-        float gv = present ? s * p.inv_heads : 0.0f, iv = present ? mx * p.inv_heads : 0.0f;
-        if (p.combine) {                // the text rows before row0 were scored by the launch before this one
-          gv += p.g_out[static_cast<size_t>(b) * p.M + j];
-          iv = fmaxf(iv, p.i_out[static_cast<size_t>(b) * p.M + j]);
-        }
-        p.g_out[static_cast<size_t>(b) * p.M + j] = gv;
-        p.i_out[static_cast<size_t>(b) * p.M + j] = iv;
+        for (int x = 0; x < PHK; ++x)
+          if (tid_a + x * kAddThreads < p.tk) ph_stage[tid_a + x * kAddThreads] = ph_acc[x];
       }
-      if (tid_a == 0) MD_TRACE(0, 10);     // scores stored
     }
     if constexpr (FILTER) {
       // filter tail, add warps: row r of the compacted outputs is copied by CTA r mod cluster
-      common_exit();
+      common_exit([] {});
       if (cluster_gave_up()) { leave_after_give_up(ft.sel.kept_cnt); return; }
       pdl_wait();
       cta_sync();   // the exp warps have finished the selection
@@ -1293,11 +1321,12 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         MD_TRACE(0, 13);   // gather done
       }
       return;
+    } else {
+      common_exit([] {});
     }
   }
 
-  common_exit();   // (score-only kernel; the filter kernel's roles have left above)
-  if (cluster_gave_up()) leave_after_give_up(nullptr);
+  if (cluster_gave_up()) leave_after_give_up(nullptr);   // (score-only kernel; the filter kernel's roles have left above)
 }
 
 // ---- host side ------------------------------------------------------------------------------------
