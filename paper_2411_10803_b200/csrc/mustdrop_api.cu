@@ -157,7 +157,8 @@ mustdrop_status_t mustdrop_filter_plan(const mustdrop_config_t* c, mustdrop_plan
     const bool force_split = c->debug_score_variant == MUSTDROP_DEBUG_VARIANT_ROW_SPLIT;
     const bool force_grid = c->debug_score_variant == MUSTDROP_DEBUG_VARIANT_GRID;
     const double k_mb = 256.0e-6 * r.B * r.H * r.L;
-    const double two_pass_us = k_mb * (0.6 + 0.7 * r.N / 128.0);   // the two-pass kernel's measured rate
+    // the two-pass kernel's measured rate, and its second pass's walk over the heads
+    const double two_pass_us = k_mb * (0.6 + 0.7 * r.N / 128.0) + 3.0 * r.H;
     double chosen_us = two_pass_us;
     p->row_split = 0;
     if (allow_fused && !force_split && !force_grid && plan_score_fused(r, p->sm_count, forced_cluster, &p->fused)) {
@@ -180,21 +181,16 @@ mustdrop_status_t mustdrop_filter_plan(const mustdrop_config_t* c, mustdrop_plan
     // the head mean, which two launches over disjoint rows cannot combine afterwards.)
     if (allow_fused && r.N > 64 && !r.per_head_max && !force_grid) {
       mustdrop::FusedGeometry ga, gb;
-      // clusters small enough for both launches to be resident at once, if such a plan exists
-      const int fit = p->sm_count / (2 * r.B);
-      bool ok = fit >= 1 && plan_score_fused(r, p->sm_count, forced_cluster, &ga, 0, 64, fit) &&
-                plan_score_fused(r, p->sm_count, forced_cluster, &gb, 64, r.N - 64, fit);
-      if (!ok)
-        ok = plan_score_fused(r, p->sm_count, forced_cluster, &ga, 0, 64) &&
-             plan_score_fused(r, p->sm_count, forced_cluster, &gb, 64, r.N - 64);
-      if (ok) {
-        const bool together = r.B * (ga.cluster + gb.cluster) <= p->sm_count;   // both launches resident at once
-        const double split_us = together ? 1.15 * (ga.est_us > gb.est_us ? ga.est_us : gb.est_us) : ga.est_us + gb.est_us;
+      if (plan_score_fused(r, p->sm_count, forced_cluster, &ga, 0, 64) &&
+          plan_score_fused(r, p->sm_count, forced_cluster, &gb, 64, r.N - 64)) {
+        // (the second launch reads no keys before the first has completed)
+        const double split_us = ga.est_us + gb.est_us + 8.0;
         if (force_split || (!want && forced_cluster == 0 && split_us < chosen_us)) {
           p->score_variant = kScoreFusedCluster;
           p->row_split = 1;
           p->fused = ga;
           p->fused_b = gb;
+          chosen_us = split_us;
         }
       }
     }
@@ -204,8 +200,7 @@ mustdrop_status_t mustdrop_filter_plan(const mustdrop_config_t* c, mustdrop_plan
     if (allow_fused && !force_split && (force_grid || (!want && forced_cluster == 0))) {
       mustdrop::FusedGeometry gg;
       if (plan_score_grid(r, p->sm_count, force_grid ? forced_cluster : 0, &gg) &&
-          (force_grid || gg.est_us < (p->row_split ? 1e30 : chosen_us) * 0.9 ||
-           (p->row_split && gg.est_us < 1.15 * (p->fused.est_us > p->fused_b.est_us ? p->fused.est_us : p->fused_b.est_us)))) {
+          (force_grid || gg.est_us < chosen_us * (p->row_split ? 1.0 : 0.9))) {
         p->score_variant = kScoreFusedCluster;
         p->row_split = 0;
         p->fused = gg;
@@ -437,9 +432,9 @@ int32_t mustdrop_plan_describe(const mustdrop_plan_t* plan, char* buf, size_t n)
                           g.cluster, g.tk, g.n_q, g.n_buf, g.n_slot, mustdrop_plan_filter_launches(plan));
     else
       len = std::snprintf(text, sizeof(text),
-                          "fused tcgen05 score%s: cluster %d, %d keys per CTA, %s %d/%d, %d tensor-memory buffers, "
+                          "fused tcgen05 score%s: cluster %d, %d head group(s), %d keys per CTA, %s %d/%d, %d tensor-memory buffers, "
                           "%d statistics slots, %d clusters resident; filter = %d launch(es)",
-                          plan->row_split ? " (text rows in two launches; second launch)" : "", g.cluster, g.tk,
+                          plan->row_split ? " (text rows in two launches; second launch)" : "", g.cluster * g.groups, g.groups, g.tk,
                           g.split ? "query/key-half rings" : "stages", g.n_q, g.split ? g.n_k : 0, g.n_buf, g.n_slot,
                           g.resident, mustdrop_plan_filter_launches(plan));
   } else {

@@ -25,7 +25,8 @@ enum ScoreVariant : int32_t {
 // Launch geometry of the fused score kernel.
 struct FusedGeometry {
   int32_t halves;     // 2: two M=64 tiles per head (N <= 64); 1: one M=128 tile
-  int32_t cluster;    // CTAs per request
+  int32_t cluster;    // CTAs that split the keys of a head
+  int32_t groups;     // head groups: a request has groups x cluster CTAs
   int32_t tk;         // keys per CTA
   int32_t cpl;        // tensor-memory columns per lane and head (= tk / halves)
   int32_t n_q, n_k;   // whole stages: n_q of them (n_k unused); split: rings of n_q query tiles and n_k key half-tiles
@@ -108,7 +109,7 @@ cudaError_t launch_score_two_pass(const mustdrop_plan& p, const void* q_text, co
                                   float* g_out, float* i_out, void* rowstats, cudaStream_t stream,
                                   const int32_t* vis_cnt = nullptr);
 bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, FusedGeometry* out, int row0 = 0,
-                      int n_rows = 0, int max_cluster = 0);
+                      int n_rows = 0);
 // Grid plan of the same kernel (all CTAs of the batch resident at once, statistics through global
 // memory); false when the batch leaves fewer than two CTAs per request or the shape does not fit.
 bool plan_score_grid(const Resolved& r, int sm_count, int forced_ctas, FusedGeometry* out);

@@ -28,6 +28,7 @@
 #include <cuda_fp16.h>
 
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <new>
 #include <type_traits>
@@ -56,6 +57,7 @@ constexpr int kMaxBufs = 8;                 // ... more when the columns per hea
 constexpr int kMaxSlots = 2 * kMaxBufs;     // statistics slots = 2 x buffers: a peer's exp warps run at most that far ahead of our add warps
 constexpr int kTmemCols = 512;
 constexpr int kMaxGatherSlots = 8;         // rows in flight per CTA in the gather tail of the filter kernel
+constexpr size_t kMinSmem = 116 * 1024;     // least dynamic shared memory of a CTA, so that two (each wanting all of tensor memory) never share an SM
 constexpr int kKeptListBytes = kMaxVis * 4; // the request's kept indices, at the start of dynamic shared memory
 constexpr long long kWaitCycles = 200000000LL;   // ~0.1 s at 2 GHz; no legitimate wait comes near it
 
@@ -67,7 +69,8 @@ struct FusedParams {
   int32_t H, N, L, M, vis_start, txt_start, causal;
   int32_t n_txt;                      // all text rows of the request (N is this launch's share)
   int32_t row0, combine;              // this launch covers text rows row0 .. row0 + N - 1; combine: add to / max with what g_out / i_out hold
-  int32_t cluster, tk, cpl;           // CTAs per request, keys per CTA, columns per TMEM lane
+  int32_t cluster, tk, cpl;           // CTAs that share the keys of a head, keys per CTA, columns per TMEM lane
+  int32_t groups;                     // head groups: a request has groups x cluster CTAs, each of a group's CTAs loops over the group's heads only
   int32_t n_q, n_k;                   // whole stages: n_q of them; split: ring sizes of query tiles and key half-tiles
   int32_t split;
   int32_t n_buf, n_slot;              // tensor-memory buffers, statistics slots (2 * n_buf, or 4 when tight)
@@ -171,6 +174,11 @@ __device__ __forceinline__ void st_async_f32x2(uint32_t addr, float a, float b, 
 __device__ __forceinline__ void cta_sync() { asm volatile("barrier.sync 0, %0;" ::"n"(kThreads) : "memory"); }
 __device__ __forceinline__ void st_remote_u32(uint32_t cluster_addr, uint32_t v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ float ld_cluster_f32(uint32_t cluster_addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr) : "memory");
+  return v;
 }
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -525,8 +533,13 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
   volatile int* abort_flag = &abort_flag_s;
   const long long wait_limit = p.wait_cycles;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = p.gx ? blockIdx.x % static_cast<uint32_t>(p.cluster) : cluster_cta_rank();
-  const int b = blockIdx.x / p.cluster;
+  // A request's CTAs: `groups` head groups of `cluster` CTAs each; the CTAs of a group split the keys.
+  const int req_ctas = p.cluster * p.groups;
+  const uint32_t req_rank = p.gx ? blockIdx.x % static_cast<uint32_t>(req_ctas) : cluster_cta_rank();
+  const uint32_t rank = req_rank % static_cast<uint32_t>(p.cluster);    // which keys
+  const int group = static_cast<int>(req_rank) / p.cluster;             // which heads: h0 .. h0 + n_heads - 1
+  const int h0 = group * p.H / p.groups, n_heads = (group + 1) * p.H / p.groups - h0;
+  const int b = blockIdx.x / req_ctas;
   MD_PIPE(p.workspace, 0, false, true);
   if (threadIdx.x == 0) MD_TRACE(0, 8);    // (CTA-level stamps use the event slots 8.. of head 0) kernel entry
   // dynamic shared memory: [n_q query tiles][n_k key half-tiles][stats: n_slot x cluster x NROWS float2]
@@ -604,6 +617,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     __syncwarp();   // a warp whose lane 0 had a role of its own is whole again before the aligned instructions below
     tc_fence_before();
     cta_sync();
+    if (p.groups > 1) cluster_sync_all();   // the head sums of every group are staged
     finish();       // (exp warps: the scores from the staged head sums)
     if (p.gx) cta_sync();   // every score of this CTA is stored before the request's CTAs meet below
     if (p.gx) {
@@ -641,7 +655,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       cta_sync();
     } else if (threadIdx.x == 0 && *abort_flag != 0) {
       record_status(p.workspace, MUSTDROP_ERR_TIMEOUT, blockIdx.x);
-      for (int c = 0; c < p.cluster; ++c) st_remote_u32(map_to_cta(smem_u32(&cluster_abort_s), c), 1u);
+      for (int c = 0; c < req_ctas; ++c) st_remote_u32(map_to_cta(smem_u32(&cluster_abort_s), c), 1u);
     }
     if (warp == kMmaWarp) {
       tc_fence_after();
@@ -657,7 +671,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
   // asynchronous statistics stores may still be on their way into this CTA's shared memory: give
   // them time to land and meet once more, so that no CTA's shared memory goes away under them.
   auto leave_after_give_up = [&](int32_t* kept_cnt) {
-    if (kept_cnt != nullptr && (rank == 0 || p.gx) && threadIdx.x == 0) {
+    if (kept_cnt != nullptr && (req_rank == 0 || p.gx) && threadIdx.x == 0) {
       pdl_wait();
       kept_cnt[b] = -1;   // this request's result is invalid
     }
@@ -678,15 +692,15 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       if (p.split) {
         int q_issued = 0, k_issued = 0;   // tiles started so far
         bool ok = true;
-        for (int h = 0; h < p.H && ok; ++h) {
+        for (int h = 0; h < n_heads && ok; ++h) {
           const int qi = h % p.n_q;
           if (!mbar_wait(smem_u32(&bars.qempty[qi]), (static_cast<uint32_t>(h / p.n_q) & 1u) ^ 1u, abort_flag, wait_limit)) break;
           const uint32_t qfull = smem_u32(&bars.qfull[qi]);
           const uint32_t q_dst = stage_base + qi * q_bytes;
           mbar_expect_tx(qfull, q_bytes);
           MD_TRACE(h, 0);
-          tma_load_4d(q_dst, &q_map, 0, 0, h, b, qfull);
-          tma_load_4d(q_dst + NROWS * 128u, &q_map, 64, 0, h, b, qfull);
+          tma_load_4d(q_dst, &q_map, 0, 0, h0 + h, b, qfull);
+          tma_load_4d(q_dst + NROWS * 128u, &q_map, 64, 0, h0 + h, b, qfull);
           q_issued = h + 1;
   #pragma unroll
           for (int hv = 0; hv < HALVES; ++hv) {
@@ -698,8 +712,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             const uint32_t full = smem_u32(&bars.full[ki]);
             const uint32_t k_dst = k_base + ki * kh_bytes;
             mbar_expect_tx(full, kh_bytes);
-            tma_load_4d_hint(k_dst, &k_map, 0, key0 + hv * p.cpl, h, b, full, stream_once);
-            tma_load_4d_hint(k_dst + p.cpl * 128u, &k_map, 64, key0 + hv * p.cpl, h, b, full, stream_once);
+            tma_load_4d_hint(k_dst, &k_map, 0, key0 + hv * p.cpl, h0 + h, b, full, stream_once);
+            tma_load_4d_hint(k_dst + p.cpl * 128u, &k_map, 64, key0 + hv * p.cpl, h0 + h, b, full, stream_once);
             ++k_issued;
           }
         }
@@ -718,7 +732,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         }
       } else {
         int issued = 0;
-        for (int h = 0; h < p.H; ++h) {
+        for (int h = 0; h < n_heads; ++h) {
           const int s = h % p.n_q;
           const uint32_t ph = static_cast<uint32_t>(h / p.n_q) & 1u;
           if (!mbar_wait(smem_u32(&bars.empty[s]), ph ^ 1u, abort_flag, wait_limit)) break;
@@ -729,11 +743,11 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           MD_TRACE(h, 0);
   #pragma unroll
           for (int slab = 0; slab < 2; ++slab) {
-            tma_load_4d(q_dst + slab * (NROWS * 128u), &q_map, slab * 64, 0, h, b, full);
+            tma_load_4d(q_dst + slab * (NROWS * 128u), &q_map, slab * 64, 0, h0 + h, b, full);
   #pragma unroll
             for (int hv = 0; hv < HALVES; ++hv)
               tma_load_4d_hint(k_dst + slab * (p.tk * 128u) + hv * (p.cpl * 128u), &k_map, slab * 64, key0 + hv * p.cpl,
-                               h, b, full, stream_once);
+                               h0 + h, b, full, stream_once);
           }
           issued = h + 1;
         }
@@ -749,7 +763,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     } else if (warp == kTmaWarp && lane == 1 && !p.split) {
       // trace build only: an onlooker that stamps the moment a stage's copies have landed (it tests
       // the barrier's phase and changes nothing; the MMA thread's own stamp comes when its turn does)
-      for (int h = 0; h < p.H; ++h) {
+      for (int h = 0; h < n_heads; ++h) {
         const uint32_t bar = smem_u32(&bars.full[h % p.n_q]);
         const uint32_t ph = static_cast<uint32_t>(h / p.n_q) & 1u;
         const long long t0 = clock64();
@@ -765,7 +779,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       if (p.split) {
         int k_used = 0;
         bool ok = true;
-        for (int h = 0; h < p.H && ok; ++h) {
+        for (int h = 0; h < n_heads && ok; ++h) {
           const int qi = h % p.n_q, buf = h % p.n_buf;
           const uint32_t bph = static_cast<uint32_t>(h / p.n_buf) & 1u;
           if (!mbar_wait(smem_u32(&bars.qfull[qi]), static_cast<uint32_t>(h / p.n_q) & 1u, abort_flag, wait_limit)) break;
@@ -800,7 +814,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           committed = h;
         }
       } else {
-        for (int h = 0; h < p.H; ++h) {
+        for (int h = 0; h < n_heads; ++h) {
           const int s = h % p.n_q, buf = h % p.n_buf;
           const uint32_t ph = static_cast<uint32_t>(h / p.n_q) & 1u;
           const uint32_t bph = static_cast<uint32_t>(h / p.n_buf) & 1u;
@@ -847,7 +861,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       const uint32_t target = static_cast<uint32_t>(p.cluster);   // one counted release per CTA and head
       const uint32_t slot_bytes_gx = slot_pairs * 8u;
       int ready = 0;   // heads below this one are known to be published by every CTA of the request
-      for (int h = 0; h < p.H; ++h) {
+      for (int h = 0; h < n_heads; ++h) {
         const int slot = h % p.n_slot;
         if (h >= p.n_slot) {
           const int u = h - p.n_slot;
@@ -885,7 +899,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       // pairs of each row into one, store it to global memory, then one fence and one counted
       // release for the CTA - the round trip of the fence is off the exp warps' path.
       pdl_wait();   // global memory of the workspace: not before the stream's earlier work is done
-      for (int h = 0; h < p.H; ++h) {
+      for (int h = 0; h < n_heads; ++h) {
         const int buf = h % p.n_buf;
         if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.gsent[buf]), static_cast<uint32_t>(h / p.n_buf) & 1u,
                                                abort_flag, wait_limit)))
@@ -946,7 +960,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     const bool sender = (half == 0);           // with two halves, lanes s and s+16 share a row: the lower one sends
     const uint32_t pair_idx = rank * NROWS + row;                              // this thread's pair in a slot
 
-    for (int h = g; h < p.H; h += kColGroups) {
+    for (int h = g; h < n_heads; h += kColGroups) {
       const int buf = h % p.n_buf;
       const uint32_t bph = static_cast<uint32_t>(h / p.n_buf) & 1u;
       const int slot = h % p.n_slot;
@@ -1070,7 +1084,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         if (lane == 0) mbar_arrive(smem_u32(&bars.gsent[buf]));
       } else if (sender) {
         for (int c = 0; c < p.cluster; ++c)
-          st_async_f32x2(map_to_cta(slot_addr, c), mx, lsum, map_to_cta(bar_addr, c));
+          st_async_f32x2(map_to_cta(slot_addr, group * p.cluster + c), mx, lsum, map_to_cta(bar_addr, group * p.cluster + c));
       }
       // Hand the head's exponentials to the add warps at once.  (The wait for the stores runs under
       // the other group's loop.  Handing over only when the group gets to its next head - two heads
@@ -1088,28 +1102,50 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     // a key per thread and all rows one after the other, it took 3.8 us at 320 keys per CTA.)
     auto finish_scores = [&]() {
       if (*abort_flag != 0) return;   // (the same answer in every thread: nothing raises it any more)
-      constexpr int kParts = 8;
-      const float* const mat = reinterpret_cast<const float*>(stage_ptr);
+      constexpr int kParts = 8, kRows = 8;
       const int ld = p.tk | 1;
+      // This CTA's share of the keys: all of its tile, or - with several head groups, whose CTAs of the
+      // same rank hold sums over different heads for the same keys - one part in `groups` of it.
+      const int c_lo = group * p.tk / p.groups, c_hi = (group + 1) * p.tk / p.groups;
+      const float* const mat = reinterpret_cast<const float*>(stage_ptr);
       float2* const parts = reinterpret_cast<float2*>(stage_ptr + ((static_cast<size_t>(NROWS) * ld * 4 + 15) & ~static_cast<size_t>(15)));
-      const int per_part = (p.N + kParts - 1) / kParts, n_groups = (p.tk + 31) / 32;
-      for (int x = warp; x < n_groups * kParts; x += kExpWarps) {
-        const int c = (x / kParts) * 32 + lane, part = x % kParts;
+      const int per_part = (p.N + kParts - 1) / kParts, n_strips = (c_hi - c_lo + 31) / 32;
+      for (int x = warp; x < n_strips * kParts; x += kExpWarps) {
+        const int c = c_lo + (x / kParts) * 32 + lane, part = x % kParts;
         const int r1 = min(p.N, (part + 1) * per_part);
-        if (c < p.tk) {
+        if (c < c_hi) {
           float sum = 0.0f, mx = -INFINITY;
-#pragma unroll 8
-          for (int r = part * per_part; r < r1; ++r) {
-            const float v = mat[r * ld + c];
-            sum += v;
-            mx = fmaxf(mx, v);
+#pragma unroll 1
+          for (int r = part * per_part; r < r1; r += kRows) {
+            float v[kRows];
+#pragma unroll
+            for (int e = 0; e < kRows; ++e) v[e] = 0.0f;
+            if (p.groups == 1) {
+#pragma unroll
+              for (int e = 0; e < kRows; ++e)
+                if (r + e < r1) v[e] = mat[(r + e) * ld + c];
+            }
+#pragma unroll 1
+            for (int gr = 0; gr < p.groups && p.groups > 1; ++gr) {   // (fixed order: sums do not depend on who is first)
+              const uint32_t src = map_to_cta(smem_u32(mat), gr * p.cluster + rank) + static_cast<uint32_t>(r * ld + c) * 4u;
+#pragma unroll
+              for (int e = 0; e < kRows; ++e)
+                if (r + e < r1) v[e] += ld_cluster_f32(src + static_cast<uint32_t>(e * ld) * 4u);
+            }
+#pragma unroll
+            for (int e = 0; e < kRows; ++e) {
+              if (r + e < r1) {
+                sum += v[e];
+                mx = fmaxf(mx, v[e]);
+              }
+            }
           }
           parts[part * p.tk + c] = make_float2(sum, mx);
         }
       }
       pdl_wait();
       asm volatile("bar.sync 1, 256;" ::: "memory");
-      for (int c = threadIdx.x; c < p.tk; c += kExpThreads) {
+      for (int c = c_lo + threadIdx.x; c < c_hi; c += kExpThreads) {
         const int j = static_cast<int>(rank) * p.tk + c - p.vis_start;   // vision-relative index
         if (j < 0 || j >= p.M) continue;
         float sum = 0.0f, mx = -INFINITY;
@@ -1119,7 +1155,12 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           sum += v.x;
           mx = fmaxf(mx, v.y);
         }
-        if constexpr (PH) mx = ph_stage[c] * (1.0f / kPhScale);
+        if constexpr (PH) {
+          mx = p.groups == 1 ? ph_stage[c] : 0.0f;
+          for (int gr = 0; gr < p.groups && p.groups > 1; ++gr)
+            mx += ld_cluster_f32(map_to_cta(smem_u32(ph_stage + c), gr * p.cluster + rank));
+          mx *= 1.0f / kPhScale;
+        }
         const bool present = j < Mb;    // beyond the request's own tokens: zeros
         float gv = present ? sum * p.inv_heads : 0.0f, iv = present ? mx * p.inv_heads : 0.0f;
         if (p.combine) {                // the text rows before row0 were scored by the launch before this one
@@ -1140,7 +1181,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       common_exit(finish_scores);
       if (cluster_gave_up()) { leave_after_give_up(ft.sel.kept_cnt); return; }
       pdl_wait();   // the outputs written below may still be read by an earlier kernel in the stream
-      filter_select(ft.sel, sel_sh, b, threadIdx.x, rank == 0, kept_list, &kept_total_s);
+      filter_select(ft.sel, sel_sh, b, threadIdx.x, req_rank == 0, kept_list, &kept_total_s);
       if (threadIdx.x == 0) MD_TRACE(0, 12);   // selection done
       cta_sync();   // the list is complete: the copy thread may start
       return;
@@ -1170,7 +1211,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     const bool real_row = row < p.N;     // lanes beyond the text rows carry padding
 
     int h = 0;
-    for (; h < p.H; ++h) {
+    for (; h < n_heads; ++h) {
       const int buf = h % p.n_buf;
       const uint32_t bph = static_cast<uint32_t>(h / p.n_buf) & 1u;
       const int slot = h % p.n_slot;
@@ -1289,7 +1330,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
 
     // the head sums go to shared memory, where the exp warps reduce them over the text rows
     mbar_arrive(smem_u32(&bars.fin));
-    if (__all_sync(0xffffffffu, h == p.H && mbar_wait(smem_u32(&bars.fin), 0u, abort_flag, wait_limit))) {
+    if (__all_sync(0xffffffffu, h == n_heads && mbar_wait(smem_u32(&bars.fin), 0u, abort_flag, wait_limit))) {
       // all TMA copies have landed and all MMAs have read them: the staging area is free
       float* const mat = reinterpret_cast<float*>(stage_ptr);
       const int ld = p.tk | 1;
@@ -1316,8 +1357,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       pdl_wait();
       cta_sync();   // the exp warps have finished the selection
       if (warp == kExpWarps && lane == 0) {
-        filter_gather(ft, gm, bars.gfull, abort_flag, kept_list, kept_total_s, stage_base, static_cast<int>(rank), b, Mb,
-                      p.cluster, p.workspace);
+        filter_gather(ft, gm, bars.gfull, abort_flag, kept_list, kept_total_s, stage_base, static_cast<int>(req_rank), b, Mb,
+                      req_ctas, p.workspace);
         MD_TRACE(0, 13);   // gather done
       }
       return;
@@ -1409,9 +1450,22 @@ FusedKernel pick_kernel(int halves, int ach, bool filter = false, bool per_head 
 }
 
 // Clusters of `cluster` CTAs that can be resident at once (GPC boundaries make this less than
-// SMs / cluster); 0 when it cannot be asked (no device) or the shape cannot launch.
-int max_resident_clusters(int halves, int ach, int cluster, size_t smem_bytes, bool per_head) {
-  FusedKernel kernel = pick_kernel(halves, ach, false, per_head);
+// SMs / cluster); 0 when it cannot be asked (no device) or the shape cannot launch.  Every
+// instantiation runs one CTA per SM (each asks for more than half of the shared memory and most of
+// the registers), so the answer depends on the size alone: one instantiation is asked, once per
+// device and size.
+int max_resident_clusters(int cluster) {
+  static std::mutex mu;
+  static std::map<std::pair<int, int>, int> known;   // (device, cluster size)
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
+  }
+  std::lock_guard<std::mutex> lock(mu);
+  const auto it = known.find({dev, cluster});
+  if (it != known.end()) return it->second;
+  FusedKernel kernel = pick_kernel(2, 10);
   if (ensure_kernel_attributes(reinterpret_cast<const void*>(kernel), true) != cudaSuccess) {
     (void)cudaGetLastError();
     return 0;
@@ -1419,7 +1473,7 @@ int max_resident_clusters(int halves, int ach, int cluster, size_t smem_bytes, b
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(cluster));
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem_bytes;
+  cfg.dynamicSmemBytes = kMinSmem;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = static_cast<unsigned>(cluster);
@@ -1432,16 +1486,15 @@ int max_resident_clusters(int halves, int ach, int cluster, size_t smem_bytes, b
     (void)cudaGetLastError();
     return 0;
   }
+  known[{dev, cluster}] = n;
   return n;
 }
 
 }  // namespace
 
 // Geometry of the fused kernel for a problem; false when the shape is outside what it covers.
-// row0 / n_rows: the text rows the launch covers (n_rows = 0: all of them); max_cluster: an upper
-// limit on the cluster size (0: none).
-bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, FusedGeometry* out, int row0, int n_rows,
-                      int max_cluster) {
+// row0 / n_rows: the text rows the launch covers (n_rows = 0: all of them).
+bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, FusedGeometry* out, int row0, int n_rows) {
   if (n_rows <= 0) { row0 = 0; n_rows = r.N; }
   const int halves = n_rows <= 64 ? 2 : 1;
   const int nrows = 128 / halves;
@@ -1453,7 +1506,6 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
   FusedGeometry g{};
   for (int c = 1; c <= kMaxCluster; ++c) {
     if (forced_cluster > 0 && c != forced_cluster) continue;
-    if (max_cluster > 0 && c > max_cluster) continue;
     const int per_cta = (r.L + c - 1) / c;
     int cpl = (per_cta + halves - 1) / halves;
     cpl = (cpl + kChunk - 1) / kChunk * kChunk;
@@ -1517,37 +1569,53 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
       if (best_d == 0) continue;
     }
     if (n_q > 4) n_q = 4;
-    // Cost model (microseconds per head and CTA): streaming the stage at ~45 GB/s per SM, or the
-    // MMA -> exp -> exchange -> add chain (~4.5 us) spread over the buffers, whichever is longer;
-    // times the number of waves of CTAs.
     size_t smem_bytes = (split ? n_q * q_tile + n_k * k_half : n_q * stage) + 1024 + extra + ph_bytes;
-    // at least 116 KB, so that two CTAs (each wanting all of tensor memory) never share an SM
-    if (smem_bytes < 116 * 1024) smem_bytes = 116 * 1024;
-    int resident = max_resident_clusters(halves, ach, c, smem_bytes, r.per_head_max != 0);
-    if (resident <= 0 && c <= 8) resident = sm_count / c;    // no device to ask: ignore GPC boundaries
-    // (a cluster of more than 8 CTAs is used only where the device says it can hold one)
-    if (resident <= 0) continue;
-    const long waves = (r.B + resident - 1) / resident;
-    const double t_stream = static_cast<double>(stage) / 45.0e3;
-    double t_chain = 4.5 / n_buf + 0.02 * c;   // the statistics exchange grows with the cluster
-    if (n_slot < 2 * n_buf) {
-      // Tight slots: the exchange over the cluster is on the critical path of every head (d = 2)
-      // or of every head twice (d = 1).  Measured per head: 2.6 .. 3.3 us at 11 .. 16 CTAs with
-      // d = 2, 4.3 us at 10 CTAs with d = 1; a third more with 128 text rows on the lanes.
-      t_chain = (n_slot == 4 ? 1.8 + 0.09 * c : 3.0 + 0.13 * c) * (halves == 1 ? 1.3 : 1.0);
-    }
-    double t_head = t_stream > t_chain ? t_stream : t_chain;
-    if (t_head < 1.4) t_head = 1.4;   // the exp stage and its hand-overs take that long per head however narrow the tile
-    // among equals: larger clusters while all of them are resident at once (a call by itself gains
-    // from spreading its keys over more SMs: measured 62 against 66 us at 16 requests), else smaller ones
-    const double tie = (waves == 1) ? 1e-4 * c : -1e-4 * c;
-    const double score = 1.0 / (static_cast<double>(waves) * t_head) + tie;
-    if (score > best) {
-      best = score;
-      g.halves = halves; g.cluster = c; g.tk = tk; g.cpl = cpl; g.n_q = n_q; g.n_k = n_k; g.split = split; g.n_buf = n_buf; g.ach = ach;
-      g.n_slot = n_slot; g.resident = resident; g.row0 = row0; g.n_rows = n_rows;
-      g.est_us = static_cast<float>(waves * r.H * t_head);
-      g.smem_bytes = smem_bytes;
+    if (smem_bytes < kMinSmem) smem_bytes = kMinSmem;
+    const bool is_tight = n_slot < 2 * n_buf;
+    // Head groups: the request's heads are dealt out over `grp` groups of c CTAs (one cluster of grp x c).
+    // A group loops over fewer heads, which costs one reduction of the groups' head sums through
+    // distributed shared memory at the end; spending the CTAs on more key ranges per head instead (a
+    // larger c) makes every head narrower, but a head costs ~1.2 us however narrow it is.  One
+    // request of 608 keys: 47.6 us as 16 key ranges, 25.2 as 4 x 4; 16 requests, budget 192: 76.1 us
+    // as 6, 64.3 as 2 groups x 3.  (Not with a forced cluster size or a tight window.)
+    const int max_s = forced_cluster > 0 || is_tight ? 1 : kMaxCluster / c;
+    for (int grp = 1; grp <= max_s && grp <= r.H; ++grp) {
+      const int size = c * grp;
+      int resident = max_resident_clusters(size);
+      if (resident <= 0 && size <= 8) resident = sm_count / size;    // no device to ask: ignore GPC boundaries
+      // (a cluster of more than 8 CTAs is used only where the device says it can hold one)
+      if (resident <= 0) continue;
+      const long waves = (r.B + resident - 1) / resident;
+      const int heads = (r.H + grp - 1) / grp;
+      const double active = static_cast<double>(size) * (r.B < resident ? r.B : resident);
+      // Cost of a head in a CTA (microseconds): streaming its stage (an SM alone draws up to 150 GB/s, all
+      // of them together ~7 TB/s), the exp stage (two heads at a time), the MMA -> exp -> exchange ->
+      // add chain spread over the buffers, the add stage.
+      const double rate = 7.0e6 / active < 150.0e3 ? 7.0e6 / active : 150.0e3;   // bytes per microsecond
+      const double t_stream = static_cast<double>(stage) / rate;
+      const double t_exp = 0.45 + 0.2 * (cpl / kChunk);
+      const double t_chain = t_exp + 1.3 + (c > 1 ? 0.4 + 0.08 * c : 0.2);
+      double t_head = t_chain / n_buf;
+      if (is_tight) {
+        // Tight slots: the exchange over the cluster is on the critical path of every head (d = 2)
+        // or of every head twice (d = 1).  Measured per head: 2.6 .. 3.3 us at 11 .. 16 CTAs with
+        // d = 2, 4.3 us at 10 CTAs with d = 1; a third more with 128 text rows on the lanes.
+        t_head = (n_slot == 4 ? 1.8 + 0.09 * c : 3.0 + 0.13 * c) * (halves == 1 ? 1.3 : 1.0);
+      }
+      if (t_head < t_exp / 2) t_head = t_exp / 2;
+      if (t_head < t_stream) t_head = t_stream;
+      if (t_head < 1.15) t_head = 1.15;
+      // ... and of a request: start, fill and exit (more where CTAs of a next wave have to wait for
+      // it), and the reduction over the head groups.
+      const double t_req = 3.0 + heads * t_head + t_chain + (grp > 1 ? 1.0 + 0.5 * grp : 0.0);
+      const double est = waves * t_req + (waves - 1) * 15.0;
+      if (best < 0.0 || est < best - 1e-9) {
+        best = est;
+        g.halves = halves; g.cluster = c; g.groups = grp; g.tk = tk; g.cpl = cpl; g.n_q = n_q; g.n_k = n_k; g.split = split;
+        g.n_buf = n_buf; g.ach = ach; g.n_slot = n_slot; g.resident = resident; g.row0 = row0; g.n_rows = n_rows;
+        g.est_us = static_cast<float>(est);
+        g.smem_bytes = smem_bytes;
+      }
     }
   }
   if (best < 0.0) return false;
@@ -1594,7 +1662,7 @@ bool plan_score_grid(const Resolved& r, int sm_count, int forced_ctas, FusedGeom
     if (n_slot > 6) n_slot = 6;
     if (n_slot > n_buf) n_slot = n_buf;
     size_t smem_bytes = n_q * stage + n_slot * slot + own + 1024 + ph_bytes;
-    if (smem_bytes < 116 * 1024) smem_bytes = 116 * 1024;
+    if (smem_bytes < kMinSmem) smem_bytes = kMinSmem;
     // Cost per head and CTA (microseconds): streaming the stage at ~45 GB/s per SM; the exp stage
     // (measured: ~0.011 us per column of a lane, two heads at a time on narrow tiles); the
     // MMA -> exp -> exchange through L2 -> add chain (~6 us) spread over the buffers.
@@ -1608,7 +1676,7 @@ bool plan_score_grid(const Resolved& r, int sm_count, int forced_ctas, FusedGeom
     if (score > best) {
       best = score;
       g.halves = halves; g.cluster = c; g.tk = tk; g.cpl = cpl; g.n_q = n_q; g.n_k = 0; g.split = 0; g.n_buf = n_buf;
-      g.ach = ach; g.n_slot = n_slot; g.gx = 1; g.resident = sm_count; g.row0 = 0; g.n_rows = r.N;
+      g.ach = ach; g.groups = 1; g.n_slot = n_slot; g.gx = 1; g.resident = sm_count; g.row0 = 0; g.n_rows = r.N;
       g.est_us = static_cast<float>(r.H * t_head + 12.0);    // (+ filling and draining the longer chain)
       g.smem_bytes = smem_bytes;
     }
@@ -1666,7 +1734,7 @@ cudaError_t launch_fused_common(const mustdrop_plan& plan, const FusedGeometry& 
   p.H = r.H; p.N = geo.n_rows; p.L = r.L; p.M = r.M; p.vis_start = r.vis_start; p.txt_start = r.txt_start;
   p.causal = r.causal;
   p.n_txt = r.N; p.row0 = geo.row0; p.combine = combine ? 1 : 0;
-  p.cluster = geo.cluster; p.tk = geo.tk; p.cpl = geo.cpl; p.n_q = geo.n_q; p.n_k = geo.n_k; p.split = geo.split;
+  p.cluster = geo.cluster; p.groups = geo.groups; p.tk = geo.tk; p.cpl = geo.cpl; p.n_q = geo.n_q; p.n_k = geo.n_k; p.split = geo.split;
   p.n_buf = geo.n_buf; p.n_slot = geo.n_slot; p.tight = (!geo.gx && geo.n_slot < 2 * geo.n_buf) ? geo.n_slot / 2 : 0;
   p.gx = geo.gx;
   p.gx_cnt = reinterpret_cast<uint32_t*>(static_cast<unsigned char*>(workspace) + plan.ws_gx_cnt_off);
@@ -1681,13 +1749,13 @@ cudaError_t launch_fused_common(const mustdrop_plan& plan, const FusedGeometry& 
   cudaError_t e = ensure_kernel_attributes(reinterpret_cast<const void*>(kernel), true);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(r.B * geo.cluster));
+  cfg.gridDim = dim3(static_cast<unsigned>(r.B * geo.cluster * geo.groups));
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = geo.gx ? 1u : static_cast<unsigned>(geo.cluster);   // grid plans: no cluster
+  attr[0].val.clusterDim.x = geo.gx ? 1u : static_cast<unsigned>(geo.cluster * geo.groups);   // grid plans: no cluster
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
