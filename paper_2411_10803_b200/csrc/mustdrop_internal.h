@@ -47,6 +47,7 @@ struct FilterGeometry {
   size_t smem_bytes;   // dynamic shared memory of the launch (>= the score geometry's)
   int32_t slot_bytes;  // one kept row: hidden row + K pieces + V pieces of all heads
   int32_t n_slot;      // rows in flight per CTA
+  int32_t val_off;     // where the selection's scores lie (bytes behind the aligned start of dynamic shared memory)
 };
 
 struct Resolved {
@@ -90,7 +91,8 @@ struct mustdrop_plan {
   int32_t score_variant;
   size_t ws_bytes;
   size_t ws_rowstats_off;   // float2 [B,H,N]: (row max in log2 units, 1 / row sum)
-  size_t ws_gx_cnt_off;     // grid plans: uint32 [4 B]: calls completed, and three counters that are zero between calls
+  size_t ws_gx_cnt_off;     // grid plans: uint32 [2 B]: calls completed, CTAs that have left the call (zero between calls)
+  size_t ws_gx_scores_off;  // grid plans: 8-byte words [B,M]
   size_t ws_gx_stats_off;   // grid plans: 8-byte words [B,H,CTAs per request,rows]
   mustdrop::FusedGeometry fused;
   int32_t row_split;        // 1: the text rows are scored by two launches (fused: rows 0..63, fused_b: the rest)

@@ -80,7 +80,8 @@ struct FusedParams {
   // the CTAs of a request are ordinary CTAs of the grid, any number of them, all resident at once).
   int32_t gx;                         // 1: grid plan (cluster = CTAs per request, launched without a cluster)
   float2* gx_stats;                   // [B][H][CTAs per request][rows] (stabiliser, sum with the call's parity as its sign)
-  uint32_t* gx_cnt;                   // [B] calls completed, then three counters per request that are zero between calls: [B] CTAs that left, [B] scores stored, [B] barrier passed
+  float2* gx_scores;                  // [B][M] (G, I with the call's parity as its sign)
+  uint32_t* gx_cnt;                   // [B] calls completed, [B] CTAs of the request that have left the call (zero between calls)
   int32_t per_head;                   // 1: i_out = head mean of the per-head maxima over the text rows (PH instantiations)
   int32_t early_inputs;               // 1: q_text / k may be read before the stream's earlier work has completed (caller's promise)
   long long wait_cycles;              // clock cycles after which a wait between the warp roles gives up
@@ -99,6 +100,8 @@ struct FilterTail {
   int32_t kv_bytes;              // bytes of a K (or V) row over all heads = H * 256
   int32_t has_k, has_v;
   int32_t slot_bytes, n_slot;    // gather ring in dynamic shared memory
+  int32_t val_off;               // where the request's scores meet, in dynamic shared memory: behind everything that is
+                                 // still in use when the first CTA of the request has its own
   int32_t vis_start;
   int32_t rebuild, N, out_rows;  // rebuild: outputs are [prefix ; kept vision ; text] (out_rows rows per request)
 };
@@ -146,18 +149,6 @@ __device__ __forceinline__ float2 ld_word(const float2* src) {
   return make_float2(__uint_as_float(static_cast<uint32_t>(v)), __uint_as_float(static_cast<uint32_t>(v >> 32)));
 }
 __device__ __forceinline__ bool has_parity(const float2& word, uint32_t parity) { return __float_as_uint(word.y) >> 31 == parity; }
-// Bounded wait until a counter has reached its target (same give-up rules as mbar_wait).
-__device__ __forceinline__ bool count_wait(const uint32_t* p, uint32_t target, volatile int* abort_flag, long long limit) {
-  if (ld_acquire_gpu(p) >= target) return true;
-  const long long t0 = clock64();
-  while (ld_acquire_gpu(p) < target) {
-    if (*abort_flag != 0 || clock64() - t0 > limit) {
-      *abort_flag = 1;
-      return false;
-    }
-  }
-  return true;
-}
 // Bounded wait.  Returns false (and raises the CTA's abort flag) when the wait ran out or the
 // CTA has already given up.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long limit) {
@@ -425,19 +416,6 @@ struct GatherMaps {
 // Both parts run once per CTA after the score part.  Functions of their own for reading only: they
 // are inlined (as real calls - like any call in this kernel - they slowed the gather by a third).
 
-// Selection of request b by the 256 threads of the exp warps (tid = 0..255); rank 0 of the
-// request's CTAs stores the list, every CTA keeps it in its shared memory.
-__device__ __forceinline__ void filter_select(const SelectParams& sel, SelectShared& sel_sh, int b, int tid, bool writer,
-                                           int32_t* kept_list, int32_t* kept_total) {
-  select_clear(sel_sh, tid);
-  const int own = (sel.M + kSelThreads - 1) / kSelThreads;
-  if (own <= 1) select_request<1, SelectSyncGroup>(sel, sel_sh, b, tid, writer, kept_list, kept_total);
-  else if (own <= 2) select_request<2, SelectSyncGroup>(sel, sel_sh, b, tid, writer, kept_list, kept_total);
-  else if (own <= 4) select_request<4, SelectSyncGroup>(sel, sel_sh, b, tid, writer, kept_list, kept_total);
-  else if (own <= 8) select_request<8, SelectSyncGroup>(sel, sel_sh, b, tid, writer, kept_list, kept_total);
-  else select_request<16, SelectSyncGroup>(sel, sel_sh, b, tid, writer, kept_list, kept_total);
-}
-
 // Gather of the request's kept rows, driven by ONE thread of the CTA: row r of the compacted
 // outputs is copied by CTA r mod cluster.
 __device__ __forceinline__ void filter_gather(const FilterTail& ft, const GatherMaps& gm, uint64_t* gfull, volatile int* abort_flag,
@@ -574,6 +552,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
   // PH only: [2][4 add warps][tk] per-head column maxima of each warp's text rows, double-buffered over heads
   float* const ph_stage = reinterpret_cast<float*>(stats + static_cast<size_t>(p.n_slot) * slot_pairs);
 
+  __shared__ SelectShared sel_sh;       // (FILTER: cleared and the key set marked long before the scores are complete)
+  if constexpr (FILTER) select_clear(sel_sh, threadIdx.x, kThreads);
   if (threadIdx.x == 0) {
     abort_flag_s = 0;
     cluster_abort_s = 0;
@@ -629,35 +609,20 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     cta_sync();
     if (p.groups > 1) cluster_sync_all();   // the head sums of every group are staged
     finish();       // (exp warps: the scores from the staged head sums)
-    if (p.gx) cta_sync();   // every score of this CTA is stored before the request's CTAs meet below
     if (p.gx) {
-      // grid plan: the request's CTAs are no cluster.  In the filter kernel they meet through a
-      // counter in global memory: every CTA's scores are stored before any CTA selects.  (A CTA
-      // that gives up tells nobody: its peers run into their own limits.)
-      if (threadIdx.x == 0) {
-        const size_t n_req = gridDim.x / p.cluster;
-        if (*abort_flag == 0) {
-          // every CTA of the request has read its parity when it gets here: the last one counts the call
-          uint32_t* const left = p.gx_cnt + n_req + b;
-          if (atomicAdd(left, 1u) == static_cast<uint32_t>(p.cluster) - 1u) {
-            p.gx_cnt[b] += 1u;
-            *left = 0u;
-          }
-        }
-        if (FILTER && *abort_flag == 0) {
-          uint32_t* const stored = p.gx_cnt + 2 * n_req + b;
-          uint32_t* const passed = stored + n_req;
-          __threadfence();
-          atomicAdd(stored, 1u);
-          if (count_wait(stored, static_cast<uint32_t>(p.cluster), abort_flag, wait_limit) &&
-              atomicAdd(passed, 1u) == static_cast<uint32_t>(p.cluster) - 1u) {
-            *stored = 0u;   // the last one through leaves the counters as the next call expects them
-            *passed = 0u;
-          }
-        }
-        if (*abort_flag != 0) {
-          record_status(p.workspace, MUSTDROP_ERR_TIMEOUT, blockIdx.x);
-          cluster_abort_s = 1;
+      // grid plan: the request's CTAs are no cluster and do not meet here: the filter's selection
+      // recognises every score by its parity.  (A CTA that gives up tells nobody: its peers run into
+      // their own limits.)
+      if (threadIdx.x == 0 && *abort_flag != 0) {
+        record_status(p.workspace, MUSTDROP_ERR_TIMEOUT, blockIdx.x);
+        cluster_abort_s = 1;
+      }
+      // every warp of this CTA has read its parity: the last CTA of the request counts the call
+      if (threadIdx.x == kThreads - 1 && *abort_flag == 0) {
+        uint32_t* const left = p.gx_cnt + gridDim.x / p.cluster + b;
+        if (atomicAdd(left, 1u) == static_cast<uint32_t>(p.cluster) - 1u) {
+          *left = 0u;
+          p.gx_cnt[b] += 1u;
         }
       }
       cta_sync();
@@ -856,6 +821,12 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         const uint32_t ph = static_cast<uint32_t>(committed / p.n_buf) & 1u;
         const long long t0 = clock64();
         while (!mbar_try_wait(bar, ph) && clock64() - t0 < kWaitCycles) {}
+      }
+    }
+    if constexpr (FILTER) {
+      if (warp == kMmaWarp + 2) {
+        pdl_wait();   // the key set may come from the kernel just before this one
+        select_mark_keys(ft.sel, sel_sh, b, lane, 32, req_rank == 0);
       }
     }
     if (warp > kMmaWarp && p.gx) {
@@ -1088,6 +1059,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     // warps once the add warps have staged the head sums: a warp takes 32 keys and an eighth of the
     // rows at a time, and the eighths of a key meet in shared memory.  (By the four add warps alone,
     // a key per thread and all rows one after the other, it took 3.8 us at 320 keys per CTA.)
+    uint32_t* const val_g = reinterpret_cast<uint32_t*>(stage_ptr + ft.val_off);
     auto finish_scores = [&]() {
       if (*abort_flag != 0) return;   // (the same answer in every thread: nothing raises it any more)
       constexpr int kParts = 8, kRows = 8;
@@ -1157,19 +1129,70 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         }
         p.g_out[static_cast<size_t>(b) * p.M + j] = gv;
         p.i_out[static_cast<size_t>(b) * p.M + j] = iv;
+        if constexpr (FILTER) {   // ... and to the selection, in every CTA of the request
+          if (p.gx) {
+            st_parity(p.gx_scores + static_cast<size_t>(b) * p.M + j, gv, iv, parity);
+          } else {
+            const uint32_t at = smem_u32(val_g + j);
+            for (int cta = 0; cta < req_ctas; ++cta) {
+              const uint32_t to = map_to_cta(at, cta);
+              st_remote_u32(to, __float_as_uint(gv));
+              st_remote_u32(to + 4u * static_cast<uint32_t>(select_pad(p.M)), __float_as_uint(iv));
+            }
+          }
+        }
       }
       if (threadIdx.x == 0) MD_TRACE(0, 10);   // scores stored
     };
     if constexpr (FILTER) {
-      // filter tail, exp warps: selection of this request.  Dynamic shared memory is free by now:
-      // all copies have landed, all MMAs have read them and every statistics pair sent to this CTA
-      // has been consumed.  Each CTA of the cluster runs the same selection on its own (identical
-      // inputs, fixed order: identical lists); rank 0 stores the list.
-      __shared__ SelectShared sel_sh;
+      // filter tail, exp warps: selection of this request.  Dynamic shared memory is free by now, but
+      // for the scores: all copies have landed, all MMAs have read them and every statistics pair
+      // sent to this CTA has been consumed.  Each CTA of the request runs the same selection on its
+      // own (identical inputs, fixed order: identical lists); rank 0 stores the list.
       common_exit(finish_scores);
       if (cluster_gave_up()) { leave_after_give_up(ft.sel.kept_cnt); return; }
       pdl_wait();   // the outputs written below may still be read by an earlier kernel in the stream
-      filter_select(ft.sel, sel_sh, b, threadIdx.x, req_rank == 0, kept_list, &kept_total_s);
+      uint32_t* const val_i = val_g + select_pad(p.M);
+      if (p.gx) {
+        // grid plan: the scores as the request's CTAs have stored them (a score that is not there
+        // yet is looked at again)
+        const float2* const words = p.gx_scores + static_cast<size_t>(b) * p.M;
+        const long long t0 = clock64();
+#pragma unroll 1
+        for (int j0 = threadIdx.x; j0 < Mb; j0 += 8 * kExpThreads) {
+          float2 w[8];
+          bool there = false;
+          while (!there) {
+            there = true;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) w[e] = ld_word(words + min(j0 + e * kExpThreads, Mb - 1));
+#pragma unroll
+            for (int e = 0; e < 8; ++e) there = there && has_parity(w[e], parity);
+            if (!there && (*abort_flag != 0 || clock64() - t0 > wait_limit)) {
+              *abort_flag = 1;
+              break;
+            }
+          }
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            const int j = j0 + e * kExpThreads;
+            if (j < Mb) {
+              val_g[j] = __float_as_uint(w[e].x);
+              val_i[j] = __float_as_uint(fabsf(w[e].y));
+            }
+          }
+        }
+      }
+      SelectScratch& scratch = *reinterpret_cast<SelectScratch*>(stage_ptr + kKeptListBytes);
+      if (p.M <= kFewTokens)
+        select_request<1, SelectSyncGroup>(ft.sel, sel_sh, scratch, val_g, val_i, b, threadIdx.x, req_rank == 0, kept_list, &kept_total_s);
+      else
+        select_request<4, SelectSyncGroup>(ft.sel, sel_sh, scratch, val_g, val_i, b, threadIdx.x, req_rank == 0, kept_list, &kept_total_s);
+      if (p.gx && *abort_flag != 0 && threadIdx.x == 0) {   // some scores never came
+        record_status(p.workspace, MUSTDROP_ERR_TIMEOUT, blockIdx.x);
+        ft.sel.kept_cnt[b] = -1;
+        kept_total_s = 0;
+      }
       if (threadIdx.x == 0) MD_TRACE(0, 12);   // selection done
       cta_sync();   // the list is complete: the copy thread may start
       return;
@@ -1752,6 +1775,7 @@ cudaError_t launch_fused_common(const mustdrop_plan& plan, const FusedGeometry& 
   p.gx = geo.gx;
   p.gx_cnt = reinterpret_cast<uint32_t*>(static_cast<unsigned char*>(workspace) + plan.ws_gx_cnt_off);
   p.gx_stats = reinterpret_cast<float2*>(static_cast<unsigned char*>(workspace) + plan.ws_gx_stats_off);
+  p.gx_scores = reinterpret_cast<float2*>(static_cast<unsigned char*>(workspace) + plan.ws_gx_scores_off);
   p.per_head = r.per_head_max;
   p.early_inputs = (r.inputs_ready && vis_cnt == nullptr) ? 1 : 0;
   p.wait_cycles = r.wait_cycles > 0 ? r.wait_cycles : kWaitCycles;
@@ -1799,10 +1823,25 @@ bool plan_filter_single(const Resolved& r, const FusedGeometry& geo, FilterGeome
   const size_t slot = hidden_pad + 2 * static_cast<size_t>(r.H) * 256;
   const size_t limit = 227 * 1024 - 4096;                          // dynamic shared memory a CTA may ask for
   const size_t fixed = 1024 + kKeptListBytes;
+  // The scores meet in every CTA while peers may still be adding their last head or reading this
+  // CTA's staged head sums: behind those sums inside the staging area, which is idle by then, or
+  // behind everything.
+  const size_t nrows = 128 / geo.halves, val = 8 * static_cast<size_t>(select_pad(r.M));
+  const size_t stage = (nrows + geo.tk) * 256;
+  const size_t staging = geo.split ? geo.n_q * nrows * 256 + static_cast<size_t>(geo.n_k) * geo.cpl * 256 : geo.n_q * stage;
+  const size_t sums = ((nrows * (geo.tk | 1) * 4 + 15) & ~static_cast<size_t>(15)) + 8 * static_cast<size_t>(geo.tk) * 8;
+  size_t val_off = (sums + 15) & ~static_cast<size_t>(15), least = geo.smem_bytes;
+  // (the selection's own scratch lies at the start of the staging area, behind the kept list)
+  if (val_off < kKeptListBytes + sizeof(SelectScratch)) val_off = kKeptListBytes + sizeof(SelectScratch);
+  if (val_off + val > staging) {
+    val_off = geo.smem_bytes - 1024 > val_off ? geo.smem_bytes - 1024 : val_off;
+    least = 1024 + val_off + val;
+  }
   size_t want = fixed + kMaxGatherSlots * slot;
-  if (want < geo.smem_bytes) want = geo.smem_bytes;
+  if (want < least) want = least;
   if (want > limit) want = limit;
-  if (want < geo.smem_bytes) return false;
+  if (want < least) return false;
+  out->val_off = static_cast<int32_t>(val_off);
   int n_slot = static_cast<int>((want - fixed) / slot);
   if (n_slot > kMaxGatherSlots) n_slot = kMaxGatherSlots;
   if (n_slot < 3) return false;
@@ -1869,6 +1908,7 @@ cudaError_t launch_filter_fused(const mustdrop_plan& plan, const void* q_text, c
   t.kv_bytes = r.H * 256;
   t.has_k = k_out != nullptr; t.has_v = v_out != nullptr;
   t.slot_bytes = plan.filter.slot_bytes; t.n_slot = plan.filter.n_slot;
+  t.val_off = plan.filter.val_off;
   t.vis_start = r.vis_start;
   if (plan.row_split) {   // first the score of text rows 0..63 alone, then the rest with the tail
     cudaError_t e = launch_fused_common(plan, plan.fused, false, q_text, k, g_out, i_out, workspace, nullptr, nullptr,

@@ -12,17 +12,47 @@
 namespace mustdrop {
 namespace {
 
-template <int OWN>
 __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectParams p) {
   __shared__ SelectShared s;
-  const int tid = threadIdx.x;
+  __shared__ SelectScratch x;
+  extern __shared__ uint32_t val[];   // G and I of the request, M rounded up to 256 words each
+  const int tid = threadIdx.x, b = blockIdx.x;
   // Work that touches no global data, then let the next kernel start its prologue and wait for
   // the kernel that produced g / i.
   MD_PIPE(p.workspace, 1, false, false);
-  select_clear(s, tid);
+  select_clear(s, tid, kSelThreads);
+  __syncthreads();
   pdl_launch_dependents();
   pdl_wait();
-  select_request<OWN, SelectSyncCta>(p, s, blockIdx.x, tid, true, nullptr, nullptr);
+  const int M = p.vis_cnt ? clamp_vis_cnt(p.vis_cnt[b], p.M) : p.M;
+  uint32_t* const val_i = val + select_pad(p.M);
+  const float* const g = p.g + static_cast<size_t>(b) * p.M;
+  const float* const i = p.i + static_cast<size_t>(b) * p.M;
+  // the key set's loads and the first strips' are under way together
+  float gv[4], iv[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int j = tid + e * kSelThreads;
+    gv[e] = j < M ? g[j] : 0.0f;
+    iv[e] = j < M ? i[j] : 0.0f;
+  }
+  select_mark_keys(p, s, b, tid, kSelThreads, true);
+#pragma unroll 1
+  for (int j0 = tid; j0 < M; j0 += 4 * kSelThreads) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int j = j0 + e * kSelThreads, next = j + 4 * kSelThreads;
+      if (j < M) {
+        val[j] = __float_as_uint(gv[e]);
+        val_i[j] = __float_as_uint(iv[e]);
+      }
+      gv[e] = next < M ? g[next] : 0.0f;
+      iv[e] = next < M ? i[next] : 0.0f;
+    }
+  }
+  __syncthreads();
+  if (p.M <= kFewTokens) select_request<1, SelectSyncCta>(p, s, x, val, val_i, b, tid, true, nullptr, nullptr);
+  else select_request<4, SelectSyncCta>(p, s, x, val, val_i, b, tid, true, nullptr, nullptr);
   MD_PIPE(p.workspace, 1, true, false);
 }
 
@@ -40,13 +70,8 @@ cudaError_t launch_select(const mustdrop_plan& plan, const float* g, const float
   p.vis_cnt = la.vis_cnt; p.orig_in = la.orig_in; p.orig_out = la.orig_out;
   p.key_idx_out = la.key_idx_out; p.key_cnt_out = la.key_cnt_out;
   p.vis_start = r.vis_start; p.N = r.N; p.gamma_default = r.gamma_default; p.alpha_default = r.alpha_default;
-  const int own = (r.M + kSelThreads - 1) / kSelThreads;
-  static_assert(kMaxOwn == 16, "dispatch below covers up to 16 tokens per thread");
-  if (own <= 1) return launch_pdl(select_kernel<1>, dim3(r.B), dim3(kSelThreads), 0, stream, p);
-  if (own <= 2) return launch_pdl(select_kernel<2>, dim3(r.B), dim3(kSelThreads), 0, stream, p);
-  if (own <= 4) return launch_pdl(select_kernel<4>, dim3(r.B), dim3(kSelThreads), 0, stream, p);
-  if (own <= 8) return launch_pdl(select_kernel<8>, dim3(r.B), dim3(kSelThreads), 0, stream, p);
-  return launch_pdl(select_kernel<16>, dim3(r.B), dim3(kSelThreads), 0, stream, p);
+  static_assert(sizeof(SelectShared) + sizeof(SelectScratch) + 8 * select_pad(kMaxVis) <= 48 * 1024, "no opt-in needed");
+  return launch_pdl(select_kernel, dim3(r.B), dim3(kSelThreads), static_cast<size_t>(8) * select_pad(r.M), stream, p);
 }
 
 }  // namespace mustdrop

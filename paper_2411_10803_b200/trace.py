@@ -101,26 +101,30 @@ def main(argv) -> int:
     rel = np.array([[(t[c, 0, 8 + e] - entry0) / 1e3 for e in range(len(names))] for c in used])
     first_tma = np.array([(t[c, 0, 0] - entry0) / 1e3 for c in used])
     first_full = np.array([(t[c, 0, 1] - entry0) / 1e3 for c in used])
-    last_add = np.array([(t[c, (w.n_heads - 1) // 2 * 2, 7] - entry0) / 1e3 for c in used])
+    last_add = np.array([(t[c, :, 7].max() - entry0) / 1e3 for c in used])
     print("phases (us after the first CTA's entry; min / median / max over CTAs):")
     for n, col in [(names[0], rel[:, 0]), (names[1], rel[:, 1]), ("first_tma_issue", first_tma), ("first_stage_full", first_full),
-                   ("last_even_head_added", last_add)] + [(names[e], rel[:, e]) for e in range(2, len(names))]:
+                   ("last_head_added", last_add)] + [(names[e], rel[:, e]) for e in range(2, len(names))]:
         col = col[col > -1e6]
         print("  %-22s %8.2f %8.2f %8.2f" % (n, col.min(), np.median(col), col.max()))
     for c in used[:2] + used[-1:]:
         t0 = t[c, 0, 0]
-        print("CTA", c)
-        for h in sorted({0, 2, 4, w.n_heads // 2 // 2 * 2, (w.n_heads - 1) // 2 * 2}):
+        heads = int((t[c, :, 7] > 0).sum())   # (a head group loops over its share of the heads)
+        print("CTA", c, "heads", heads)
+        for h in sorted({0, 2, 4, heads // 2 // 2 * 2, (heads - 1) // 2 * 2} & set(range(heads))):
             print("  head %02d " % h + " ".join("%s=%.2f" % (n, (t[c, h, e] - t0) / 1e3) for e, n in enumerate(EVENTS))
                   + (" landed=%.2f" % ((t[c, h, 14] - t0) / 1e3) if t[c, h, 14] > 0 else ""))
-        done = t[c, :, 7]
-        print("  add_done per head: mean %.2f us" % (np.diff(done)[4:].mean() / 1e3))
-        if t[c, 4, 14] > 0:   # whole-stage plans: an onlooker stamps the landing of every stage
-            hs = t[c, 4:]
+        done = t[c, :heads, 7]
+        first = min(4, heads // 2)            # (the pipeline is filling before)
+        if heads < 4:
+            continue
+        print("  add_done per head: mean %.2f us" % (np.diff(done)[first:].mean() / 1e3))
+        if t[c, first, 14] > 0:   # whole-stage plans: an onlooker stamps the landing of every stage
+            hs = t[c, first:heads]
             print("  stage: copies issued -> landed %.2f us, landed -> MMA thread takes it %.2f us, issue -> next issue "
                   "into the same stage %.2f us" % ((hs[:, 14] - hs[:, 0]).mean() / 1e3, (hs[:, 2] - hs[:, 14]).mean() / 1e3,
-                                                  np.diff(t[c, 4:, 0]).mean() / 1e3))
-        ev = t[c, 4::2]
+                                                  np.diff(hs[:, 0]).mean() / 1e3))
+        ev = t[c, first // 2 * 2:heads:2]
         print("  exp stage %.2f us, exp_done -> statistics complete %.2f us, add stage %.2f us" % (
             (ev[:, 4] - ev[:, 3]).mean() / 1e3, (ev[:, 5] - ev[:, 4]).mean() / 1e3, (ev[:, 7] - ev[:, 6]).mean() / 1e3))
     return 0
