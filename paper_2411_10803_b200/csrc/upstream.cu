@@ -6,9 +6,10 @@
 //     above an adaptive threshold form the key set O.  The paper names no threshold rule; here it
 //     is Tukey's upper fence Q3 + 1.5 (Q3 - Q1) with linearly interpolated quartiles.
 // A thread-block cluster of up to eight CTAs of 256 threads works on one image (windows, rows and
-// heads are dealt out over the cluster's CTAs; flags and partial attention sums cross through
-// distributed shared memory, in a fixed order); both kernels are bound by reading their input
-// once (1.2 MB per image at 576 tokens x 1024 channels).
+// tokens are dealt out over the cluster's CTAs; flags, softmax statistics and attention cross through
+// distributed shared memory, in a fixed order).  Bound: reading the input once (1.2 MB per image at
+// 576 tokens x 1024 channels, the merge also writes ~0.9 MB), and the serial steps between the
+// cluster's barriers, which all images of a batch reach at about the same time.
 #include <cuda_bf16.h>
 
 #include "mustdrop_internal.h"
@@ -19,7 +20,7 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxSlots = 4096;            // tokens per image
-constexpr int kOwn = kMaxSlots / kThreads; // consecutive slots per thread in the scans
+constexpr int kWords = kMaxSlots / 32;     // words of a token bitmap
 
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
@@ -61,27 +62,37 @@ __device__ __forceinline__ uint32_t peer_addr(const void* local, uint32_t rank) 
   return r;
 }
 
-// Exclusive prefix sum of one int per thread over the CTA (fixed order); returns the total too.
-__device__ __forceinline__ int cta_exclusive_scan(int v, int* warp_sums, int* total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int inc = v;
+// Set bits of a bitmap of kWords words before each of the four words 4 lane .. 4 lane + 3; every
+// warp calls it for itself.
+__device__ __forceinline__ void bitmap_prefix(const uint32_t* words, int lane, int (&before)[4], int* total) {
+  const uint4 w = *reinterpret_cast<const uint4*>(&words[4 * lane]);
+  const int c0 = __popc(w.x), c1 = c0 + __popc(w.y), c2 = c1 + __popc(w.z), c3 = c2 + __popc(w.w);
+  int inc = c3;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
     const int t = __shfl_up_sync(0xffffffffu, inc, d);
     if (lane >= d) inc += t;
   }
-  __syncthreads();
-  if (lane == 31) warp_sums[warp] = inc;
-  __syncthreads();
-  int base = 0, tot = 0;
-#pragma unroll
-  for (int w = 0; w < kWarps; ++w) {
-    const int s = warp_sums[w];
-    if (w < warp) base += s;
-    tot += s;
-  }
-  *total = tot;
-  return base + inc - v;
+  *total = __shfl_sync(0xffffffffu, inc, 31);
+  before[0] = inc - c3;
+  before[1] = before[0] + c0;
+  before[2] = before[0] + c1;
+  before[3] = before[0] + c2;
+}
+
+// Two fp32 operations per instruction.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void fma2(uint64_t& acc, uint64_t a, uint64_t b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ float sum2(uint64_t v) {
+  float lo, hi;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+  return lo + hi;
 }
 
 // ---- Local Spatial Merging ----------------------------------------------------------------------
@@ -92,147 +103,173 @@ struct MergeParams {
   int32_t* merged_cnt;   // [B]
   float* window_sim;     // [B, (g/2)^2] or null
   int32_t grid, vecs;    // vecs = C / 8
+  uint32_t inv_grid, inv_half;   // ceil(2^20 / grid), ceil(2^20 / (grid / 2)): exact quotients of numbers below 4096
   float tau;
 };
 
-__global__ void __launch_bounds__(kThreads) spatial_merge_kernel(MergeParams p) {
+__device__ __forceinline__ uint4 ld_row(const uint4* p, uint64_t policy) {
+  uint4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p), "l"(policy));
+  return v;
+}
+
+__device__ __forceinline__ int quotient(int x, uint32_t inv) { return static_cast<int>((static_cast<uint32_t>(x) * inv) >> 20); }
+
+__global__ void __launch_bounds__(kThreads, 4) spatial_merge_kernel(MergeParams p) {
   __shared__ unsigned char merged_flag[kMaxSlots / 4];
-  __shared__ int warp_sums[kWarps];
+  __shared__ __align__(16) uint32_t emit[kWords];   // slots that emit a token: all of an unmerged window, the first of a merged one
+  __shared__ int first_row[kWords];                 // output row of a word's first emitting slot
   const int C = static_cast<int>(cluster_size()), rank = static_cast<int>(cluster_rank());
   const int b = blockIdx.x / C, g = p.grid, gw = g / 2, n_win = gw * gw, n_slot = g * g;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   cluster_arrive();          // "this CTA runs": peers wait for it before their first remote store
   bool peers_started = false;
+  for (int w = threadIdx.x; w < kWords; w += kThreads) emit[w] = 0u;
   pdl_launch_dependents();
   pdl_wait();
   const uint4* in = p.tokens + static_cast<size_t>(b) * n_slot * p.vecs;
+  // The tokens are read twice, the second time from L2, where the first reading keeps them and the
+  // merged rows pass through (64 images of 576 x 1024: 39.4 us with the hints, 43.6 without).
+  uint64_t keep, once;
+  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(keep));
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(once));
 
-  // 1. per window: the four norms and six dot products, fp32 accumulation.  The cluster's warps
-  //    share the windows; a window's flag is stored into every CTA's copy of the flag array.
+  // 1. per window: the four norms and six dot products, fp32 accumulation, two channels per
+  //    instruction.  The cluster's warps share the windows; a window's flag is stored into every
+  //    CTA's copy of the flag array.
   for (int w = rank * kWarps + warp; w < n_win; w += C * kWarps) {
-    const int wy = w / gw, wx = w % gw;
-    const int s0 = (2 * wy) * g + 2 * wx;
-    const uint4* r0 = in + static_cast<size_t>(s0) * p.vecs;
+    const int wy = quotient(w, p.inv_half), wx = w - wy * gw;
+    const uint4* r0 = in + static_cast<size_t>(2 * wy * g + 2 * wx) * p.vecs;
     const uint4* r1 = r0 + p.vecs;                          // (y, x+1)
     const uint4* r2 = r0 + static_cast<size_t>(g) * p.vecs; // (y+1, x)
     const uint4* r3 = r2 + p.vecs;
-    float n0 = 0, n1 = 0, n2 = 0, n3 = 0, d01 = 0, d02 = 0, d03 = 0, d12 = 0, d13 = 0, d23 = 0;
-#pragma unroll 2
+    uint64_t acc[10] = {};   // |0|^2 |1|^2 |2|^2 |3|^2 01 | 02 03 12 13 23
+#pragma unroll 1
     for (int x = lane; x < p.vecs; x += 32) {
-      const uint4 a = r0[x], c = r1[x], e = r2[x], f = r3[x];
+      const uint4 a = ld_row(r0 + x, keep), c = ld_row(r1 + x, keep), e = ld_row(r2 + x, keep), f = ld_row(r3 + x, keep);
       const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, cw[4] = {c.x, c.y, c.z, c.w};
       const uint32_t ew[4] = {e.x, e.y, e.z, e.w}, fw[4] = {f.x, f.y, f.z, f.w};
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-#pragma unroll
-        for (int hsel = 0; hsel < 2; ++hsel) {
-          const float v0 = hsel ? bf16_hi(aw[q]) : bf16_lo(aw[q]);
-          const float v1 = hsel ? bf16_hi(cw[q]) : bf16_lo(cw[q]);
-          const float v2 = hsel ? bf16_hi(ew[q]) : bf16_lo(ew[q]);
-          const float v3 = hsel ? bf16_hi(fw[q]) : bf16_lo(fw[q]);
-          n0 = fmaf(v0, v0, n0); n1 = fmaf(v1, v1, n1); n2 = fmaf(v2, v2, n2); n3 = fmaf(v3, v3, n3);
-          d01 = fmaf(v0, v1, d01); d02 = fmaf(v0, v2, d02); d03 = fmaf(v0, v3, d03);
-          d12 = fmaf(v1, v2, d12); d13 = fmaf(v1, v3, d13); d23 = fmaf(v2, v3, d23);
-        }
+        const uint64_t v0 = pack2(bf16_lo(aw[q]), bf16_hi(aw[q])), v1 = pack2(bf16_lo(cw[q]), bf16_hi(cw[q]));
+        const uint64_t v2 = pack2(bf16_lo(ew[q]), bf16_hi(ew[q])), v3 = pack2(bf16_lo(fw[q]), bf16_hi(fw[q]));
+        fma2(acc[0], v0, v0); fma2(acc[1], v1, v1); fma2(acc[2], v2, v2); fma2(acc[3], v3, v3);
+        fma2(acc[4], v0, v1); fma2(acc[5], v0, v2); fma2(acc[6], v0, v3);
+        fma2(acc[7], v1, v2); fma2(acc[8], v1, v3); fma2(acc[9], v2, v3);
       }
     }
-    n0 = warp_sum(n0); n1 = warp_sum(n1); n2 = warp_sum(n2); n3 = warp_sum(n3);
-    d01 = warp_sum(d01); d02 = warp_sum(d02); d03 = warp_sum(d03);
-    d12 = warp_sum(d12); d13 = warp_sum(d13); d23 = warp_sum(d23);
+    // sums over the lanes: the half-warps exchange five sums for five, then each reduces its own five
+    const bool upper = lane >= 16;
+    float v[5], o[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      const float lo = sum2(acc[i]), hi = sum2(acc[i + 5]);
+      v[i] = (upper ? hi : lo) + __shfl_xor_sync(0xffffffffu, upper ? lo : hi, 16);
+    }
+#pragma unroll
+    for (int d = 8; d >= 1; d >>= 1)
+#pragma unroll
+      for (int i = 0; i < 5; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], d);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) o[i] = __shfl_xor_sync(0xffffffffu, v[i], 16);   // (lower lanes: the upper ones' sums)
     if (!peers_started) {   // (warp-uniform) every CTA of the cluster has started: its shared memory exists
       cluster_wait();
       peers_started = true;
     }
-    if (lane == 0) {
-      const float tiny = 1e-30f;
-      const float l0 = fmaxf(sqrtf(n0), tiny), l1 = fmaxf(sqrtf(n1), tiny), l2 = fmaxf(sqrtf(n2), tiny),
-                  l3 = fmaxf(sqrtf(n3), tiny);
-      const float sim = (d01 / (l0 * l1) + d02 / (l0 * l2) + d03 / (l0 * l3) + d12 / (l1 * l2) + d13 / (l1 * l3) +
-                         d23 / (l2 * l3)) * (1.0f / 6.0f);
-      const uint32_t flag = sim > p.tau ? 1u : 0u;
-      for (int c = 0; c < C; ++c)
-        asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(peer_addr(&merged_flag[w], c)), "r"(flag) : "memory");
-      if (p.window_sim != nullptr) p.window_sim[static_cast<size_t>(b) * n_win + w] = sim;
-    }
+    const float tiny = 1e-30f;
+    const float l0 = fmaxf(sqrtf(v[0]), tiny), l1 = fmaxf(sqrtf(v[1]), tiny), l2 = fmaxf(sqrtf(v[2]), tiny), l3 = fmaxf(sqrtf(v[3]), tiny);
+    const float sim = (v[4] / (l0 * l1) + o[0] / (l0 * l2) + o[1] / (l0 * l3) + o[2] / (l1 * l2) + o[3] / (l1 * l3) +
+                       o[4] / (l2 * l3)) * (1.0f / 6.0f);   // (lane 0's is the one that counts)
+    const uint32_t flag = __shfl_sync(0xffffffffu, sim > p.tau ? 1u : 0u, 0);
+    if (lane < C)
+      asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(peer_addr(&merged_flag[w], lane)), "r"(flag) : "memory");
+    if (lane == 0 && p.window_sim != nullptr) p.window_sim[static_cast<size_t>(b) * n_win + w] = sim;
   }
   if (!peers_started) cluster_wait();   // a warp without a window: complete the prologue's barrier
   cluster_barrier();   // every flag has arrived in every CTA; no remote store after this point
 
-  // 2. which slots emit a token (all slots of an unmerged window, the first slot of a merged
-  //    one) and where: exclusive scan in raster order, by every CTA for itself; CTA 0 stores it
-  const int j0 = threadIdx.x * kOwn;
-  uint32_t emit = 0;
-#pragma unroll
-  for (int e = 0; e < kOwn; ++e) {
-    const int s = j0 + e;
-    if (s < n_slot) {
-      const int y = s / g, x = s % g;
-      const bool m = merged_flag[(y >> 1) * gw + (x >> 1)] != 0;
-      if (!m || (((y | x) & 1) == 0)) emit |= 1u << e;
-    }
+  // 2. which slots emit a token and where: a bitmap in raster order and its prefix counts, by every
+  //    CTA for itself
+  const int n_word = (n_slot + 31) / 32;
+  for (int w = warp; w < n_word; w += kWarps) {
+    const int s = 32 * w + lane, y = quotient(s, p.inv_grid), x = s - y * g;
+    const bool m = s < n_slot && merged_flag[(y >> 1) * gw + (x >> 1)] != 0;
+    const uint32_t word = __ballot_sync(0xffffffffu, s < n_slot && (!m || ((y | x) & 1) == 0));
+    if (lane == 0) emit[w] = word;
   }
-  int total;
-  int pos = cta_exclusive_scan(__popc(emit), warp_sums, &total);
-  __shared__ int16_t out_pos[kMaxSlots];     // output row of each emitting slot, -1 otherwise
-#pragma unroll
-  for (int e = 0; e < kOwn; ++e) {
-    const int s = j0 + e;
-    if (s < n_slot) {
-      if ((emit >> e) & 1u) {
-        out_pos[s] = static_cast<int16_t>(pos);
-        if (rank == 0) p.slots[static_cast<size_t>(b) * n_slot + pos] = s;
-        ++pos;
-      } else {
-        out_pos[s] = -1;
-      }
-    }
-  }
-  if (threadIdx.x == 0 && rank == 0) p.merged_cnt[b] = total;
   __syncthreads();
+  if (warp == 0) {
+    int before[4], total;
+    bitmap_prefix(emit, lane, before, &total);
+    *reinterpret_cast<int4*>(&first_row[4 * lane]) = make_int4(before[0], before[1], before[2], before[3]);
+    if (lane == 0 && rank == 0) p.merged_cnt[b] = total;
+  }
+  __syncthreads();
+  auto row_of = [&](int s) { return first_row[s >> 5] + __popc(emit[s >> 5] & ((1u << (s & 31)) - 1u)); };
+  for (int w = rank * kWarps + warp; w < n_word; w += C * kWarps)
+    if ((emit[w] >> lane) & 1u) p.slots[static_cast<size_t>(b) * n_slot + row_of(32 * w + lane)] = 32 * w + lane;
 
-  // 3. write the surviving rows: a copy, or the plain average of the window in fp32, rounded once
+  // 3. the surviving rows: copies of the tokens of unmerged windows, two rows and eight 16-byte loads
+  //    per lane in flight, ...
   uint4* out = p.merged + static_cast<size_t>(b) * n_slot * p.vecs;
-  for (int s = rank * kWarps + warp; s < n_slot; s += C * kWarps) {
-    const int o = out_pos[s];
-    if (o < 0) continue;
-    const int y = s / g, x = s % g;
-    const bool m = merged_flag[(y >> 1) * gw + (x >> 1)] != 0;
+  for (int s0 = rank * kWarps + warp; s0 < n_slot; s0 += 2 * C * kWarps) {
+    const uint4* src[2];
+    uint4* dst[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int s = s0 + i * C * kWarps, y = quotient(s, p.inv_grid), x = s - y * g;
+      const bool copy = s < n_slot && merged_flag[(y >> 1) * gw + (x >> 1)] == 0;
+      src[i] = copy ? in + static_cast<size_t>(s) * p.vecs : nullptr;
+      dst[i] = copy ? out + static_cast<size_t>(row_of(s)) * p.vecs : nullptr;
+    }
+    for (int v0 = lane; v0 < p.vecs; v0 += 4 * 32) {
+      uint4 t[2][4];
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (src[i] != nullptr && v0 + 32 * u < p.vecs) t[i][u] = ld_row(src[i] + v0 + 32 * u, once);
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (src[i] != nullptr && v0 + 32 * u < p.vecs) __stcs(dst[i] + v0 + 32 * u, t[i][u]);
+    }
+  }
+  //    ... and the plain average of every merged window in fp32, rounded once
+  for (int w = rank * kWarps + warp; w < n_win; w += C * kWarps) {
+    if (merged_flag[w] == 0) continue;
+    const int wy = quotient(w, p.inv_half), wx = w - wy * gw, s = 2 * wy * g + 2 * wx;
     const uint4* r0 = in + static_cast<size_t>(s) * p.vecs;
-    uint4* dst = out + static_cast<size_t>(o) * p.vecs;
-    if (!m) {
-      // a copy: four independent 16-byte loads in flight per lane, then the stores
-      for (int v0 = lane; v0 < p.vecs; v0 += 4 * 32) {
-        uint4 t[4];
+    const uint4* r1 = r0 + p.vecs;
+    const uint4* r2 = r0 + static_cast<size_t>(g) * p.vecs;
+    const uint4* r3 = r2 + p.vecs;
+    uint4* dst = out + static_cast<size_t>(row_of(s)) * p.vecs;
+#pragma unroll 1
+    for (int v = lane; v < p.vecs; v += 32) {
+      const uint4 a = ld_row(r0 + v, once), c = ld_row(r1 + v, once), e = ld_row(r2 + v, once), f = ld_row(r3 + v, once);
+      const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, cw[4] = {c.x, c.y, c.z, c.w};
+      const uint32_t ew[4] = {e.x, e.y, e.z, e.w}, fw[4] = {f.x, f.y, f.z, f.w};
+      uint32_t ow[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (v0 + 32 * u < p.vecs) t[u] = r0[v0 + 32 * u];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (v0 + 32 * u < p.vecs) dst[v0 + 32 * u] = t[u];
+      for (int q = 0; q < 4; ++q) {
+        const float lo = ((bf16_lo(aw[q]) + bf16_lo(cw[q])) + (bf16_lo(ew[q]) + bf16_lo(fw[q]))) * 0.25f;
+        const float hi = ((bf16_hi(aw[q]) + bf16_hi(cw[q])) + (bf16_hi(ew[q]) + bf16_hi(fw[q]))) * 0.25f;
+        const __nv_bfloat16 bl = __float2bfloat16_rn(lo), bh = __float2bfloat16_rn(hi);
+        ow[q] = static_cast<uint32_t>(__bfloat16_as_ushort(bl)) | (static_cast<uint32_t>(__bfloat16_as_ushort(bh)) << 16);
       }
-    } else {
-      const uint4* r1 = r0 + p.vecs;
-      const uint4* r2 = r0 + static_cast<size_t>(g) * p.vecs;
-      const uint4* r3 = r2 + p.vecs;
-      for (int v = lane; v < p.vecs; v += 32) {
-        const uint4 a = r0[v], c = r1[v], e = r2[v], f = r3[v];
-        const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, cw[4] = {c.x, c.y, c.z, c.w};
-        const uint32_t ew[4] = {e.x, e.y, e.z, e.w}, fw[4] = {f.x, f.y, f.z, f.w};
-        uint32_t ow[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float lo = ((bf16_lo(aw[q]) + bf16_lo(cw[q])) + (bf16_lo(ew[q]) + bf16_lo(fw[q]))) * 0.25f;
-          const float hi = ((bf16_hi(aw[q]) + bf16_hi(cw[q])) + (bf16_hi(ew[q]) + bf16_hi(fw[q]))) * 0.25f;
-          const __nv_bfloat16 bl = __float2bfloat16_rn(lo), bh = __float2bfloat16_rn(hi);
-          ow[q] = static_cast<uint32_t>(__bfloat16_as_ushort(bl)) | (static_cast<uint32_t>(__bfloat16_as_ushort(bh)) << 16);
-        }
-        dst[v] = make_uint4(ow[0], ow[1], ow[2], ow[3]);
-      }
+      __stcs(dst + v, make_uint4(ow[0], ow[1], ow[2], ow[3]));
     }
   }
 }
 
 // ---- Key Retaining ------------------------------------------------------------------------------
+constexpr int kParts = 2;         // a head's tokens of a CTA are two warps' work: 12 or 16 heads deal out evenly
+constexpr int kRanked = 64;       // tokens that are ranked against each other for a quartile, one per thread
+constexpr int kHalf = kThreads / 2;   // threads that work on a quartile
+
 struct KeySetParams {
   const __nv_bfloat16* q_cls;   // [B, H, D]
   const uint4* k;               // [B, H, M, D/8]
@@ -241,156 +278,264 @@ struct KeySetParams {
   int32_t* key_idx;             // [B, key_max]
   int32_t* key_cnt;             // [B]
   int32_t H, D, M, key_max;
+  int32_t part;                 // tokens of a warp's unit of work: ceil(ceil(M / CTAs) / kParts)
+  int32_t block;                // heads whose logits fit a CTA's shared memory at a time
   float scale_log2e;
 };
 
-__global__ void __launch_bounds__(kThreads) key_set_kernel(KeySetParams p) {
-  __shared__ __align__(16) float a[kMaxSlots];      // head-mean attention
-  __shared__ float z[kMaxSlots];      // one head's logits (log2 units)
-  __shared__ __align__(16) float q_s[256];
-  __shared__ float red[kWarps];
-  __shared__ float order[4];          // the four order statistics the quartiles interpolate
-  __shared__ int warp_sums[kWarps];
-  extern __shared__ float slab[];     // [cluster size][M] partial sums of the cluster's CTAs
+// The cluster's CTAs share the TOKENS: every CTA reads its share of every head's keys (all its loads
+// are independent, nothing is between them), a warp at a time the logits of one head and half of the
+// CTA's tokens, their maximum and the sum of their exponentials; one exchange of these statistics
+// over the cluster normalises all heads.  (Sharing the heads put six CTA-wide barriers into every
+// head and left the partial sums of all tokens to be exchanged: 36 us for 64 images of 576 tokens,
+// 16 heads x 64, where reading the keys takes 11.5 us; now 30.)
+__global__ void __launch_bounds__(kThreads, 4) key_set_kernel(KeySetParams p) {
+  __shared__ __align__(16) float a[kMaxSlots];      // CTA 0: head-mean attention; the others: of their own tokens
+  __shared__ __align__(16) uint32_t words[kWords];
+  __shared__ __align__(16) int hist[2][256];        // (one set per quartile)
+  __shared__ uint32_t ranked[2][kRanked], over[2];  // values of the cut bin; the smallest value above it
+  __shared__ int n_ranked[2];
+  __shared__ uint32_t order[2][2];                  // per quartile the two order statistics it interpolates
+  __shared__ uint32_t band[kWarps], bor[kWarps];
+  extern __shared__ __align__(16) unsigned char dyn[];
   const int C = static_cast<int>(cluster_size()), rank = static_cast<int>(cluster_rank());
   const int b = blockIdx.x / C, M = p.M, dv = p.D / 8;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float2* const stat = reinterpret_cast<float2*>(dyn);                  // [CTA][unit] (maximum, sum)
+  float2* const norm = stat + C * p.block * kParts;                     // [head] (maximum, 1 / (H sum)) over all tokens
+  float* const logits = reinterpret_cast<float*>(norm + p.block);       // [unit][part], log2 units
   cluster_arrive();          // "this CTA runs": peers wait for it before their first remote store
+  bool peers_started = false;
+  hist[0][threadIdx.x] = 0;
+  hist[1][threadIdx.x] = 0;
+  if (threadIdx.x < kWords) words[threadIdx.x] = 0u;
+  if (threadIdx.x < 2) {
+    n_ranked[threadIdx.x] = 0;
+    over[threadIdx.x] = 0xffffffffu;
+  }
   pdl_launch_dependents();
   pdl_wait();
-  for (int j = threadIdx.x; j < M; j += kThreads) a[j] = 0.0f;
   const float inv_h = 1.0f / static_cast<float>(p.H);
+  const int own = kParts * p.part, t0 = rank * own, n_own = max(0, min(own, M - t0));   // this CTA's tokens
+  // Coalesced rows: a group of `grp` lanes (the power of two >= D/8) reads one token's row as
+  // 16-byte vectors, a warp takes 32/grp consecutive tokens per step, five steps in flight (with 32 warps on
+  // an SM: eight in flight, a second trip for the ninth step of 36 tokens, took 36 us instead of 30).
+  int grp = 1;
+  while (grp < dv) grp <<= 1;
+  const int sub = lane & (grp - 1), tok = lane / grp, per_warp = 32 / grp;
+  float* const mine = a + t0;                       // (at the place where CTA 0 wants them)
 
-  for (int h = rank; h < p.H; h += C) {   // the cluster's CTAs share the heads
-    __syncthreads();   // q_s, z and red are free again
-    for (int d = threadIdx.x; d < p.D; d += kThreads)
-      q_s[d] = __bfloat162float(p.q_cls[(static_cast<size_t>(b) * p.H + h) * p.D + d]);
-    __syncthreads();
-    const uint4* kh = p.k + (static_cast<size_t>(b) * p.H + h) * M * dv;
-    // Coalesced rows: a group of `grp` lanes (the power of two >= D/8) reads one token's row as
-    // 16-byte vectors; a warp takes 32/grp consecutive tokens per step, four steps in flight.  Each
-    // lane keeps its eight query values in registers for the whole head.
-    int grp = 1;
-    while (grp < dv) grp <<= 1;
-    const int sub = lane % grp, tok_in_warp = lane / grp, per_warp = 32 / grp;
-    float qv[8];
+  for (int hb = 0; hb < p.H; hb += p.block) {
+    const int nh = min(p.block, p.H - hb), units = nh * kParts;
+    for (int u = warp; u < units; u += kWarps) {
+      const int h = hb + u / kParts, first = (u % kParts) * p.part, n = max(0, min(p.part, n_own - first));
+      uint4 qw = make_uint4(0, 0, 0, 0);
+      if (sub < dv) qw = reinterpret_cast<const uint4*>(p.q_cls)[(static_cast<size_t>(b) * p.H + h) * dv + sub];
+      const float qv[8] = {bf16_lo(qw.x), bf16_hi(qw.x), bf16_lo(qw.y), bf16_hi(qw.y),
+                           bf16_lo(qw.z), bf16_hi(qw.z), bf16_lo(qw.w), bf16_hi(qw.w)};
+      const uint4* const rows = p.k + ((static_cast<size_t>(b) * p.H + h) * M + t0 + first) * dv;
+      float* const z = logits + u * p.part;
+      float mx = -INFINITY;
+      constexpr int kFly = 5;
+      for (int base = 0; base < n; base += kFly * per_warp) {   // warp-uniform trip count
+        uint4 kv[kFly];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) qv[e] = sub < dv ? q_s[sub * 8 + e] : 0.0f;
-    float mx = -INFINITY;
-    const int step = kWarps * per_warp;
-    constexpr int kFly = 4;   // key rows in flight per lane
-    for (int base = warp * per_warp; base < M; base += kFly * step) {   // warp-uniform trip count
-      int jt[kFly];
-      uint4 kv[kFly];
+        for (int x = 0; x < kFly; ++x) {
+          const int j = base + x * per_warp + tok;
+          kv[x] = make_uint4(0, 0, 0, 0);
+          if (j < n && sub < dv) kv[x] = rows[static_cast<size_t>(j) * dv + sub];
+        }
 #pragma unroll
-      for (int u = 0; u < kFly; ++u) {
-        jt[u] = base + u * step + tok_in_warp;
-        kv[u] = make_uint4(0, 0, 0, 0);
-        if (jt[u] < M && sub < dv) kv[u] = kh[static_cast<size_t>(jt[u]) * dv + sub];
-      }
-#pragma unroll
-      for (int u = 0; u < kFly; ++u) {
-        float da = bf16_lo(kv[u].x) * qv[0];
-        da = fmaf(bf16_hi(kv[u].x), qv[1], da);
-        da = fmaf(bf16_lo(kv[u].y), qv[2], da);
-        da = fmaf(bf16_hi(kv[u].y), qv[3], da);
-        da = fmaf(bf16_lo(kv[u].z), qv[4], da);
-        da = fmaf(bf16_hi(kv[u].z), qv[5], da);
-        da = fmaf(bf16_lo(kv[u].w), qv[6], da);
-        da = fmaf(bf16_hi(kv[u].w), qv[7], da);
-        for (int d = grp >> 1; d >= 1; d >>= 1) da += __shfl_xor_sync(0xffffffffu, da, d);   // sum over the group's lanes (fixed tree)
-        if (sub == 0 && jt[u] < M) {
-          const float zz = da * p.scale_log2e;
-          z[jt[u]] = zz;
-          mx = fmaxf(mx, zz);
+        for (int x = 0; x < kFly; ++x) {
+          const int j = base + x * per_warp + tok;
+          float da = bf16_lo(kv[x].x) * qv[0];
+          da = fmaf(bf16_hi(kv[x].x), qv[1], da);
+          da = fmaf(bf16_lo(kv[x].y), qv[2], da);
+          da = fmaf(bf16_hi(kv[x].y), qv[3], da);
+          da = fmaf(bf16_lo(kv[x].z), qv[4], da);
+          da = fmaf(bf16_hi(kv[x].z), qv[5], da);
+          da = fmaf(bf16_lo(kv[x].w), qv[6], da);
+          da = fmaf(bf16_hi(kv[x].w), qv[7], da);
+          for (int d = grp >> 1; d >= 1; d >>= 1) da += __shfl_xor_sync(0xffffffffu, da, d);   // over the group's lanes (fixed tree)
+          if (j < n) {
+            da *= p.scale_log2e;
+            if (sub == 0) z[j] = da;
+            mx = fmaxf(mx, da);
+          }
         }
       }
-    }
 #pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
-    if (lane == 0) red[warp] = mx;
+      for (int d = 16; d >= 1; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
+      __syncwarp();
+      float sum = 0.0f;
+      for (int j = lane; j < n; j += 32) sum += exp2f(z[j] - mx);
+      sum = warp_sum(sum);
+      if (!peers_started) {   // (warp-uniform) every CTA of the cluster has started: its shared memory exists
+        cluster_wait();
+        peers_started = true;
+      }
+      if (lane < C)
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(peer_addr(&stat[rank * units + u], lane)), "f"(mx), "f"(sum)
+                     : "memory");
+    }
+    if (!peers_started) {
+      cluster_wait();
+      peers_started = true;
+    }
+    cluster_barrier();   // every CTA's statistics of these heads are everywhere
+    for (int h = threadIdx.x; h < nh; h += kThreads) {
+      float m = -INFINITY, total = 0.0f;
+      for (int c = 0; c < C; ++c)
+        for (int x = 0; x < kParts; ++x) m = fmaxf(m, stat[c * units + h * kParts + x].x);
+      for (int c = 0; c < C; ++c)
+        for (int x = 0; x < kParts; ++x) {
+          const float2 v = stat[c * units + h * kParts + x];
+          total = fmaf(v.y, exp2f(v.x - m), total);       // (no token: (-inf, 0))
+        }
+      norm[h] = make_float2(m, inv_h / total);
+    }
     __syncthreads();
-    mx = red[0];
-#pragma unroll
-    for (int w = 1; w < kWarps; ++w) mx = fmaxf(mx, red[w]);
-    float sum = 0.0f;
-    for (int j = threadIdx.x; j < M; j += kThreads) {
-      const float e = exp2f(z[j] - mx);
-      z[j] = e;
-      sum += e;
+    for (int t = threadIdx.x; t < n_own; t += kThreads) {
+      const int part = t / p.part, at = t - part * p.part;
+      float sum = hb == 0 ? 0.0f : mine[t];
+      for (int h = 0; h < nh; ++h)   // (from the logits: tokens with equal keys get equal bits whoever holds them)
+        sum = fmaf(exp2f(logits[(h * kParts + part) * p.part + at] - norm[h].x), norm[h].y, sum);
+      mine[t] = sum;
     }
-    sum = warp_sum(sum);
-    __syncthreads();   // everyone has read red
-    if (lane == 0) red[warp] = sum;
-    __syncthreads();
-    sum = 0.0f;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) sum += red[w];   // fixed order
-    const float f = inv_h / sum;
-    for (int j = threadIdx.x; j < M; j += kThreads) a[j] = fmaf(z[j], f, a[j]);
+    if (hb + p.block < p.H) cluster_barrier();   // the statistics are read: the next heads' may come
   }
-  // every CTA hands its partial sums to every CTA; each adds them in rank order (same result everywhere)
-  cluster_wait();            // every CTA of the cluster has started: its shared memory exists
-  for (int c = 0; c < C; ++c)
-    for (int j = threadIdx.x; j < M; j += kThreads)
-      asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(peer_addr(&slab[static_cast<size_t>(rank) * M + j], c)), "f"(a[j])
-                   : "memory");
-  cluster_barrier();
-  for (int j = threadIdx.x; j < M; j += kThreads) {
-    float sum = 0.0f;
-    for (int c = 0; c < C; ++c) sum += slab[static_cast<size_t>(c) * M + j];
-    a[j] = sum;
-  }
-  const int M4 = (M + 3) & ~3;
-  if (threadIdx.x < M4 - M) a[M + threadIdx.x] = INFINITY;   // padding that is never counted
-  __syncthreads();
-
-  // quartiles by rank counting: the element with r smaller ones (ties by index) is order statistic r.
-  // The cluster's CTAs share the tokens; whoever finds one of the four needed statistics stores it in CTA 0.
-  const float p1 = 0.25f * static_cast<float>(M - 1), p3 = 0.75f * static_cast<float>(M - 1);
-  const int r1 = static_cast<int>(floorf(p1)), r3 = static_cast<int>(floorf(p3));
-  const int r1h = min(r1 + 1, M - 1), r3h = min(r3 + 1, M - 1);
-  for (int j = threadIdx.x * C + rank; j < M; j += kThreads * C) {
-    const float aj = a[j];
-    int rk = 0;
-    for (int i = 0; i < M4; i += 4) {                          // four candidates per shared load
-      const float4 v = *reinterpret_cast<const float4*>(&a[i]);
-      rk += (v.x < aj || (v.x == aj && i < j)) ? 1 : 0;
-      rk += (v.y < aj || (v.y == aj && i + 1 < j)) ? 1 : 0;
-      rk += (v.z < aj || (v.z == aj && i + 2 < j)) ? 1 : 0;
-      rk += (v.w < aj || (v.w == aj && i + 3 < j)) ? 1 : 0;
-    }
-    if (rk == r1) asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(peer_addr(&order[0], 0)), "f"(aj) : "memory");
-    if (rk == r1h) asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(peer_addr(&order[1], 0)), "f"(aj) : "memory");
-    if (rk == r3) asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(peer_addr(&order[2], 0)), "f"(aj) : "memory");
-    if (rk == r3h) asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(peer_addr(&order[3], 0)), "f"(aj) : "memory");
+  for (int t = threadIdx.x; t < n_own; t += kThreads) {   // (each thread its own sums)
+    const float v = mine[t];
+    if (p.a_cls != nullptr) p.a_cls[static_cast<size_t>(b) * M + t0 + t] = v;
+    if (rank != 0) asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(peer_addr(&a[t0 + t], 0)), "f"(v) : "memory");
   }
   cluster_barrier();
   if (rank != 0) return;   // CTA 0 finishes alone; no store into another CTA's memory after this point
-  const float q1 = order[0] + (order[1] - order[0]) * (p1 - static_cast<float>(r1));
-  const float q3 = order[2] + (order[3] - order[2]) * (p3 - static_cast<float>(r3));
+
+  // Quartiles.  Each needs two neighbouring order statistics; half of the CTA finds the ones of Q1, half
+  // those of Q3.  Radix passes over the (non-negative) values from the highest bit in which two of
+  // them differ, until the cut bin holds few enough values to rank them against each other.
+  const float pos[2] = {0.25f * static_cast<float>(M - 1), 0.75f * static_cast<float>(M - 1)};
+  const int half = threadIdx.x / kHalf, th = threadIdx.x % kHalf;
+  const int want = static_cast<int>(floorf(half ? pos[1] : pos[0]));
+  uint32_t all_and = 0xffffffffu, all_or = 0u;
+  for (int j = threadIdx.x; j < M; j += kThreads) {
+    const uint32_t u = __float_as_uint(a[j]);
+    all_and &= u;
+    all_or |= u;
+  }
+  all_and = __reduce_and_sync(0xffffffffu, all_and);
+  all_or = __reduce_or_sync(0xffffffffu, all_or);
+  if (lane == 0) {
+    band[warp] = all_and;
+    bor[warp] = all_or;
+  }
+  __syncthreads();
+  all_and = __reduce_and_sync(0xffffffffu, band[lane & (kWarps - 1)]);
+  all_or = __reduce_or_sync(0xffffffffu, bor[lane & (kWarps - 1)]);
+  auto meet = [&]() {   // (of this half)
+    if (half == 0) asm volatile("bar.sync 1, %0;" ::"n"(kHalf) : "memory");
+    else asm volatile("bar.sync 2, %0;" ::"n"(kHalf) : "memory");
+  };
+  const uint32_t differ = all_and ^ all_or;
+  const int hb = differ ? 31 - __clz(differ) : 7;
+  uint32_t mask = hb >= 31 ? 0u : ~((2u << hb) - 1u), prefix = all_and & mask;
+  int rest = want, here = 0;
+  for (int shift = hb >= 7 ? hb - 7 : 0;; shift = shift > 8 ? shift - 8 : 0) {
+    for (int j = th; j < M; j += kHalf) {
+      const uint32_t u = __float_as_uint(a[j]);
+      if ((u & mask) == prefix) atomicAdd(&hist[half][(u >> shift) & 255u], 1);
+    }
+    meet();
+    // every warp scans the bins for itself: eight per lane
+    const int4 lo = *reinterpret_cast<const int4*>(&hist[half][8 * lane]), hi = *reinterpret_cast<const int4*>(&hist[half][8 * lane + 4]);
+    const int bins[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+    int sum = 0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) sum += bins[e];
+    int inc = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, inc, d);
+      if (lane >= d) inc += t;
+    }
+    int below = inc - sum, digit = -1, off = 0, cnt = 0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      if (below <= rest && rest < below + bins[e]) {
+        digit = 8 * lane + e;
+        off = rest - below;
+        cnt = bins[e];
+      }
+      below += bins[e];
+    }
+    const int owner = __ffs(__ballot_sync(0xffffffffu, digit >= 0)) - 1;
+    digit = __shfl_sync(0xffffffffu, digit, owner);
+    rest = __shfl_sync(0xffffffffu, off, owner);
+    here = __shfl_sync(0xffffffffu, cnt, owner);
+    prefix = (prefix & ~(255u << shift)) | (static_cast<uint32_t>(digit) << shift);
+    mask |= 255u << shift;
+    if (here <= kRanked || shift == 0) break;
+    meet();
+    hist[half][th] = 0;
+    hist[half][th + kHalf] = 0;
+    meet();
+  }
+  // the cut bin's values (beyond kRanked of them all digits are resolved and they are all the prefix),
+  // and the smallest value above it
+  uint32_t next = 0xffffffffu;
+  for (int j = th; j < M; j += kHalf) {
+    const uint32_t u = __float_as_uint(a[j]);
+    if ((u & mask) > prefix) next = min(next, u);
+    else if ((u & mask) == prefix && here <= kRanked) ranked[half][atomicAdd(&n_ranked[half], 1)] = u;
+  }
+  next = __reduce_min_sync(0xffffffffu, next);
+  if (lane == 0) atomicMin(&over[half], next);
+  meet();
+  if (here > kRanked) {
+    if (th == 0) {
+      order[half][0] = prefix;
+      order[half][1] = rest + 1 < here ? prefix : over[half];
+    }
+  } else if (th < here) {
+    const uint32_t me = ranked[half][th];
+    int rk = 0;
+#pragma unroll 4
+    for (int y = 0; y < here; ++y) {
+      const uint32_t o = ranked[half][y];
+      rk += o < me || (o == me && y < th) ? 1 : 0;
+    }
+    if (rk == rest) order[half][0] = me;
+    if (rk == rest + 1) order[half][1] = me;
+    if (rk == rest && rest + 1 >= here) order[half][1] = over[half];
+  }
+  __syncthreads();
+  float quart[2];
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const float lo = __uint_as_float(order[x][0]);
+    const float hi = static_cast<int>(floorf(pos[x])) + 1 < M ? __uint_as_float(order[x][1]) : lo;
+    quart[x] = lo + (hi - lo) * (pos[x] - floorf(pos[x]));
+  }
+  const float q1 = quart[0], q3 = quart[1];
   const float mu = q3 + 1.5f * (q3 - q1);
   if (threadIdx.x == 0 && p.mu_out != nullptr) p.mu_out[b] = mu;
 
   // O = { j : a[j] > mu }, ascending; at most key_max of them are stored (the lowest indices)
-  const int j0 = threadIdx.x * kOwn;
-  uint32_t is_key = 0;
-#pragma unroll
-  for (int e = 0; e < kOwn; ++e) {
-    const int j = j0 + e;
-    if (j < M) {
-      if (p.a_cls != nullptr) p.a_cls[static_cast<size_t>(b) * M + j] = a[j];
-      if (a[j] > mu) is_key |= 1u << e;
-    }
+  const int n_word = (M + 31) / 32;
+  for (int w = warp; w < n_word; w += kWarps) {
+    const int j = 32 * w + lane;
+    const uint32_t word = __ballot_sync(0xffffffffu, j < M && a[j] > mu);
+    if (lane == 0) words[w] = word;
   }
-  int total;
-  int pos = cta_exclusive_scan(__popc(is_key), warp_sums, &total);
-#pragma unroll
-  for (int e = 0; e < kOwn; ++e) {
-    if ((is_key >> e) & 1u) {
-      if (pos < p.key_max) p.key_idx[static_cast<size_t>(b) * p.key_max + pos] = j0 + e;
-      ++pos;
-    }
+  __syncthreads();
+  int before[4], total;
+  bitmap_prefix(words, lane, before, &total);
+  const int slot = warp & 3, mine_before = slot == 0 ? before[0] : (slot == 1 ? before[1] : (slot == 2 ? before[2] : before[3]));
+  for (int w = warp; w < n_word; w += kWarps) {   // (w & 3 is the same for all words of a warp)
+    const uint32_t word = words[w];
+    const int pos = __shfl_sync(0xffffffffu, mine_before, w >> 2) + __popc(word & ((1u << lane) - 1u));
+    if (((word >> lane) & 1u) && pos < p.key_max) p.key_idx[static_cast<size_t>(b) * p.key_max + pos] = 32 * w + lane;
   }
   if (threadIdx.x == 0) p.key_cnt[b] = total < p.key_max ? total : p.key_max;
 }
@@ -442,6 +587,8 @@ extern "C" mustdrop_status_t mustdrop_spatial_merge(int32_t batch, int32_t grid,
   p.merged = static_cast<uint4*>(merged);
   p.slots = slots; p.merged_cnt = merged_cnt; p.window_sim = window_sim;
   p.grid = grid; p.vecs = channels / 8; p.tau = tau;
+  p.inv_grid = ((1u << 20) + grid - 1) / grid;
+  p.inv_half = ((1u << 20) + grid / 2 - 1) / (grid / 2);
   const int n_win = (grid / 2) * (grid / 2);
   int cluster = 8;                                   // no more CTAs than there are rounds of windows for them
   while (cluster > 1 && (cluster - 1) * kWarps >= n_win) cluster >>= 1;
@@ -466,8 +613,14 @@ extern "C" mustdrop_status_t mustdrop_key_set(int32_t batch, int32_t n_heads, in
   p.H = n_heads; p.D = head_dim; p.M = n_tokens; p.key_max = key_max;
   p.scale_log2e = 1.4426950408889634f / sqrtf(static_cast<float>(head_dim));
   int cluster = 8;
-  while (cluster > n_heads) cluster >>= 1;           // 1, 2, 4 or 8 CTAs, at most one per head
-  const size_t smem = static_cast<size_t>(cluster) * n_tokens * sizeof(float);
+  while (cluster > 1 && n_tokens < 8 * cluster) cluster >>= 1;   // 1, 2, 4 or 8 CTAs
+  p.part = ((n_tokens + cluster - 1) / cluster + kParts - 1) / kParts;
+  // as many heads at a time as leave four CTAs on an SM (32 KB besides the static part), at least one
+  const size_t per_head = kParts * (sizeof(float2) * cluster + sizeof(float) * p.part) + sizeof(float2);
+  p.block = static_cast<int>(32 * 1024 / per_head);
+  if (p.block > n_heads) p.block = n_heads;
+  if (p.block < 1) p.block = 1;
+  const size_t smem = p.block * per_head;
   cudaError_t e = ensure_kernel_attributes(reinterpret_cast<const void*>(key_set_kernel), false);
   if (e != cudaSuccess) return finish(e);
   return finish(launch_cluster(key_set_kernel, batch, cluster, smem, static_cast<cudaStream_t>(cuda_stream), p));
