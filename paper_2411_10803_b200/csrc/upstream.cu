@@ -107,14 +107,6 @@ struct MergeParams {
   float tau;
 };
 
-__device__ __forceinline__ uint4 ld_row(const uint4* p, uint64_t policy) {
-  uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(p), "l"(policy));
-  return v;
-}
-
 __device__ __forceinline__ int quotient(int x, uint32_t inv) { return static_cast<int>((static_cast<uint32_t>(x) * inv) >> 20); }
 
 __global__ void __launch_bounds__(kThreads, 4) spatial_merge_kernel(MergeParams p) {
@@ -130,11 +122,6 @@ __global__ void __launch_bounds__(kThreads, 4) spatial_merge_kernel(MergeParams 
   pdl_launch_dependents();
   pdl_wait();
   const uint4* in = p.tokens + static_cast<size_t>(b) * n_slot * p.vecs;
-  // The tokens are read twice, the second time from L2, where the first reading keeps them and the
-  // merged rows pass through (64 images of 576 x 1024: 39.4 us with the hints, 43.6 without).
-  uint64_t keep, once;
-  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(keep));
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(once));
 
   // 1. per window: the four norms and six dot products, fp32 accumulation, two channels per
   //    instruction.  The cluster's warps share the windows; a window's flag is stored into every
@@ -148,7 +135,7 @@ __global__ void __launch_bounds__(kThreads, 4) spatial_merge_kernel(MergeParams 
     uint64_t acc[10] = {};   // |0|^2 |1|^2 |2|^2 |3|^2 01 | 02 03 12 13 23
 #pragma unroll 1
     for (int x = lane; x < p.vecs; x += 32) {
-      const uint4 a = ld_row(r0 + x, keep), c = ld_row(r1 + x, keep), e = ld_row(r2 + x, keep), f = ld_row(r3 + x, keep);
+      const uint4 a = r0[x], c = r1[x], e = r2[x], f = r3[x];
       const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, cw[4] = {c.x, c.y, c.z, c.w};
       const uint32_t ew[4] = {e.x, e.y, e.z, e.w}, fw[4] = {f.x, f.y, f.z, f.w};
 #pragma unroll
@@ -212,7 +199,9 @@ __global__ void __launch_bounds__(kThreads, 4) spatial_merge_kernel(MergeParams 
     if ((emit[w] >> lane) & 1u) p.slots[static_cast<size_t>(b) * n_slot + row_of(32 * w + lane)] = 32 * w + lane;
 
   // 3. the surviving rows: copies of the tokens of unmerged windows, two rows and eight 16-byte loads
-  //    per lane in flight, ...
+  //    per lane in flight, ...  (The tokens are read a second time, from L2 as far as they are still
+  //    there.  Hints that keep them - evict_last on the first reading - make this kernel 10 % faster and
+  //    the key set behind it slower by more.)
   uint4* out = p.merged + static_cast<size_t>(b) * n_slot * p.vecs;
   for (int s0 = rank * kWarps + warp; s0 < n_slot; s0 += 2 * C * kWarps) {
     const uint4* src[2];
@@ -230,7 +219,7 @@ __global__ void __launch_bounds__(kThreads, 4) spatial_merge_kernel(MergeParams 
       for (int i = 0; i < 2; ++i)
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-          if (src[i] != nullptr && v0 + 32 * u < p.vecs) t[i][u] = ld_row(src[i] + v0 + 32 * u, once);
+          if (src[i] != nullptr && v0 + 32 * u < p.vecs) t[i][u] = src[i][v0 + 32 * u];
 #pragma unroll
       for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -249,7 +238,7 @@ __global__ void __launch_bounds__(kThreads, 4) spatial_merge_kernel(MergeParams 
     uint4* dst = out + static_cast<size_t>(row_of(s)) * p.vecs;
 #pragma unroll 1
     for (int v = lane; v < p.vecs; v += 32) {
-      const uint4 a = ld_row(r0 + v, once), c = ld_row(r1 + v, once), e = ld_row(r2 + v, once), f = ld_row(r3 + v, once);
+      const uint4 a = r0[v], c = r1[v], e = r2[v], f = r3[v];
       const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, cw[4] = {c.x, c.y, c.z, c.w};
       const uint32_t ew[4] = {e.x, e.y, e.z, e.w}, fw[4] = {f.x, f.y, f.z, f.w};
       uint32_t ow[4];
