@@ -134,15 +134,18 @@ mustdrop_status_t mustdrop_filter_plan(const mustdrop_config_t* c, mustdrop_plan
     return MUSTDROP_ERR_INVALID_ARG;
   }
 
-  // The device is only consulted for the SM count; a box without a GPU still gets a plan.
+  // The device is only consulted for the SM count and the L2 size; a box without a GPU still gets a plan.
   p->device = -1;
   p->sm_count = 148;
+  p->l2_bytes = 126 << 20;
   int dev = 0;
   if (cudaGetDevice(&dev) == cudaSuccess) {
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0) {
       p->device = dev;
       p->sm_count = sms;
+      int l2 = 0;
+      if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) == cudaSuccess && l2 > 0) p->l2_bytes = l2;
     }
   }
   (void)cudaGetLastError();

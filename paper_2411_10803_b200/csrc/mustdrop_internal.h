@@ -88,6 +88,7 @@ struct mustdrop_plan {
   mustdrop::Resolved r;
   int32_t device;
   int32_t sm_count;
+  int64_t l2_bytes;
   int32_t score_variant;
   size_t ws_bytes;
   size_t ws_rowstats_off;   // float2 [B,H,N]: (row max in log2 units, 1 / row sum)

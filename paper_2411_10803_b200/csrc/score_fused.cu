@@ -85,6 +85,7 @@ struct FusedParams {
   int32_t per_head;                   // 1: i_out = head mean of the per-head maxima over the text rows (PH instantiations)
   int32_t early_inputs;               // 1: q_text / k may be read before the stream's earlier work has completed (caller's promise)
   long long wait_cycles;              // clock cycles after which a wait between the warp roles gives up
+  int32_t keep_keys;                  // 1: the keys are left in L2 for the gather that follows
   float scale_log2e, inv_heads;
 };
 
@@ -200,8 +201,7 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
       ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
       : "memory");
 }
-// The same copy with an L2 eviction-priority hint (keys are read exactly once: evict them first,
-// so that they do not push out data other kernels left in L2).
+// The same copy with an L2 eviction-priority hint.
 __device__ __forceinline__ void tma_load_4d_hint(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
                                                  uint32_t bar, uint64_t policy) {
   asm volatile(
@@ -232,6 +232,11 @@ __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.
 __device__ __forceinline__ uint64_t l2_evict_first_policy() {
   uint64_t policy;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+  return policy;
+}
+__device__ __forceinline__ uint64_t l2_normal_policy() {
+  uint64_t policy;
+  asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy));
   return policy;
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -660,7 +665,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     if (warp == kTmaWarp && lane == 0) {
       // ---------------- TMA producer ----------------
       const int key0 = static_cast<int>(rank) * p.tk;
-      const uint64_t stream_once = l2_evict_first_policy();
+      const uint64_t key_policy = p.keep_keys ? l2_normal_policy() : l2_evict_first_policy();
       if (!p.early_inputs) pdl_wait();   // q_text / k may be the output of the kernel just before this one
       if (p.split) {
         int q_issued = 0, k_issued = 0;   // tiles started so far
@@ -685,8 +690,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             const uint32_t full = smem_u32(&bars.full[ki]);
             const uint32_t k_dst = k_base + ki * kh_bytes;
             mbar_expect_tx(full, kh_bytes);
-            tma_load_4d_hint(k_dst, &k_map, 0, key0 + hv * p.cpl, h0 + h, b, full, stream_once);
-            tma_load_4d_hint(k_dst + p.cpl * 128u, &k_map, 64, key0 + hv * p.cpl, h0 + h, b, full, stream_once);
+            tma_load_4d_hint(k_dst, &k_map, 0, key0 + hv * p.cpl, h0 + h, b, full, key_policy);
+            tma_load_4d_hint(k_dst + p.cpl * 128u, &k_map, 64, key0 + hv * p.cpl, h0 + h, b, full, key_policy);
             ++k_issued;
           }
         }
@@ -720,7 +725,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
   #pragma unroll
             for (int hv = 0; hv < HALVES; ++hv)
               tma_load_4d_hint(k_dst + slab * (p.tk * 128u) + hv * (p.cpl * 128u), &k_map, slab * 64, key0 + hv * p.cpl,
-                               h0 + h, b, full, stream_once);
+                               h0 + h, b, full, key_policy);
           }
           issued = h + 1;
         }
@@ -1779,6 +1784,13 @@ cudaError_t launch_fused_common(const mustdrop_plan& plan, const FusedGeometry& 
   p.per_head = r.per_head_max;
   p.early_inputs = (r.inputs_ready && vis_cnt == nullptr) ? 1 : 0;
   p.wait_cycles = r.wait_cycles > 0 ? r.wait_cycles : kWaitCycles;
+  // The gather reads the kept tokens' keys a second time.  Where the keys of the requests that are
+  // resident at once are not far beyond L2 they stay there with normal priority (16 requests of 640
+  // keys, budget 192: 64.1 -> 57.1 us a call; 8 of 2944: 83.3 -> 82.7; two waves of 33 requests of 704
+  // keys and 40 heads: 245 -> 242); beyond twice its size they leave first, so that they do not push
+  // out what other kernels keep there (64 requests of 640 keys: 105.4, with normal priority 107.4).
+  const int64_t at_once = geo.resident > 0 && geo.resident < r.B && !geo.gx ? geo.resident : r.B;
+  p.keep_keys = at_once * r.H * r.L * 256 <= 2 * plan.l2_bytes;
   p.scale_log2e = r.scale_log2e;
   p.inv_heads = 1.0f / static_cast<float>(r.H);
 
