@@ -186,7 +186,9 @@ __device__ __forceinline__ float ld_cluster_f32(uint32_t cluster_addr) {
   asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr) : "memory");
   return v;
 }
+// (.aligned: every lane of the warp together, so the warp is made whole first)
 __device__ __forceinline__ void cluster_sync_all() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ uint32_t cluster_cta_rank() {
@@ -614,6 +616,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     cta_sync();
     if (p.groups > 1) cluster_sync_all();   // the head sums of every group are staged
     finish();       // (exp warps: the scores from the staged head sums)
+    __syncwarp();   // a warp whose lanes had different keys is whole again before what is aligned below
     if (p.gx) {
       // grid plan: the request's CTAs are no cluster and do not meet here: the filter's selection
       // recognises every score by its parity.  (A CTA that gives up tells nobody: its peers run into
@@ -1054,6 +1057,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       // the other group's loop.  Handing over only when the group gets to its next head - two heads
       // on - saves that wait but measured the same, and with two buffers that next head needs the
       // very buffer: its MMAs wait for the add warps, who wait for the hand-over.)
+      __syncwarp();   // (only the senders were in the branch above)
       tc_wait_st();
       tc_fence_before();
       __syncwarp();
@@ -1109,7 +1113,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         }
       }
       pdl_wait();
-      asm volatile("bar.sync 1, 256;" ::: "memory");
+      SelectSyncGroup::sync();
       for (int c = c_lo + threadIdx.x; c < c_hi; c += kExpThreads) {
         const int j = static_cast<int>(rank) * p.tk + c - p.vis_start;   // vision-relative index
         if (j < 0 || j >= p.M) continue;
@@ -1134,10 +1138,11 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         }
         p.g_out[static_cast<size_t>(b) * p.M + j] = gv;
         p.i_out[static_cast<size_t>(b) * p.M + j] = iv;
-        if constexpr (FILTER) {   // ... and to the selection, in every CTA of the request
-          if (p.gx) {
-            st_parity(p.gx_scores + static_cast<size_t>(b) * p.M + j, gv, iv, parity);
-          } else {
+        // ... and to the selection, in every CTA of the request.  (Grid plans: by the score call as well -
+        // every call counts, so every call has to leave words of its own parity behind.)
+        if (p.gx) st_parity(p.gx_scores + static_cast<size_t>(b) * p.M + j, gv, iv, parity);
+        if constexpr (FILTER) {
+          if (!p.gx) {
             const uint32_t at = smem_u32(val_g + j);
             for (int cta = 0; cta < req_ctas; ++cta) {
               const uint32_t to = map_to_cta(at, cta);

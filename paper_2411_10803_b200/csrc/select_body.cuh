@@ -77,7 +77,11 @@ struct SelectSyncCta {
   static __device__ __forceinline__ void sync() { __syncthreads(); }
 };
 struct SelectSyncGroup {
-  static __device__ __forceinline__ void sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+  // (bar.sync is aligned: every lane of the warp together)
+  static __device__ __forceinline__ void sync() {
+    __syncwarp();
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+  }
 };
 
 // Larger float <=> larger unsigned image (handles negative values and -0 as well).

@@ -42,6 +42,7 @@ __device__ __forceinline__ uint32_t cluster_size() {
   return r;
 }
 __device__ __forceinline__ void cluster_barrier() {
+  __syncwarp();   // (.aligned: every lane of the warp together)
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // The two halves of the barrier.  Shared memory of another CTA may only be touched once that CTA
@@ -423,6 +424,7 @@ __global__ void __launch_bounds__(kThreads, 4) key_set_kernel(KeySetParams p) {
   all_and = __reduce_and_sync(0xffffffffu, band[lane & (kWarps - 1)]);
   all_or = __reduce_or_sync(0xffffffffu, bor[lane & (kWarps - 1)]);
   auto meet = [&]() {   // (of this half)
+    __syncwarp();
     if (half == 0) asm volatile("bar.sync 1, %0;" ::"n"(kHalf) : "memory");
     else asm volatile("bar.sync 2, %0;" ::"n"(kHalf) : "memory");
   };
