@@ -50,7 +50,6 @@ constexpr int kMmaWarp = kTmaWarp + 1;            // warp 13; warps 14-15 only f
 constexpr int kThreads = 16 * 32;
 constexpr int kChunk = 16;                  // TMEM columns per tcgen05.ld / st
 constexpr int kMaxCluster = 16;               // beyond 8 the cluster size is non-portable (opt-in per kernel)
-constexpr int kMaxGridCtas = 32;              // CTAs per request of a grid plan
 constexpr int kMaxQBufs = 4;                  // shared-memory ring of text-query tiles (one per head)
 constexpr int kMaxKBufs = 8;                  // shared-memory ring of key half-tiles (HALVES per head)
 constexpr int kMinBufs = 3;                 // tensor-memory buffers: MMA, exp and add stages in flight (two for 176-column tiles) ...
@@ -79,9 +78,8 @@ struct FusedParams {
   // Statistics exchange through global memory instead of distributed shared memory ("grid" plans:
   // the CTAs of a request are ordinary CTAs of the grid, any number of them, all resident at once).
   int32_t gx;                         // 1: grid plan (cluster = CTAs per request, launched without a cluster)
-  float2* gx_stats;                   // [B][H][CTAs per request][rows] (stabiliser, sum with the call's parity as its sign)
-  float2* gx_scores;                  // [B][M] (G, I with the call's parity as its sign)
-  uint32_t* gx_cnt;                   // [B] calls completed, [B] CTAs of the request that have left the call (zero between calls)
+  float2* gx_stats;                   // [B][H][CTAs per request][rows][pairs] (stabiliser, sum)
+  uint32_t* gx_cnt;                   // [B*H] CTAs that published a head, [B] scores stored, [B] barrier passed, [B] CTAs that left; zero between calls
   int32_t per_head;                   // 1: i_out = head mean of the per-head maxima over the text rows (PH instantiations)
   int32_t early_inputs;               // 1: q_text / k may be read before the stream's earlier work has completed (caller's promise)
   long long wait_cycles;              // clock cycles after which a wait between the warp roles gives up
@@ -137,19 +135,18 @@ __device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p) {
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
-// Statistics of a row on their way through global memory: one 64-bit word of the stabiliser and
-// the sum, whose sign - a sum is never negative - carries the parity of the call.  Every call
-// writes every word once, so a reader recognises this call's word by itself: no fence, no counter.
-__device__ __forceinline__ void st_parity(float2* dst, float m, float l, uint32_t parity) {
-  const uint32_t lo = __float_as_uint(m), hi = (__float_as_uint(l) & 0x7fffffffu) | (parity << 31);
-  asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(dst), "l"(static_cast<uint64_t>(hi) << 32 | lo) : "memory");
+// Bounded wait until a counter has reached its target (same give-up rules as mbar_wait).
+__device__ __forceinline__ bool count_wait(const uint32_t* p, uint32_t target, volatile int* abort_flag, long long limit) {
+  if (ld_acquire_gpu(p) >= target) return true;
+  const long long t0 = clock64();
+  while (ld_acquire_gpu(p) < target) {
+    if (*abort_flag != 0 || clock64() - t0 > limit) {
+      *abort_flag = 1;
+      return false;
+    }
+  }
+  return true;
 }
-__device__ __forceinline__ float2 ld_word(const float2* src) {
-  uint64_t v;
-  asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(src) : "memory");
-  return make_float2(__uint_as_float(static_cast<uint32_t>(v)), __uint_as_float(static_cast<uint32_t>(v >> 32)));
-}
-__device__ __forceinline__ bool has_parity(const float2& word, uint32_t parity) { return __float_as_uint(word.y) >> 31 == parity; }
 // Bounded wait.  Returns false (and raises the CTA's abort flag) when the wait ran out or the
 // CTA has already given up.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long limit) {
@@ -411,6 +408,7 @@ struct __align__(8) Barriers {
   uint64_t sfull[kMaxSlots];    // all CTAs' (max, sum) pairs of a head have arrived
   uint64_t fin;                  // add warps meet before staging the head sums
   uint64_t ph;                   // add warps meet once per head (per-head maxima of Eq. 10)
+  uint64_t gsent[kMaxBufs];      // grid plans: exp warps -> publishing thread: this CTA's pairs of a head are in global memory
   uint64_t gfull[kMaxGatherSlots];   // filter tail: a gathered row has landed in its slot
 };
 
@@ -558,6 +556,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
   const uint32_t slot_pairs = static_cast<uint32_t>(p.cluster) * NROWS;
   // PH only: [2][4 add warps][tk] per-head column maxima of each warp's text rows, double-buffered over heads
   float* const ph_stage = reinterpret_cast<float*>(stats + static_cast<size_t>(p.n_slot) * slot_pairs);
+  // grid plans only: [n_buf][rows] the pairs of this CTA's own exp warps, per tensor-memory buffer
+  float2* const own_pairs = reinterpret_cast<float2*>(ph_stage + (PH ? 2 * kAddWarps * p.tk : 0));
 
   __shared__ SelectShared sel_sh;       // (FILTER: cleared and the key set marked long before the scores are complete)
   if constexpr (FILTER) select_clear(sel_sh, threadIdx.x, kThreads);
@@ -575,6 +575,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     for (int s = 0; s < kMaxSlots; ++s) mbar_init(smem_u32(&bars.sfull[s]), p.gx ? 32 : 1);
     mbar_init(smem_u32(&bars.fin), kAddThreads);
     mbar_init(smem_u32(&bars.ph), kAddThreads);
+    for (int s = 0; s < kMaxBufs; ++s) mbar_init(smem_u32(&bars.gsent[s]), kExpWarps / kColGroups);
     for (int s = 0; s < kMaxGatherSlots; ++s) mbar_init(smem_u32(&bars.gfull[s]), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -618,19 +619,35 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     finish();       // (exp warps: the scores from the staged head sums)
     __syncwarp();   // a warp whose lanes had different keys is whole again before what is aligned below
     if (p.gx) {
-      // grid plan: the request's CTAs are no cluster and do not meet here: the filter's selection
-      // recognises every score by its parity.  (A CTA that gives up tells nobody: its peers run into
-      // their own limits.)
-      if (threadIdx.x == 0 && *abort_flag != 0) {
-        record_status(p.workspace, MUSTDROP_ERR_TIMEOUT, blockIdx.x);
-        cluster_abort_s = 1;
-      }
-      // every warp of this CTA has read its parity: the last CTA of the request counts the call
-      if (threadIdx.x == kThreads - 1 && *abort_flag == 0) {
-        uint32_t* const left = p.gx_cnt + gridDim.x / p.cluster + b;
-        if (atomicAdd(left, 1u) == static_cast<uint32_t>(p.cluster) - 1u) {
-          *left = 0u;
-          p.gx_cnt[b] += 1u;
+      // grid plan: the request's CTAs are no cluster.  In the filter kernel they meet through a
+      // counter in global memory: every CTA's scores are stored before any CTA selects.  (A CTA
+      // that gives up tells nobody: its peers run into their own limits.)
+      if (threadIdx.x == 0) {
+        const size_t n_req = gridDim.x / p.cluster;
+        if (*abort_flag == 0) {
+          // every CTA has seen all of its heads complete when it gets here: the last one of the
+          // request to do so clears the heads' counters for the next call (one counted visit per
+          // CTA instead of one per head, whose returned value the fetch warp would have to wait for)
+          uint32_t* const left = p.gx_cnt + n_req * p.H + 2 * n_req + b;
+          if (atomicAdd(left, 1u) == static_cast<uint32_t>(p.cluster) - 1u) {
+            for (int hh = 0; hh < p.H; ++hh) p.gx_cnt[static_cast<size_t>(b) * p.H + hh] = 0u;
+            *left = 0u;
+          }
+        }
+        if (FILTER && *abort_flag == 0) {
+          uint32_t* const stored = p.gx_cnt + n_req * p.H + b;
+          uint32_t* const passed = stored + n_req;
+          __threadfence();
+          atomicAdd(stored, 1u);
+          if (count_wait(stored, static_cast<uint32_t>(p.cluster), abort_flag, wait_limit) &&
+              atomicAdd(passed, 1u) == static_cast<uint32_t>(p.cluster) - 1u) {
+            *stored = 0u;   // the last one through leaves the counters as the next call expects them
+            *passed = 0u;
+          }
+        }
+        if (*abort_flag != 0) {
+          record_status(p.workspace, MUSTDROP_ERR_TIMEOUT, blockIdx.x);
+          cluster_abort_s = 1;
         }
       }
       cta_sync();
@@ -832,26 +849,23 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       }
     }
     if constexpr (FILTER) {
-      if (warp == kMmaWarp + 2) {
+      if (warp == kMmaWarp + 1) {
         pdl_wait();   // the key set may come from the kernel just before this one
         select_mark_keys(ft.sel, sel_sh, b, lane, 32, req_rank == 0);
       }
     }
-    if (warp > kMmaWarp && p.gx) {
-      // ---------------- statistics fetch warps (grid plans) ----------------
-      // Two warps, alternate heads.  Every CTA's exp warps store their rows' words straight to global
-      // memory.  A fetch warp copies the head's block of words (all CTAs of the request) into a
-      // statistics slot, looks at four words of each CTA (one per exp warp), and copies again until
-      // all of them are this call's - the add warps find their statistics in shared memory as with a
-      // cluster, and the round trips to L2 are off their path.  (They look at every word's parity as
-      // they read it, and fetch for themselves what was not there after all.)  A trip to L2 takes
-      // ~1.3 us here, with every SM streaming keys, so their number is what counts.  (A publishing warp
-      // that fenced and counted and a fetch warp that polled the counter before it copied needed
-      // four: 8 requests of 2944 keys 97.4 us a call, now 92.7.)
-      // A slot is reused once the add warps are done with the head that used it.
-      pdl_wait();   // parity and words belong to the workspace: an earlier call may still use them
-      const uint32_t parity = (ld_acquire_gpu(p.gx_cnt + b) + 1u) & 1u;
-      for (int h = warp - kMmaWarp - 1; h < n_heads; h += 2) {
+    if (warp == kMmaWarp + 1 && p.gx) {
+      // ---------------- statistics fetch warp (grid plans) ----------------
+      // Per head: wait until every CTA of the request has published its pairs (a counter in global
+      // memory), then copy the head's block of pairs from global memory (L2) into a statistics slot
+      // with asynchronous copies that arrive on the slot's barrier - the add warps find their
+      // statistics in shared memory exactly as with a cluster, and the round trips to L2 are off
+      // their path.  A slot is reused once the add warps are done with the head that used it.
+      pdl_wait();   // the counters belong to the workspace: an earlier call may still be resetting them
+      const uint32_t target = static_cast<uint32_t>(p.cluster);   // one counted release per CTA and head
+      const uint32_t slot_bytes_gx = slot_pairs * 8u;
+      int ready = 0;   // heads below this one are known to be published by every CTA of the request
+      for (int h = 0; h < n_heads; ++h) {
         const int slot = h % p.n_slot;
         if (h >= p.n_slot) {
           const int u = h - p.n_slot;
@@ -859,27 +873,51 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                                                  static_cast<uint32_t>(u / p.n_buf) & 1u, abort_flag, wait_limit)))
             break;
         }
-        const float2* const src = p.gx_stats + (static_cast<size_t>(b) * p.H + h) * slot_pairs;
-        float2* const dst = stats + static_cast<size_t>(slot) * slot_pairs;
-        const long long t0 = clock64();
-        bool there = false, ok = true;
-        while (!there && ok) {
-          for (uint32_t r = 2u * lane; r < slot_pairs; r += 64u)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst + r)), "l"(src + r) : "memory");
-          asm volatile("cp.async.wait_all;" ::: "memory");
-          __syncwarp();
-          there = true;
-#pragma unroll
-          for (int e = 0; e < kMaxGridCtas / 8; ++e) {
-            const int x = min(lane + 32 * e, 4 * p.cluster - 1);
-            there = there && has_parity(dst[(x + 1) * (NROWS / 4) - 1], parity);
+        const size_t bh = static_cast<size_t>(b) * p.H + h;
+        if (h >= ready) {
+          // one round trip tells about 32 heads: lane i looks at the counter of head h + i, and
+          // the run of complete heads from h on is taken in one go
+          const uint32_t* const mine = p.gx_cnt + static_cast<size_t>(b) * p.H + (h + lane < p.H ? h + lane : p.H - 1);
+          const long long t0 = clock64();
+          bool ok = true;
+          for (;;) {
+            const bool full = ld_acquire_gpu(mine) >= target;
+            const unsigned not_full = __ballot_sync(0xffffffffu, !(full && h + lane < p.H));
+            const int run = not_full == 0u ? 32 : __ffs(not_full) - 1;
+            if (run > 0) { ready = h + run; break; }
+            if (*abort_flag != 0 || clock64() - t0 > wait_limit) { *abort_flag = 1; ok = false; }
+            if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
           }
-          there = __all_sync(0xffffffffu, there);
-          if (!there && (*abort_flag != 0 || clock64() - t0 > wait_limit)) *abort_flag = 1;
-          ok = __all_sync(0xffffffffu, there || *abort_flag == 0);
+          if (!ok) break;
         }
-        if (!ok) break;
-        mbar_arrive(smem_u32(&bars.sfull[slot]));
+        const unsigned char* const src = reinterpret_cast<const unsigned char*>(p.gx_stats + bh * slot_pairs);
+        const uint32_t dst = smem_u32(stats + static_cast<size_t>(slot) * slot_pairs);
+        for (uint32_t off = lane * 16u; off < slot_bytes_gx; off += 32u * 16u)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + off), "l"(src + off) : "memory");
+        asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&bars.sfull[slot])) : "memory");
+      }
+      asm volatile("cp.async.wait_all;" ::: "memory");   // no copy of this warp is in flight when the CTA leaves
+    } else if (warp == kMmaWarp + 2 && p.gx) {
+      // ---------------- publishing warp (grid plans) ----------------
+      // Once all exp warps of this CTA have left their pairs of a head in shared memory: merge the
+      // pairs of each row into one, store it to global memory, then one fence and one counted
+      // release for the CTA - the round trip of the fence is off the exp warps' path.
+      pdl_wait();   // global memory of the workspace: not before the stream's earlier work is done
+      for (int h = 0; h < n_heads; ++h) {
+        const int buf = h % p.n_buf;
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.gsent[buf]), static_cast<uint32_t>(h / p.n_buf) & 1u,
+                                               abort_flag, wait_limit)))
+          break;
+        const size_t bh = static_cast<size_t>(b) * p.H + h;
+        float2* const dst = p.gx_stats + (bh * p.cluster + rank) * NROWS;
+        for (int r = lane; r < NROWS; r += 32) {
+          dst[r] = own_pairs[buf * NROWS + r];
+        }
+        __syncwarp();
+        if (lane == 0) {
+          __threadfence();
+          atomicAdd(p.gx_cnt + bh, 1u);
+        }
       }
     }
     if constexpr (FILTER) {
@@ -926,11 +964,6 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     const bool sender = (half == 0);           // with two halves, lanes s and s+16 share a row: the lower one sends
     const uint32_t pair_idx = rank * NROWS + row;                              // this thread's pair in a slot
 
-    uint32_t parity = 0u;                      // grid plans: marks this call's words of statistics
-    if (p.gx) {
-      pdl_wait();   // (the workspace is not touched before the stream's earlier work is done)
-      parity = (ld_acquire_gpu(p.gx_cnt + b) + 1u) & 1u;
-    }
     for (int h = g; h < n_heads; h += kColGroups) {
       const int buf = h % p.n_buf;
       const uint32_t bph = static_cast<uint32_t>(h / p.n_buf) & 1u;
@@ -1048,7 +1081,11 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       }
       if (HALVES == 2) lsum += __shfl_xor_sync(0xffffffffu, lsum, 16);
       if (p.gx) {
-        if (sender) st_parity(p.gx_stats + (static_cast<size_t>(b) * p.H + h) * slot_pairs + pair_idx, mx, lsum, parity);
+        // grid plan: the pair stays in this CTA's shared memory; the publishing warp merges the CTA's
+        // pairs of a row and sends one pair per row on its way through global memory
+        if (sender) own_pairs[buf * NROWS + row] = make_float2(mx, lsum);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bars.gsent[buf]));
       } else if (sender) {
         for (int c = 0; c < p.cluster; ++c)
           st_async_f32x2(map_to_cta(slot_addr, group * p.cluster + c), mx, lsum, map_to_cta(bar_addr, group * p.cluster + c));
@@ -1138,10 +1175,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         }
         p.g_out[static_cast<size_t>(b) * p.M + j] = gv;
         p.i_out[static_cast<size_t>(b) * p.M + j] = iv;
-        // ... and to the selection, in every CTA of the request.  (Grid plans: by the score call as well -
-        // every call counts, so every call has to leave words of its own parity behind.)
-        if (p.gx) st_parity(p.gx_scores + static_cast<size_t>(b) * p.M + j, gv, iv, parity);
-        if constexpr (FILTER) {
+        if constexpr (FILTER) {   // ... and to the selection, in every CTA of the request (grid plans: through g_out / i_out)
           if (!p.gx) {
             const uint32_t at = smem_u32(val_g + j);
             for (int cta = 0; cta < req_ctas; ++cta) {
@@ -1164,31 +1198,24 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       pdl_wait();   // the outputs written below may still be read by an earlier kernel in the stream
       uint32_t* const val_i = val_g + select_pad(p.M);
       if (p.gx) {
-        // grid plan: the scores as the request's CTAs have stored them (a score that is not there
-        // yet is looked at again)
-        const float2* const words = p.gx_scores + static_cast<size_t>(b) * p.M;
-        const long long t0 = clock64();
+        // grid plan: the scores as the request's CTAs have stored them, eight strips' loads in flight
+        const float* const g_row = p.g_out + static_cast<size_t>(b) * p.M;
+        const float* const i_row = p.i_out + static_cast<size_t>(b) * p.M;
 #pragma unroll 1
         for (int j0 = threadIdx.x; j0 < Mb; j0 += 8 * kExpThreads) {
-          float2 w[8];
-          bool there = false;
-          while (!there) {
-            there = true;
+          float gv[8], iv[8];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) w[e] = ld_word(words + min(j0 + e * kExpThreads, Mb - 1));
-#pragma unroll
-            for (int e = 0; e < 8; ++e) there = there && has_parity(w[e], parity);
-            if (!there && (*abort_flag != 0 || clock64() - t0 > wait_limit)) {
-              *abort_flag = 1;
-              break;
-            }
+          for (int e = 0; e < 8; ++e) {
+            const int j = min(j0 + e * kExpThreads, Mb - 1);
+            gv[e] = __ldcg(g_row + j);
+            iv[e] = __ldcg(i_row + j);
           }
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
             const int j = j0 + e * kExpThreads;
             if (j < Mb) {
-              val_g[j] = __float_as_uint(w[e].x);
-              val_i[j] = __float_as_uint(fabsf(w[e].y));
+              val_g[j] = __float_as_uint(gv[e]);
+              val_i[j] = __float_as_uint(iv[e]);
             }
           }
         }
@@ -1198,11 +1225,6 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         select_request<1, SelectSyncGroup>(ft.sel, sel_sh, scratch, val_g, val_i, b, threadIdx.x, req_rank == 0, kept_list, &kept_total_s);
       else
         select_request<4, SelectSyncGroup>(ft.sel, sel_sh, scratch, val_g, val_i, b, threadIdx.x, req_rank == 0, kept_list, &kept_total_s);
-      if (p.gx && *abort_flag != 0 && threadIdx.x == 0) {   // some scores never came
-        record_status(p.workspace, MUSTDROP_ERR_TIMEOUT, blockIdx.x);
-        ft.sel.kept_cnt[b] = -1;
-        kept_total_s = 0;
-      }
       if (threadIdx.x == 0) MD_TRACE(0, 12);   // selection done
       cta_sync();   // the list is complete: the copy thread may start
       return;
@@ -1230,11 +1252,6 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
 #pragma unroll
     for (int x = 0; x < PHK; ++x) ph_acc[x] = 0.0f;
     const bool real_row = row < p.N;     // lanes beyond the text rows carry padding
-    uint32_t parity = 0u;                // grid plans: the sign of this call's words of statistics
-    if (p.gx) {
-      pdl_wait();
-      parity = (ld_acquire_gpu(p.gx_cnt + b) + 1u) << 31;
-    }
 
     int h = 0;
     for (; h < n_heads; ++h) {
@@ -1250,42 +1267,20 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         // f = 1 / sum over CTAs of l_c 2^(m_c - m_own).  Independent terms, four loads in flight: the
         // loop is on every head's serial path (as a maximum first and a sum over the CTAs second it
         // took 0.5 us with 2 CTAs and 0.8 us with 16).  A sum that overflows means that this CTA's
-        // share is below 2^-127: f = 0.  (Grid plans: the sign of a sum is the call's parity.)
+        // share is below 2^-127: f = 0.  Grid plans: one merged pair per CTA in the slot; this CTA's own
+        // stabilisers are still in its shared memory (until the buffer is released below).
         const float2* const srow = stats + slot * slot_pairs + row;
-        float own = srow[rank * NROWS].x;
+        const float own = p.gx ? own_pairs[buf * NROWS + row].x : srow[rank * NROWS].x;
         float l0 = 0.0f, l1 = 0.0f;
-        uint32_t signs = 0u;   // sign set: some word does not carry the parity of this call
 #pragma unroll 1
         for (int c = 0; c < p.cluster; c += 4) {
           float2 v[4];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            v[e] = c + e < p.cluster ? srow[(c + e) * NROWS] : make_float2(-INFINITY, __uint_as_float(parity));
-            signs |= __float_as_uint(v[e].y) ^ parity;
-          }
-          l0 = fmaf(fabsf(v[0].y), ex2(v[0].x - own), l0);     // an empty pair is (-inf, 0): contributes 0
-          l1 = fmaf(fabsf(v[1].y), ex2(v[1].x - own), l1);
-          l0 = fmaf(fabsf(v[2].y), ex2(v[2].x - own), l0);
-          l1 = fmaf(fabsf(v[3].y), ex2(v[3].x - own), l1);
-        }
-        if (p.gx && (signs >> 31) != 0u) {   // (rare) a word was copied before it was stored: fetch the row's words again
-          const float2* const row_words = p.gx_stats + (static_cast<size_t>(b) * p.H + h) * slot_pairs + row;
-          const long long t0 = clock64();
-          auto fetch = [&](int c) {
-            float2 v = ld_word(row_words + c * NROWS);
-            while (((__float_as_uint(v.y) ^ parity) >> 31) != 0u && *abort_flag == 0) {
-              if (clock64() - t0 > wait_limit) *abort_flag = 1;
-              v = ld_word(row_words + c * NROWS);
-            }
-            return v;
-          };
-          own = fetch(static_cast<int>(rank)).x;
-          l0 = l1 = 0.0f;
-#pragma unroll 1
-          for (int c = 0; c < p.cluster; ++c) {
-            const float2 v = fetch(c);
-            l0 = fmaf(fabsf(v.y), ex2(v.x - own), l0);
-          }
+          for (int e = 0; e < 4; ++e) v[e] = c + e < p.cluster ? srow[(c + e) * NROWS] : make_float2(-INFINITY, 0.0f);
+          l0 = fmaf(v[0].y, ex2(v[0].x - own), l0);     // an empty pair is (-inf, 0): contributes 0
+          l1 = fmaf(v[1].y, ex2(v[1].x - own), l1);
+          l0 = fmaf(v[2].y, ex2(v[2].x - own), l0);
+          l1 = fmaf(v[3].y, ex2(v[3].x - own), l1);
         }
         f = own == -INFINITY ? 0.0f : 1.0f / (l0 + l1);   // (own = -inf: the row sees none of this CTA's keys)
       }
@@ -1677,7 +1672,7 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
 bool plan_score_grid(const Resolved& r, int sm_count, int forced_ctas, FusedGeometry* out) {
   const int halves = r.N <= 64 ? 2 : 1;
   const int nrows = 128 / halves;
-  const int max_g = sm_count / r.B < kMaxGridCtas ? sm_count / r.B : kMaxGridCtas;
+  const int max_g = sm_count / r.B < 32 ? sm_count / r.B : 32;
   double best = -1.0;
   FusedGeometry g{};
   for (int c = 2; c <= max_g; ++c) {
@@ -1695,19 +1690,21 @@ bool plan_score_grid(const Resolved& r, int sm_count, int forced_ctas, FusedGeom
     int n_buf = kTmemCols / cpl;
     if (n_buf > kMaxBufs) n_buf = kMaxBufs;
     if (n_buf < kMinBufs) continue;
-    // shared memory: statistics slots the fetch warps fill (a head's words of all the request's
+    // shared memory: statistics slots the fetch warp fills (a head's pairs of all the request's
     // CTAs; at least two, so that the next head's are fetched while this one is added) and stages
-    const size_t slot = static_cast<size_t>(c) * nrows * 8;                 // one word per row and CTA
-    if (avail < 2 * slot + 2 * stage) continue;
-    // (No more slots than buffers: the fetch warps learn that a slot is free from the buffer barrier
-    // of the head that used it, by parity; were one n_buf heads behind the add warps, that barrier
-    // could complete a second phase unseen.  Slots before a third stage: a slot is held for a trip to
-    // L2 or two, a stage for a load and an MMA.)
-    int n_slot = static_cast<int>((avail - 2 * stage) / slot);
-    if (n_slot > n_buf) n_slot = n_buf;
-    int n_q = static_cast<int>((avail - n_slot * slot) / stage);
+    const int epr = ach <= 5 ? 1 : kColGroups;   // (room for two pairs per row on wide tiles: see plan_score_fused)
+    const size_t slot = static_cast<size_t>(c) * nrows * 8;                 // one merged pair per row and CTA
+    const size_t own = static_cast<size_t>(n_buf) * nrows * epr * 8;        // the CTA's own pairs, per buffer
+    if (avail < own + 2 * slot + 2 * stage) continue;
+    int n_q = static_cast<int>((avail - own - 2 * slot) / stage);
     if (n_q > 3) n_q = 3;
-    size_t smem_bytes = n_q * stage + n_slot * slot + 1024 + ph_bytes;
+    // (No more slots than buffers: the fetch warp learns that a slot is free from the buffer barrier
+    // of the head that used it, by parity; were it n_buf heads behind the add warps, that barrier
+    // could complete a second phase unseen.)
+    int n_slot = static_cast<int>((avail - own - n_q * stage) / slot);
+    if (n_slot > 6) n_slot = 6;
+    if (n_slot > n_buf) n_slot = n_buf;
+    size_t smem_bytes = n_q * stage + n_slot * slot + own + 1024 + ph_bytes;
     if (smem_bytes < kMinSmem) smem_bytes = kMinSmem;
     // Cost per head and CTA (microseconds): streaming the stage at ~45 GB/s per SM; the exp stage
     // (measured: ~0.011 us per column of a lane, two heads at a time on narrow tiles); the
@@ -1734,7 +1731,7 @@ bool plan_score_grid(const Resolved& r, int sm_count, int forced_ctas, FusedGeom
 
 size_t grid_plan_stats_bytes(const Resolved& r, const FusedGeometry& g) {
   const int nrows = 128 / g.halves;
-  return static_cast<size_t>(r.B) * r.H * g.cluster * nrows * 8;   // one word per row, CTA and head
+  return static_cast<size_t>(r.B) * r.H * g.cluster * nrows * sizeof(float2);   // one merged pair per row, CTA and head
 }
 
 namespace {
@@ -1785,7 +1782,6 @@ cudaError_t launch_fused_common(const mustdrop_plan& plan, const FusedGeometry& 
   p.gx = geo.gx;
   p.gx_cnt = reinterpret_cast<uint32_t*>(static_cast<unsigned char*>(workspace) + plan.ws_gx_cnt_off);
   p.gx_stats = reinterpret_cast<float2*>(static_cast<unsigned char*>(workspace) + plan.ws_gx_stats_off);
-  p.gx_scores = reinterpret_cast<float2*>(static_cast<unsigned char*>(workspace) + plan.ws_gx_scores_off);
   p.per_head = r.per_head_max;
   p.early_inputs = (r.inputs_ready && vis_cnt == nullptr) ? 1 : 0;
   p.wait_cycles = r.wait_cycles > 0 ? r.wait_cycles : kWaitCycles;
