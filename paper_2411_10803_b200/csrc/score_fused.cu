@@ -79,7 +79,7 @@ struct FusedParams {
   // the CTAs of a request are ordinary CTAs of the grid, any number of them, all resident at once).
   int32_t gx;                         // 1: grid plan (cluster = CTAs per request, launched without a cluster)
   float2* gx_stats;                   // [B][H][CTAs per request][rows][pairs] (stabiliser, sum)
-  uint32_t* gx_cnt;                   // [B*H] CTAs that published a head, [B] scores stored, [B] barrier passed, [B] CTAs that left; zero between calls
+  uint32_t* gx_cnt;                   // [B*H] CTAs that published a head, [B] scores stored, [B] CTAs that left; zero between calls
   int32_t per_head;                   // 1: i_out = head mean of the per-head maxima over the text rows (PH instantiations)
   int32_t early_inputs;               // 1: q_text / k may be read before the stream's earlier work has completed (caller's promise)
   long long wait_cycles;              // clock cycles after which a wait between the warp roles gives up
@@ -134,6 +134,9 @@ __device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p) {
   uint32_t v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
+}
+__device__ __forceinline__ void add_release_gpu(uint32_t* p) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
 }
 // Bounded wait until a counter has reached its target (same give-up rules as mbar_wait).
 __device__ __forceinline__ bool count_wait(const uint32_t* p, uint32_t target, volatile int* abort_flag, long long limit) {
@@ -623,27 +626,10 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       // counter in global memory: every CTA's scores are stored before any CTA selects.  (A CTA
       // that gives up tells nobody: its peers run into their own limits.)
       if (threadIdx.x == 0) {
-        const size_t n_req = gridDim.x / p.cluster;
-        if (*abort_flag == 0) {
-          // every CTA has seen all of its heads complete when it gets here: the last one of the
-          // request to do so clears the heads' counters for the next call (one counted visit per
-          // CTA instead of one per head, whose returned value the fetch warp would have to wait for)
-          uint32_t* const left = p.gx_cnt + n_req * p.H + 2 * n_req + b;
-          if (atomicAdd(left, 1u) == static_cast<uint32_t>(p.cluster) - 1u) {
-            for (int hh = 0; hh < p.H; ++hh) p.gx_cnt[static_cast<size_t>(b) * p.H + hh] = 0u;
-            *left = 0u;
-          }
-        }
         if (FILTER && *abort_flag == 0) {
-          uint32_t* const stored = p.gx_cnt + n_req * p.H + b;
-          uint32_t* const passed = stored + n_req;
-          __threadfence();
-          atomicAdd(stored, 1u);
-          if (count_wait(stored, static_cast<uint32_t>(p.cluster), abort_flag, wait_limit) &&
-              atomicAdd(passed, 1u) == static_cast<uint32_t>(p.cluster) - 1u) {
-            *stored = 0u;   // the last one through leaves the counters as the next call expects them
-            *passed = 0u;
-          }
+          uint32_t* const stored = p.gx_cnt + static_cast<size_t>(gridDim.x / p.cluster) * p.H + b;
+          add_release_gpu(stored);   // (the CTA's scores: ordered before it by the barrier above)
+          (void)count_wait(stored, static_cast<uint32_t>(p.cluster), abort_flag, wait_limit);
         }
         if (*abort_flag != 0) {
           record_status(p.workspace, MUSTDROP_ERR_TIMEOUT, blockIdx.x);
@@ -677,6 +663,19 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     while (clock64() - t0 < 40000) {}
     __syncwarp();
     cluster_sync_all();
+  };
+  // Grid plans, one thread of a role that has nothing else to do by then: every CTA has seen all of its
+  // heads complete and all scores stored when it is counted, and the last one of the request clears
+  // the request's counters for the next call.
+  auto count_leaving = [&]() {
+    if (!p.gx || threadIdx.x != kTmaWarp * 32) return;
+    const size_t n_req = gridDim.x / p.cluster;
+    uint32_t* const left = p.gx_cnt + n_req * p.H + n_req + b;
+    if (atomicAdd(left, 1u) == static_cast<uint32_t>(p.cluster) - 1u) {
+      for (int hh = 0; hh < p.H; ++hh) p.gx_cnt[static_cast<size_t>(b) * p.H + hh] = 0u;
+      p.gx_cnt[n_req * p.H + b] = 0u;
+      *left = 0u;
+    }
   };
   int32_t* const kept_list = reinterpret_cast<int32_t*>(stage_ptr);   // filter tail: the request's kept indices
 
@@ -914,20 +913,19 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           dst[r] = own_pairs[buf * NROWS + r];
         }
         __syncwarp();
-        if (lane == 0) {
-          __threadfence();
-          atomicAdd(p.gx_cnt + bh, 1u);
-        }
+        if (lane == 0) add_release_gpu(p.gx_cnt + bh);   // (the warp's stores: ordered before it by __syncwarp)
       }
     }
     if constexpr (FILTER) {
       // filter tail, TMA / MMA warps: nothing to do but to meet the others
       common_exit([] {});
       if (cluster_gave_up()) { leave_after_give_up(ft.sel.kept_cnt); return; }
+      count_leaving();
       cta_sync();   // pairs with the barrier after the selection
       return;
     } else {
       common_exit([] {});
+      if (!cluster_gave_up()) count_leaving();
     }
   } else if (warp < kExpWarps) {
     // ---------------- exp warps ----------------
@@ -1651,7 +1649,8 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
       // ... and of a request: start, fill and exit (more where CTAs of a next wave have to wait for
       // it), and the reduction over the head groups.
       const double t_req = 3.0 + heads * t_head + t_chain + (grp > 1 ? 1.0 + 0.5 * grp : 0.0);
-      const double est = waves * t_req + (waves - 1) * 15.0;
+      // (every CTA at work is worth a little: the gather is shared by all of them)
+      const double est = waves * t_req + (waves - 1) * 15.0 - 0.03 * (active < sm_count ? active : sm_count);
       if (best < 0.0 || est < best - 1e-9) {
         best = est;
         g.halves = halves; g.cluster = c; g.groups = grp; g.tk = tk; g.cpl = cpl; g.n_q = n_q; g.n_k = n_k; g.split = split;
