@@ -160,8 +160,14 @@ mustdrop_status_t mustdrop_filter_plan(const mustdrop_config_t* c, mustdrop_plan
     const bool force_split = c->debug_score_variant == MUSTDROP_DEBUG_VARIANT_ROW_SPLIT;
     const bool force_grid = c->debug_score_variant == MUSTDROP_DEBUG_VARIANT_GRID;
     const double k_mb = 256.0e-6 * r.B * r.H * r.L;
-    // the two-pass kernel's measured rate, and its second pass's walk over the heads
-    const double two_pass_us = k_mb * (0.6 + 0.7 * r.N / 128.0) + 3.0 * r.H;
+    // the two-pass kernel's measured rate, less where heads x requests leave SMs without a CTA (one request
+    // of 8 heads, 4124 keys and 78 text rows: 175 us, 59 as a grid plan; the factor is bounded because a
+    // handful of heads is also where the grid plan's own start counts), and its second pass's walk over the
+    // heads
+    double idle = static_cast<double>(p->sm_count) / (r.B * r.H);
+    idle = idle < 1.0 ? 1.0 : (idle > 2.0 ? 2.0 : idle);
+    const double two_pass_us =
+        k_mb * (0.6 + 0.7 * r.N / 128.0) * idle + 3.0 * r.H + mustdrop::gather_us(r, p->sm_count);
     double chosen_us = two_pass_us;
     p->row_split = 0;
     if (allow_fused && !force_split && !force_grid && plan_score_fused(r, p->sm_count, forced_cluster, &p->fused)) {
@@ -186,8 +192,8 @@ mustdrop_status_t mustdrop_filter_plan(const mustdrop_config_t* c, mustdrop_plan
       mustdrop::FusedGeometry ga, gb;
       if (plan_score_fused(r, p->sm_count, forced_cluster, &ga, 0, 64) &&
           plan_score_fused(r, p->sm_count, forced_cluster, &gb, 64, r.N - 64)) {
-        // (the second launch reads no keys before the first has completed)
-        const double split_us = ga.est_us + gb.est_us + 8.0;
+        // (the second launch reads no keys before the first has completed, and starts and fills anew)
+        const double split_us = ga.est_us + gb.est_us + 20.0;
         if (force_split || (!want && forced_cluster == 0 && split_us < chosen_us)) {
           p->score_variant = kScoreFusedCluster;
           p->row_split = 1;
@@ -203,7 +209,7 @@ mustdrop_status_t mustdrop_filter_plan(const mustdrop_config_t* c, mustdrop_plan
     if (allow_fused && !force_split && (force_grid || (!want && forced_cluster == 0))) {
       mustdrop::FusedGeometry gg;
       if (plan_score_grid(r, p->sm_count, force_grid ? forced_cluster : 0, &gg) &&
-          (force_grid || gg.est_us < chosen_us * (p->row_split ? 1.0 : 0.9))) {
+          (force_grid || gg.est_us < chosen_us * 0.97)) {
         p->score_variant = kScoreFusedCluster;
         p->row_split = 0;
         p->fused = gg;

@@ -112,6 +112,7 @@ cudaError_t launch_score_two_pass(const mustdrop_plan& p, const void* q_text, co
                                   const int32_t* vis_cnt = nullptr);
 bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, FusedGeometry* out, int row0 = 0,
                       int n_rows = 0);
+double gather_us(const Resolved& r, double ctas);   // the planner's estimate of the gather
 // Grid plan of the same kernel (all CTAs of the batch resident at once, statistics through global
 // memory); false when the batch leaves fewer than two CTAs per request or the shape does not fit.
 bool plan_score_grid(const Resolved& r, int sm_count, int forced_ctas, FusedGeometry* out);

@@ -27,6 +27,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -1533,6 +1534,14 @@ int max_resident_clusters(int cluster) {
 
 }  // namespace
 
+// Time of the gather when `ctas` CTAs share it: a CTA's one copying thread moves ~33 GB/s (one way), all of
+// them together what the memory takes.  (25 requests of 179 rows: 55 us a call on 125 CTAs, 64 on 100.)
+double gather_us(const Resolved& r, double ctas) {
+  const double rows = r.rebuild ? r.out_rows : (r.mode == MUSTDROP_MODE_BUDGET ? r.cap : r.cap / 3.0);
+  const double bytes = rows * r.B * (2.0 * r.hidden + 2.0 * 256.0 * r.H);
+  return std::max(bytes / (33.0e3 * ctas), 2.0 * bytes / 7.0e6);
+}
+
 // Geometry of the fused kernel for a problem; false when the shape is outside what it covers.
 // row0 / n_rows: the text rows the launch covers (n_rows = 0: all of them).
 bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, FusedGeometry* out, int row0, int n_rows) {
@@ -1629,28 +1638,32 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
       const long waves = (r.B + resident - 1) / resident;
       const int heads = (r.H + grp - 1) / grp;
       const double active = static_cast<double>(size) * (r.B < resident ? r.B : resident);
-      // Cost of a head in a CTA (microseconds): streaming its stage (an SM alone draws up to 150 GB/s, all
-      // of them together ~7 TB/s), the exp stage (two heads at a time), the MMA -> exp -> exchange ->
-      // add chain spread over the buffers, the add stage.
-      const double rate = 7.0e6 / active < 150.0e3 ? 7.0e6 / active : 150.0e3;   // bytes per microsecond
-      const double t_stream = static_cast<double>(stage) / rate;
-      const double t_exp = 0.45 + 0.2 * (cpl / kChunk);
-      const double t_chain = t_exp + 1.3 + (c > 1 ? 0.4 + 0.08 * c : 0.2);
+      // Cost of a head in a CTA (microseconds): streaming its stage (an SM alone draws up to 150 GB/s; the
+      // keys of all of them come from memory at ~7 TB/s, the queries they share mostly from L2), the exp
+      // stage (two heads at a time), the MMA -> exp -> exchange -> add chain spread over the buffers, the
+      // add stage.
+      const double t_memory = (tk + nrows / c) * 256.0 * active / 7.0e6;
+      const double t_stream = std::max(static_cast<double>(stage) / 150.0e3, t_memory);
+      const double t_exp = 0.35 + 0.24 * (cpl / kChunk);
+      const double t_chain = t_exp + 1.0 + (c > 1 ? 0.4 + 0.08 * c : 0.2);
       double t_head = t_chain / n_buf;
       if (is_tight) {
         // Tight slots: the exchange over the cluster is on the critical path of every head (d = 2)
-        // or of every head twice (d = 1).  Measured per head: 2.6 .. 3.3 us at 11 .. 16 CTAs with
+        // or of every head twice (d = 1).  Measured per head: 2.1 .. 2.8 us at 11 .. 16 CTAs with
         // d = 2, 4.3 us at 10 CTAs with d = 1; a third more with 128 text rows on the lanes.
-        t_head = (n_slot == 4 ? 1.8 + 0.09 * c : 3.0 + 0.13 * c) * (halves == 1 ? 1.3 : 1.0);
+        t_head = (n_slot == 4 ? 1.5 + 0.08 * c : 3.0 + 0.13 * c) * (halves == 1 ? 1.3 : 1.0);
       }
       if (t_head < t_exp / 2) t_head = t_exp / 2;
       if (t_head < t_stream) t_head = t_stream;
       if (t_head < 1.15) t_head = 1.15;
       // ... and of a request: start, fill and exit (more where CTAs of a next wave have to wait for
-      // it), and the reduction over the head groups.
-      const double t_req = 3.0 + heads * t_head + t_chain + (grp > 1 ? 1.0 + 0.5 * grp : 0.0);
-      // (every CTA at work is worth a little: the gather is shared by all of them)
-      const double est = waves * t_req + (waves - 1) * 15.0 - 0.03 * (active < sm_count ? active : sm_count);
+      // it), the first exchange of 128 rows, and the reduction over the head groups.
+      const double t_req = 3.0 + heads * t_head + t_chain + (c > 1 && halves == 1 ? 1.0 : 0.0) +
+                           (grp > 1 ? 1.0 + 0.5 * grp : 0.0);
+      // (a launch of the last text rows also selects and gathers; what it shares out besides the rows' bytes
+      // makes every CTA worth a little)
+      double est = waves * t_req + (waves - 1) * 20.0;
+      if (row0 + n_rows == r.N) est += gather_us(r, active) - 0.015 * active;
       if (best < 0.0 || est < best - 1e-9) {
         best = est;
         g.halves = halves; g.cluster = c; g.groups = grp; g.tk = tk; g.cpl = cpl; g.n_q = n_q; g.n_k = n_k; g.split = split;
@@ -1719,7 +1732,7 @@ bool plan_score_grid(const Resolved& r, int sm_count, int forced_ctas, FusedGeom
       best = score;
       g.halves = halves; g.cluster = c; g.tk = tk; g.cpl = cpl; g.n_q = n_q; g.n_k = 0; g.split = 0; g.n_buf = n_buf;
       g.ach = ach; g.groups = 1; g.n_slot = n_slot; g.gx = 1; g.resident = sm_count; g.row0 = 0; g.n_rows = r.N;
-      g.est_us = static_cast<float>(r.H * t_head + 12.0);    // (+ filling and draining the longer chain)
+      g.est_us = static_cast<float>(r.H * t_head + 12.0 + gather_us(r, c * r.B));   // (+ filling and draining the longer chain)
       g.smem_bytes = smem_bytes;
     }
   }
