@@ -192,7 +192,7 @@ mustdrop_status_t mustdrop_filter_plan(const mustdrop_config_t* c, mustdrop_plan
       mustdrop::FusedGeometry ga, gb;
       if (plan_score_fused(r, p->sm_count, forced_cluster, &ga, 0, 64) &&
           plan_score_fused(r, p->sm_count, forced_cluster, &gb, 64, r.N - 64)) {
-        // (the second launch reads no keys before the first has completed, and starts and fills anew)
+        // (the second launch starts and fills anew)
         const double split_us = ga.est_us + gb.est_us + 20.0;
         if (force_split || (!want && forced_cluster == 0 && split_us < chosen_us)) {
           p->score_variant = kScoreFusedCluster;

@@ -83,6 +83,9 @@ struct FusedParams {
   uint32_t* gx_cnt;                   // [B*H] CTAs that published a head, [B] scores stored, [B] CTAs that left; zero between calls
   int32_t per_head;                   // 1: i_out = head mean of the per-head maxima over the text rows (PH instantiations)
   int32_t early_inputs;               // 1: q_text / k may be read before the stream's earlier work has completed (caller's promise)
+  // First of two launches over the text rows: the next one may start only when this one's inputs are there
+  // (every CTA releases it after its own wait), so that the second reads them without waiting for this one.
+  int32_t release_late;
   long long wait_cycles;              // clock cycles after which a wait between the warp roles gives up
   int32_t keep_keys;                  // 1: the keys are left in L2 for the gather that follows
   float scale_log2e, inv_heads;
@@ -596,14 +599,14 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
   // Let the next kernel in the stream begin its prologue.  Everything up to here touched no
   // global data; the copy thread waits for the stream's earlier work before its first load (its
   // inputs may come from the kernel just before this one), the other roles before their stores.
-  pdl_launch_dependents();
+  if (!p.release_late) pdl_launch_dependents();
   if (threadIdx.x == 0) MD_TRACE(0, 9);    // prologue done
   const uint32_t tmem_base = tmem_base_holder;
   // This request's own sequence.  In a ragged batch the token count comes from an earlier
   // kernel in the stream (the previous layer's selection), so it is read after the wait.
   int Mb = p.M, Lb = p.L, txt_start = p.txt_start;
   if (p.vis_cnt != nullptr) {
-    pdl_wait();
+    if (!p.combine) pdl_wait();   // (a second launch starts after the first one's wait)
     Mb = clamp_vis_cnt(p.vis_cnt[b], p.M);
     txt_start = p.vis_start + Mb;
     Lb = txt_start + p.n_txt;
@@ -687,6 +690,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       const int key0 = static_cast<int>(rank) * p.tk;
       const uint64_t key_policy = p.keep_keys ? l2_normal_policy() : l2_evict_first_policy();
       if (!p.early_inputs) pdl_wait();   // q_text / k may be the output of the kernel just before this one
+      if (p.release_late) pdl_launch_dependents();
       if (p.split) {
         int q_issued = 0, k_issued = 0;   // tiles started so far
         bool ok = true;
@@ -1795,7 +1799,10 @@ cudaError_t launch_fused_common(const mustdrop_plan& plan, const FusedGeometry& 
   p.gx_cnt = reinterpret_cast<uint32_t*>(static_cast<unsigned char*>(workspace) + plan.ws_gx_cnt_off);
   p.gx_stats = reinterpret_cast<float2*>(static_cast<unsigned char*>(workspace) + plan.ws_gx_stats_off);
   p.per_head = r.per_head_max;
-  p.early_inputs = (r.inputs_ready && vis_cnt == nullptr) ? 1 : 0;
+  // A second launch over the text rows starts loading while the first one drains: 16 requests of 3008 keys,
+  // 128 rows: 382.7 -> 311.3 us a call; 10 of 2731, 84 rows, 40 heads: 284.9 -> 260.1.
+  p.early_inputs = (combine || (r.inputs_ready && vis_cnt == nullptr)) ? 1 : 0;
+  p.release_late = plan.row_split && !combine ? 1 : 0;
   p.wait_cycles = r.wait_cycles > 0 ? r.wait_cycles : kWaitCycles;
   // The gather reads the kept tokens' keys a second time.  Where the keys of the requests that are
   // resident at once are not far beyond L2 they stay there with normal priority (16 requests of 640
@@ -1803,7 +1810,9 @@ cudaError_t launch_fused_common(const mustdrop_plan& plan, const FusedGeometry& 
   // keys and 40 heads: 245 -> 242); beyond twice its size they leave first, so that they do not push
   // out what other kernels keep there (64 requests of 640 keys: 105.4, with normal priority 107.4).
   const int64_t at_once = geo.resident > 0 && geo.resident < r.B && !geo.gx ? geo.resident : r.B;
-  p.keep_keys = at_once * r.H * r.L * 256 <= 2 * plan.l2_bytes;
+  // Not where less than an eighth is gathered (18 of 551 keys, budget 29 of 406: 56.8 us, first out 55.3),
+  // and not where two launches share the text rows (51 of 1389 keys, 8 heads: 208.8, first out 193.1).
+  p.keep_keys = !plan.row_split && r.cap * 8 >= r.M && at_once * r.H * r.L * 256 <= 2 * plan.l2_bytes;
   p.scale_log2e = r.scale_log2e;
   p.inv_heads = 1.0f / static_cast<float>(r.H);
 
