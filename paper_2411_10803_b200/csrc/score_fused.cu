@@ -632,7 +632,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       if (threadIdx.x == 0) {
         if (FILTER && *abort_flag == 0) {
           uint32_t* const stored = p.gx_cnt + static_cast<size_t>(gridDim.x / p.cluster) * p.H + b;
-          add_release_gpu(stored);   // (the CTA's scores: ordered before it by the barrier above)
+          add_release_gpu(stored);   // (the CTA's scores: ordered before it by the barrier that ends finish())
           (void)count_wait(stored, static_cast<uint32_t>(p.cluster), abort_flag, wait_limit);
         }
         if (*abort_flag != 0) {
@@ -1188,6 +1188,11 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             }
           }
         }
+      }
+      // Grid plans: the scores of all eight warps are stored before one thread announces them to the
+      // request's other CTAs (common_exit): the release orders what this barrier has gathered.
+      if constexpr (FILTER) {
+        if (p.gx) SelectSyncGroup::sync();
       }
       if (threadIdx.x == 0) MD_TRACE(0, 10);   // scores stored
     };

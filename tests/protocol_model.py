@@ -24,6 +24,9 @@ global memory and adds one to the head's counter; a fetch role waits until the c
 CTA, copies the head's pairs into a statistics slot and completes the slot's barrier - it learns
 that a slot is free from the buffer barrier (``tempty``) of the head that used it, by parity.
 
+``Meeting`` models the end of the score part in the one-launch filter: who has stored its scores - and,
+with head groups, staged its head sums - before whom they are read.
+
 The model checks what the kernel relies on: no statistics slot is written before its previous
 content has been read, no buffer is refilled before it was released, every head is processed
 exactly once per CTA, and a missing arrive ends in a clean time-out everywhere instead of a hang.
@@ -305,3 +308,69 @@ class Cluster:
                 self.cluster_abort = True
         self.kept_cnt = -1 if self.cluster_abort else self.geo["H"]
         return True
+
+
+class Meeting:
+    """The end of the score part of one request in the one-launch filter: from the head sums of its CTAs
+    to the selection, which every CTA runs on ALL of the request's scores.  A thread stands for a warp of
+    the reducing (exp) warps; ``slow`` maps (CTA, warp) to a delay before that warp's stores.
+
+    Grid plans (``groups`` = 1): a warp stores its share of the CTA's scores to global memory; the CTA's
+    warps meet; warp 0 adds one to the request's counter and waits until it shows every CTA; the CTA's
+    warps meet again and read all scores.  ``gathered=False`` leaves out the first of the two meetings.
+
+    Head groups (a cluster of groups x C CTAs): the CTAs stage their head sums, meet, add the groups'
+    sums for their part of the keys, push the scores into every CTA and meet again.  ``staged=False``
+    leaves out the first of these two meetings."""
+
+    def __init__(self, C=3, groups=1, warps=4, grid=True, slow=None, gathered=True, staged=True, limit=5.0):
+        self.C, self.groups, self.warps, self.grid = C, groups, warps, grid
+        self.n = C * groups
+        self.slow, self.gathered, self.staged, self.limit = slow or {}, gathered, staged, limit
+        self.cta = [threading.Barrier(warps) for _ in range(self.n)]
+        self.cluster = threading.Barrier(self.n * warps)
+        # scores[copy][CTA that reduced them][warp]: one copy in global memory, or one per CTA
+        self.scores = [[[False] * warps for _ in range(self.n)] for _ in range(1 if grid else self.n)]
+        self.sums = [[False] * warps for _ in range(self.n)]
+        self.stored, self.lock = 0, threading.Lock()
+        self.errors = []
+
+    def _warp(self, cta, w):
+        if not self.grid:
+            time.sleep(self.slow.get((cta, w), 0.0))
+            self.sums[cta][w] = True
+            if self.staged:
+                self.cluster.wait(self.limit)
+            same_keys = range(cta % self.C, self.n, self.C)      # the CTAs of all groups that hold these keys
+            if not all(self.sums[c][x] for c in same_keys for x in range(self.warps)):
+                self.errors.append("CTA %d warp %d adds head sums that are not staged" % (cta, w))
+            for copy in self.scores:
+                copy[cta][w] = True
+            self.cluster.wait(self.limit)
+        else:
+            time.sleep(self.slow.get((cta, w), 0.0))
+            self.scores[0][cta][w] = True
+            if self.gathered:
+                self.cta[cta].wait(self.limit)
+            if w == 0:
+                with self.lock:
+                    self.stored += 1
+                t0 = time.monotonic()
+                while self.stored < self.n and time.monotonic() - t0 < self.limit:
+                    time.sleep(0.0002)
+                # what the first warp could read as soon as the counter lets it through
+                self._check(cta)
+            self.cta[cta].wait(self.limit)
+        self._check(cta)
+
+    def _check(self, cta):
+        if not all(all(ws) for ws in self.scores[0 if self.grid else cta]):
+            self.errors.append("CTA %d selects from scores that are not stored" % cta)
+
+    def run(self):
+        threads = [threading.Thread(target=self._warp, args=(c, w), daemon=True) for c in range(self.n) for w in range(self.warps)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join(2 * self.limit)
+        return not any(t.is_alive() for t in threads)

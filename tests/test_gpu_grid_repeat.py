@@ -44,6 +44,47 @@ def test_many_grid_calls_in_a_row(n_txt, ctas):
         y.close()
 
 
+@pytest.mark.parametrize("n_vis,n_txt,ctas", [(1631, 40, 6), (2048, 96, 16)])
+def test_every_call_of_a_grid_plan_selects_from_its_own_scores(n_vis, n_txt, ctas):
+    # Inputs change with every call and every output holds NaN bits before it, so that a score read before
+    # it is stored shows: each CTA of a request selects for itself, and copies rows of its own list.  The
+    # list must be the one the stand-alone selection makes of the call's own scores, the rows those of the
+    # list, the scores those of a cluster plan (other orders of fp32 sums: 1e-5).
+    w = small(batch=9, n_vis=n_vis, n_txt=n_txt, n_heads=2, hidden=256, key_cnt=20, budget=200, vis_start=21)
+    f = md.Filter(cfg(w, debug_score_variant=md.MUSTDROP_DEBUG_VARIANT_GRID, debug_cluster=ctas))
+    assert "grid plan" in f.description
+    select = md.Filter(cfg(w))
+    x = [inputs(w, 40 + n) for n in range(5)]
+    want = []
+    for y in x:
+        r = md.Filter(cfg(w, debug_score_variant=md.MUSTDROP_DEBUG_VARIANT_TWO_PASS))
+        r.score(y[0], y[1])
+        want.append((r.g.clone(), r.i.clone()))
+        r.close()
+    outs = (f.g, f.i, f.kept_idx, f.kept_cnt, f.hidden_out, f.k_out, f.v_out)
+    rows = torch.arange(w.batch, device="cuda")[:, None]
+    wrong = torch.zeros(4, dtype=torch.int64, device="cuda")
+    for n in range(300):
+        q, k, v, hid, key_idx, key_cnt = x[n % 5]
+        for t in outs:
+            t.view(torch.uint8).fill_(0xFF)
+        f.filter(q, k, v, hid, key_idx, key_cnt)
+        select.g.copy_(f.g)
+        select.i.copy_(f.i)
+        select.select(key_idx, key_cnt)
+        at = w.vis_start + f.kept_idx.long().clamp(0, w.n_vis - 1)
+        for e, (a, b) in enumerate(zip((f.g, f.i), want[n % 5])):
+            wrong[e] += (~((a - b).abs() <= 1e-5 * b.abs() + 1e-12)).sum()
+        wrong[2] += (f.kept_idx != select.kept_idx).sum() + (f.kept_cnt != select.kept_cnt).sum()
+        wrong[3] += (f.hidden_out.view(torch.int16) != hid[rows, at].view(torch.int16)).sum()
+        for src, out in ((k, f.k_out), (v, f.v_out)):
+            wrong[3] += (out.transpose(1, 2).view(torch.int16) != src.transpose(1, 2)[rows, at].view(torch.int16)).sum()
+    assert wrong.tolist() == [0, 0, 0, 0]
+    assert f.device_status() == (0, 0)
+    f.close()
+    select.close()
+
+
 def test_score_and_filter_calls_share_a_grid_plan_s_workspace():
     w = small(batch=3, n_vis=700, n_txt=30, n_heads=3, hidden=384, key_cnt=5, budget=90, vis_start=0)
     force = dict(debug_score_variant=md.MUSTDROP_DEBUG_VARIANT_GRID, debug_cluster=6)

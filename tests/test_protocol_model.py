@@ -3,7 +3,7 @@ cluster): it completes for the geometries the planner produces, its slot and buf
 exactly enough, and a role that skips an arrive ends in a time-out in every CTA - no hang."""
 import pytest
 
-from protocol_model import OK, TIMEOUT, Cluster
+from protocol_model import OK, TIMEOUT, Cluster, Meeting
 
 GEOMETRIES = [
     dict(C=1, n_q=2, n_buf=3),
@@ -121,3 +121,26 @@ def test_grid_protocol_times_out_everywhere_after_a_skipped_signal(fault):
     assert cl.errors == []
     assert all(c.status == TIMEOUT for c in cl.ctas)
     assert cl.kept_cnt == -1
+
+
+# ---- the end of the score part: every score stored before any CTA of the request selects -----------
+
+MEETINGS = [dict(C=3), dict(C=16), dict(C=2, groups=4, grid=False), dict(C=4, groups=1, grid=False)]
+
+
+@pytest.mark.parametrize("slow", [None, (0, 1), (1, 0), (1, 3)])
+@pytest.mark.parametrize("geo", MEETINGS, ids=lambda g: "_".join("%s%d" % x for x in g.items()))
+def test_every_score_is_stored_before_any_cta_selects(geo, slow):
+    m = Meeting(slow={slow: 0.02} if slow else None, **geo)
+    assert m.run() and m.errors == []
+
+
+def test_scores_announced_by_one_warp_without_a_meeting_are_caught_by_the_model():
+    # one warp counts its CTA as done while another warp of it has not stored yet: its peers select too early
+    m = Meeting(C=3, slow={(1, 2): 0.05}, gathered=False)
+    assert m.run() and m.errors
+
+
+def test_head_sums_read_before_they_are_staged_are_caught_by_the_model():
+    m = Meeting(C=2, groups=2, grid=False, slow={(3, 1): 0.05}, staged=False)
+    assert m.run() and m.errors
