@@ -893,6 +893,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
           }
           if (!ok) break;
+          __syncwarp();   // what lane i has acquired (the pairs behind head h + i's counter) is ordered before every lane's copies
         }
         const unsigned char* const src = reinterpret_cast<const unsigned char*>(p.gx_stats + bh * slot_pairs);
         const uint32_t dst = smem_u32(stats + static_cast<size_t>(slot) * slot_pairs);

@@ -22,7 +22,9 @@ Grid plans (``grid=True``): the CTAs of the request are no cluster; the exp role
 the CTA's own memory and arrives on ``gsent``; a publishing role stores the pair to (modelled)
 global memory and adds one to the head's counter; a fetch role waits until the counter shows every
 CTA, copies the head's pairs into a statistics slot and completes the slot's barrier - it learns
-that a slot is free from the buffer barrier (``tempty``) of the head that used it, by parity.
+that a slot is free from the buffer barrier (``tempty``) of the head that used it, by parity.  The
+fetch role is a warp: one lane acquires each counter, all lanes copy.  ``lanes_meet=False`` leaves out
+the warp barrier between the two, without which the other lanes' copies are not ordered behind it.
 
 ``Meeting`` models the end of the score part in the one-launch filter: who has stored its scores - and,
 with head groups, staged its head sums - before whom they are read.
@@ -36,6 +38,7 @@ import time
 
 OK, TIMEOUT = 0, 6          # MUSTDROP_OK, MUSTDROP_ERR_TIMEOUT
 N_GROUPS = 2                # groups of exp warps per CTA; they alternate heads
+LANES = 4                   # lanes of a (short) warp
 
 
 class ProtocolError(AssertionError):
@@ -111,7 +114,7 @@ class Cluster:
     arrive ("full", "tfull", "eready", "tempty", "empty") or one statistics store ("stats")."""
 
     def __init__(self, C=2, H=12, n_q=2, n_buf=3, n_slot=None, tight=0, limit=0.25, fault=None, jitter=None,
-                 grid=False, handover="auto"):
+                 grid=False, handover="auto", lanes_meet=True):
         n_slot = (min(n_buf, 4) if grid else 2 * n_buf) if n_slot is None else n_slot
         self.grid = grid
         self.g_lock = threading.Lock()
@@ -120,7 +123,7 @@ class Cluster:
         self.geo = dict(C=C, H=H, n_q=n_q, n_buf=n_buf, n_slot=n_slot, tight=tight)
         # "auto": what the kernel does (at once); "late": one head of the group later
         self.eager = handover == "auto"
-        self.limit, self.fault, self.jitter = limit, fault, jitter or {}
+        self.limit, self.fault, self.jitter, self.lanes_meet = limit, fault, jitter or {}, lanes_meet
         self.ctas = [Cta(self, r, self.geo) for r in range(C)]
         self.errors = []
         self.cluster_abort = False
@@ -256,6 +259,8 @@ class Cluster:
 
     def fetch(self, c):
         g = self.geo
+        ready = 0                                   # heads below are known to be published
+        sees = [set() for _ in range(LANES)]        # heads whose pairs a lane is ordered behind
         for h in range(g["H"]):
             slot = h % g["n_slot"]
             self._pause(c.rank, "fetch_late")       # (a fetch role that gets to its next head late)
@@ -264,15 +269,25 @@ class Cluster:
                 if not c.wait(c.tempty[u % g["n_buf"]], (u // g["n_buf"]) & 1, self.limit):
                     return
             t0 = time.monotonic()
-            while True:
-                with self.g_lock:
-                    if self.g_cnt[h] >= g["C"]:
-                        break
+            while h >= ready:
+                with self.g_lock:                   # lane i looks at head h + i; the run of complete heads is taken
+                    for lane in range(LANES):
+                        if h + lane >= g["H"] or self.g_cnt[h + lane] < g["C"]:
+                            break
+                        sees[lane].add(h + lane)
+                        ready = h + lane + 1
+                if ready > h:
+                    if self.lanes_meet:
+                        every = set().union(*sees)
+                        sees = [set(every) for _ in range(LANES)]
+                    break
                 if c.abort or time.monotonic() - t0 > self.limit:
                     c.abort = True
                     return
                 time.sleep(0.0002)
             self._pause(c.rank, "fetch")
+            if not all(h in s for s in sees):
+                raise ProtocolError("a lane copies the pairs of head %d unordered behind its counter" % h)
             with c.guard:
                 if c.stats[slot] != [None] * g["C"]:
                     raise ProtocolError("slot %d of CTA %d refilled for head %d before heads %s were read"

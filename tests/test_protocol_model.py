@@ -123,6 +123,12 @@ def test_grid_protocol_times_out_everywhere_after_a_skipped_signal(fault):
     assert cl.kept_cnt == -1
 
 
+def test_copies_of_lanes_that_did_not_acquire_the_counter_are_caught_by_the_model():
+    # lane i of the fetch warp acquires the counter of head h + i, every lane copies every head's pairs
+    cl = Cluster(C=3, H=12, n_q=2, n_buf=3, limit=0.3, grid=True, lanes_meet=False)
+    assert cl.run(join_limit=10.0) and cl.errors and cl.kept_cnt == -1
+
+
 # ---- the end of the score part: every score stored before any CTA of the request selects -----------
 
 MEETINGS = [dict(C=3), dict(C=16), dict(C=2, groups=4, grid=False), dict(C=4, groups=1, grid=False)]
