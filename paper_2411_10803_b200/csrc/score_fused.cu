@@ -658,11 +658,12 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
   // The way out after a give-up, taken by every thread of every CTA of the cluster.  A peer's
   // asynchronous statistics stores may still be on their way into this CTA's shared memory: give
   // them time to land and meet once more, so that no CTA's shared memory goes away under them.
+  // A grid completes only behind the stream's earlier work: the next kernel's wait covers this grid, and
+  // through it what came before.  Where the copy thread starts without waiting (early_inputs) a CTA that
+  // gives up has not waited anywhere yet.
   auto leave_after_give_up = [&](int32_t* kept_cnt) {
-    if (kept_cnt != nullptr && (req_rank == 0 || p.gx) && threadIdx.x == 0) {
-      pdl_wait();
-      kept_cnt[b] = -1;   // this request's result is invalid
-    }
+    pdl_wait();
+    if (kept_cnt != nullptr && (req_rank == 0 || p.gx) && threadIdx.x == 0) kept_cnt[b] = -1;   // this request's result is invalid
     const long long t0 = clock64();
     while (clock64() - t0 < 40000) {}
     __syncwarp();

@@ -269,6 +269,43 @@ def test_a_wait_that_runs_out_is_reported_and_the_next_call_is_unaffected(cluste
     good.close()
 
 
+@pytest.mark.parametrize("path", ["filter", "score"])
+def test_a_call_that_gives_up_still_ends_behind_the_work_before_it(path):
+    """A call whose inputs are ready starts without waiting for the stream; when it gives up at once it
+    must not complete before the (long) kernel ahead of it: the selection behind it reads that one's scores."""
+    w = small(batch=1, n_vis=250, n_txt=20, n_heads=512, hidden=256, key_cnt=0, budget=100, vis_start=0)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    q = torch.randn((1, w.n_heads, w.n_txt, 128), generator=gen, device="cuda").to(torch.bfloat16)
+    k = torch.randn((1, w.n_heads, w.seq_len, 128), generator=gen, device="cuda").to(torch.bfloat16)
+    # one CTA with 512 heads in sequence, which lets the kernels behind it start after its prologue
+    ahead = md.Filter(cfg(w, debug_score_variant=md.MUSTDROP_DEBUG_VARIANT_FUSED, debug_cluster=1))
+    ahead.score(q, k)
+    ahead.select()
+    torch.cuda.synchronize()
+    want = ahead.kept_idx.clone()
+    small_w = small(batch=2, n_vis=200, n_txt=20, n_heads=3, hidden=384, key_cnt=0, budget=20, vis_start=0)
+    d = synth.make_batch(small_w)
+    x = [to_dev_bf16(d[n]) for n in ("q_text", "k", "v", "hidden")]
+    bad = md.Filter(cfg(small_w, flags=md.MUSTDROP_FLAG_INPUTS_READY, debug_wait_cycles=64))
+    for _ in range(5):
+        ahead.g.copy_(torch.rand_like(ahead.g))       # scores of another order, should they be read too early
+        ahead.i.zero_()
+        ahead.kept_idx.fill_(-1)
+        torch.cuda.synchronize()
+        ahead.score(q, k)
+        if path == "filter":
+            bad.filter(*x)
+        else:
+            bad.score(x[0], x[1])
+        ahead.select()
+        torch.cuda.synchronize()
+        assert torch.equal(ahead.kept_idx, want)
+        assert bad.device_status()[0] == md.MUSTDROP_ERR_TIMEOUT
+        bad.workspace.zero_()
+    ahead.close()
+    bad.close()
+
+
 def test_compact_skips_a_request_marked_invalid():
     """kept_cnt = -1 (a request whose selection failed) and a count beyond the capacity: nothing is
     written for the first, the second is clamped; both are recorded; nothing lands outside the outputs."""
