@@ -1865,23 +1865,20 @@ bool plan_filter_single(const Resolved& r, const FusedGeometry& geo, FilterGeome
   const size_t limit = 227 * 1024 - 4096;                          // dynamic shared memory a CTA may ask for
   const size_t fixed = 1024 + kKeptListBytes;
   // The scores meet in every CTA while peers may still be adding their last head or reading this
-  // CTA's staged head sums: behind those sums inside the staging area, which is idle by then, or
-  // behind everything.
+  // CTA's staged head sums: behind those sums inside the staging area, which is idle by then.  (Every
+  // geometry of the planners has that room: tests/test_abi_host.py.)
   const size_t nrows = 128 / geo.halves, val = 8 * static_cast<size_t>(select_pad(r.M));
   const size_t stage = (nrows + geo.tk) * 256;
   const size_t staging = geo.split ? geo.n_q * nrows * 256 + static_cast<size_t>(geo.n_k) * geo.cpl * 256 : geo.n_q * stage;
   const size_t sums = ((nrows * (geo.tk | 1) * 4 + 15) & ~static_cast<size_t>(15)) + 8 * static_cast<size_t>(geo.tk) * 8;
-  size_t val_off = (sums + 15) & ~static_cast<size_t>(15), least = geo.smem_bytes;
+  size_t val_off = (sums + 15) & ~static_cast<size_t>(15);
   // (the selection's own scratch lies at the start of the staging area, behind the kept list)
   if (val_off < kKeptListBytes + sizeof(SelectScratch)) val_off = kKeptListBytes + sizeof(SelectScratch);
-  if (val_off + val > staging) {
-    val_off = geo.smem_bytes - 1024 > val_off ? geo.smem_bytes - 1024 : val_off;
-    least = 1024 + val_off + val;
-  }
+  if (val_off + val > staging) return false;
   size_t want = fixed + kMaxGatherSlots * slot;
-  if (want < least) want = least;
+  if (want < geo.smem_bytes) want = geo.smem_bytes;
   if (want > limit) want = limit;
-  if (want < least) return false;
+  if (want < geo.smem_bytes) return false;
   out->val_off = static_cast<int32_t>(val_off);
   int n_slot = static_cast<int>((want - fixed) / slot);
   if (n_slot > kMaxGatherSlots) n_slot = kMaxGatherSlots;

@@ -200,3 +200,27 @@ def test_filter_layer_rejects_bad_arguments_without_a_gpu():
     import pytest as _pytest
     with _pytest.raises(TypeError):
         md.mustdrop_filter_layer(0, 256, 0, no_such_field=1)
+
+
+def test_every_fused_geometry_has_room_for_the_selection_s_scores():
+    """The one-launch filter keeps a request's scores behind the staged head sums.  No geometry of the fused
+    kernel - any number of CTAs per request, clusters or not, 64 or 128 text rows on the lanes, both readings
+    of Eq. 10 - leaves less room than that takes: with rows that fit the gather's ring there is no plan of
+    separate launches."""
+    seen = set()
+    for variant, most in ((md.MUSTDROP_DEBUG_VARIANT_FUSED, 16), (md.MUSTDROP_DEBUG_VARIANT_ROW_SPLIT, 16),
+                          (md.MUSTDROP_DEBUG_VARIANT_GRID, 32)):
+        for ctas in range(1, most + 1):
+            for n_txt in (1, 64, 65, 128):
+                for n_vis in (1, 40, 255, 256, 257, 700, 1024, 1025, 2000, 3000, 3600, 4095, 4096):
+                    for flags in (0, md.MUSTDROP_FLAG_PER_HEAD_MAX):
+                        c = md.Config(batch=1, n_heads=4, hidden=512, seq_len=n_vis + n_txt, vis_start=0, n_vis=n_vis, txt_start=n_vis,
+                                      n_txt=n_txt, budget=n_vis, flags=flags, debug_score_variant=variant, debug_cluster=ctas)
+                        st, plan, _ = md.mustdrop_filter_plan(c)
+                        assert st == md.MUSTDROP_OK
+                        text, launches = md.mustdrop_plan_describe(plan), md.mustdrop_plan_filter_launches(plan)
+                        md.mustdrop_plan_destroy(plan)
+                        if "fused" in text:
+                            seen.add((variant, "two launches" in text, "grid" in text))
+                            assert launches == (2 if "two launches" in text else 1), (text, n_vis, n_txt, flags)
+    assert len(seen) >= 3
