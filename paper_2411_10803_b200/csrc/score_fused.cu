@@ -1276,9 +1276,11 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         // Statistics of this row over the whole key range, relative to this CTA's own stabiliser:
         // f = 1 / sum over CTAs of l_c 2^(m_c - m_own).  Independent terms, four loads in flight: the
         // loop is on every head's serial path (as a maximum first and a sum over the CTAs second it
-        // took 0.5 us with 2 CTAs and 0.8 us with 16).  A sum that overflows means that this CTA's
-        // share is below 2^-127: f = 0.  Grid plans: one merged pair per CTA in the slot; this CTA's own
-        // stabilisers are still in its shared memory (until the buffer is released below).
+        // took 0.5 us with 2 CTAs and 0.8 us with 16).  A pair's sum is below 2^45 (22 chunks of less than
+        // kSumLimit each): a total that overflows 2^128 means that this CTA's share of the row is below
+        // 2^-83 (f = 0), and a term that ex2 flushes to zero is below 2^-81 of it.  Grid plans: one pair per
+        // row and CTA in the slot as well; this CTA's own stabilisers are still in its shared memory (until the
+        // buffer is released below).
         const float2* const srow = stats + slot * slot_pairs + row;
         const float own = p.gx ? own_pairs[buf * NROWS + row].x : srow[rank * NROWS].x;
         float l0 = 0.0f, l1 = 0.0f;

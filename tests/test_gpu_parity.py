@@ -177,6 +177,35 @@ def test_score_with_logits_that_grow_along_the_keys(n_txt, variant):
     f.close()
 
 
+@pytest.mark.parametrize("above", [20, 41, 62, 85, 100, 120])
+@pytest.mark.parametrize("variant", ["fused:2", "grid:2"], indirect=True)
+def test_score_with_stabilisers_of_two_ctas_far_apart(variant, above):
+    """The first CTA's sum grows to 2^43 over its stabiliser (the later chunks stay just under the limit of
+    2^40 that sends a warp down the careful path); the other CTA's stabiliser lies `above` powers of two
+    higher, so that the merged sum runs up to and over the range of fp32."""
+    w = small(batch=1, n_vis=214, n_txt=70, n_heads=2, hidden=256, n_salient=0)       # 2 x 144 keys, one tile each
+    per_z = np.log2(np.e) * 16.0 / np.sqrt(128.0)                                     # powers of two per unit of a key's entry
+    q = np.zeros((1, 2, w.n_txt, 128), np.float32)
+    q[..., 0] = 16.0
+    z = np.zeros(w.seq_len, np.float32)
+    z[16:144] = 35.5                                                                  # 16 columns: below 2^39.5 + 0.3 a chunk
+    z[144:214] = above
+    z[160:214] += 5.0
+    k = np.zeros((1, 2, w.seq_len, 128), np.float32)
+    k[..., 0] = z / per_z
+    qb, kb = synth.f32_to_bf16_bits(q), synth.f32_to_bf16_bits(k)
+    G, I = oracle.score(qb, kb, w.vis_start, w.n_vis, w.txt_start)
+    f = md.Filter(cfg(w))
+    check_variant(f, variant)
+    assert "144 keys per CTA" in f.description
+    g, i = f.score(to_dev_bf16(qb), to_dev_bf16(kb))
+    torch.cuda.synchronize()
+    assert f.device_status() == (0, 0)
+    assert_scores_close(g.cpu().numpy(), G, "G")
+    assert_scores_close(i.cpu().numpy(), I, "I")
+    f.close()
+
+
 # ---- select ----------------------------------------------------------------------------------
 
 def _random_scores(seed, B, M, N=9):
