@@ -82,7 +82,8 @@ typedef enum {
  * leaves open: i_out[b][j] = mean over heads of ( max over text tokens of p^h[i][vis_start + j] )
  * instead of the maximum of the head-mean attention.  g_out (Eq. 8) is the same under both.
  * (On the fused kernel each head's maximum is rounded to 11 significant bits before the mean over
- * heads is taken in fp32: at most 5e-4 relative, inside the 2e-3 the scores are held to.)
+ * heads is taken in fp32: at most 5e-4 relative, inside the 2e-3 the scores are held to.  Small calls, which
+ * the two-pass kernel or a grid plan with fp32 maxima answers, are not rounded.)
  */
 #define MUSTDROP_FLAG_PER_HEAD_MAX 2
 

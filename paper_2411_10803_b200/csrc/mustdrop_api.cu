@@ -159,7 +159,6 @@ mustdrop_status_t mustdrop_filter_plan(const mustdrop_config_t* c, mustdrop_plan
     const bool allow_fused = c->debug_score_variant != MUSTDROP_DEBUG_VARIANT_TWO_PASS;
     const bool force_split = c->debug_score_variant == MUSTDROP_DEBUG_VARIANT_ROW_SPLIT;
     const bool force_grid = c->debug_score_variant == MUSTDROP_DEBUG_VARIANT_GRID;
-    const double k_mb = 256.0e-6 * r.B * r.H * r.L;
     // the two-pass kernel's measured rate, less where heads x requests leave SMs without a CTA (one request
     // of 8 heads, 4124 keys and 78 text rows: 175 us, 59 as a grid plan; the factor is bounded because a
     // handful of heads is also where the grid plan's own start counts), and its second pass's walk over the
@@ -167,7 +166,7 @@ mustdrop_status_t mustdrop_filter_plan(const mustdrop_config_t* c, mustdrop_plan
     double idle = static_cast<double>(p->sm_count) / (r.B * r.H);
     idle = idle < 1.0 ? 1.0 : (idle > 2.0 ? 2.0 : idle);
     const double two_pass_us =
-        k_mb * (0.6 + 0.7 * r.N / 128.0) * idle + 3.0 * r.H + mustdrop::gather_us(r, p->sm_count);
+        mustdrop::two_pass_keys_us(r) * idle + 3.0 * r.H + mustdrop::gather_us(r, p->sm_count);
     double chosen_us = two_pass_us;
     p->row_split = 0;
     if (allow_fused && !force_split && !force_grid && plan_score_fused(r, p->sm_count, forced_cluster, &p->fused)) {

@@ -37,6 +37,7 @@ struct FusedGeometry {
   int32_t row0, n_rows;   // the text rows this geometry's launch covers
   int32_t gx;         // 1: grid plan - the request's CTAs are ordinary CTAs of the grid (cluster = their number) and
                       //    exchange their statistics through global memory
+  int32_t exact_max;  // grid plans: the per-head maxima of Eq. 10 are taken in fp32
   int32_t resident;   // clusters the device can hold at once (0: not asked)
   float est_us;       // the planner's estimate of the score time
   size_t smem_bytes;  // dynamic shared memory
@@ -112,7 +113,8 @@ cudaError_t launch_score_two_pass(const mustdrop_plan& p, const void* q_text, co
                                   const int32_t* vis_cnt = nullptr);
 bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, FusedGeometry* out, int row0 = 0,
                       int n_rows = 0);
-double gather_us(const Resolved& r, double ctas);   // the planner's estimate of the gather
+double gather_us(const Resolved& r, double ctas);   // the planner's estimates of the gather ...
+double two_pass_keys_us(const Resolved& r);         // ... and of the two-pass kernel on a full GPU
 // Grid plan of the same kernel (all CTAs of the batch resident at once, statistics through global
 // memory); false when the batch leaves fewer than two CTAs per request or the shape does not fit.
 bool plan_score_grid(const Resolved& r, int sm_count, int forced_ctas, FusedGeometry* out);

@@ -42,7 +42,8 @@ namespace {
 
 constexpr int kExpWarps = 8;                // warps 0-7: 4 TMEM lane quadrants x 2 column groups
 constexpr int kColGroups = 2;
-constexpr float kPhScale = 16384.0f;        // per-head maxima travel as fp16 times 2^14
+constexpr int kPhPairs = 1, kPhExact = 2;    // per-head maxima (Eq. 10): how they travel between the lanes
+constexpr float kPhScale = 16384.0f;        // ... as fp16 pairs: times 2^14
 constexpr int kAddWarps = 4;                // warps 8-11: one per lane quadrant, all columns
 constexpr int kExpThreads = kExpWarps * 32;
 constexpr int kAddThreads = kAddWarps * 32;
@@ -515,7 +516,8 @@ __device__ __forceinline__ void filter_gather(const FilterTail& ft, const Gather
 // FILTER: after the scores, the cluster also selects the request's tokens and gathers them.
 // PH: the other reading of Eq. 10 - per head the column maximum over the text rows, then the head
 //     mean - computed by the add warps from the same normalised probabilities (G is unchanged).
-template <int HALVES, int ACH, bool FILTER, bool PH>
+//     kPhPairs: the maxima travel as fp16 pairs; kPhExact: in fp32 (some grid plans).
+template <int HALVES, int ACH, bool FILTER, int PH>
 __global__ void __launch_bounds__(kThreads, 1)
 score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                    const FusedParams p, const __grid_constant__ GatherMaps gm, const __grid_constant__ FilterTail ft) {
@@ -1170,7 +1172,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           mx = p.groups == 1 ? ph_stage[c] : 0.0f;
           for (int gr = 0; gr < p.groups && p.groups > 1; ++gr)
             mx += ld_cluster_f32(map_to_cta(smem_u32(ph_stage + c), gr * p.cluster + rank));
-          mx *= 1.0f / kPhScale;
+          if (PH == kPhPairs) mx *= 1.0f / kPhScale;
         }
         const bool present = j < Mb;    // beyond the request's own tokens: zeros
         float gv = present ? sum * p.inv_heads : 0.0f, iv = present ? mx * p.inv_heads : 0.0f;
@@ -1315,14 +1317,39 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             for (int j = 0; j < kChunk; j += 2)
               acc[c0 + 1][j >> 1] = fma2(pack2(e[1][j], e[1][j + 1]), f_2, acc[c0 + 1][j >> 1]);
           }
-          if constexpr (PH) {
+          if constexpr (PH == kPhExact) {
             // Column maxima over this warp's text rows (the lanes): recursive halving - in each of
             // four steps a lane keeps half of its columns and takes its partner's maxima for them,
-            // so that lane j of a 16-lane group ends up with column j's maximum over the group.  The
-            // probabilities travel as fp16 pairs (two columns per register: half the shuffles,
-            // selects and maxima), scaled by 2^14 so that nothing above 4e-9 is subnormal; rounding
-            // them costs 2^-11 relative, a quarter of the score tolerance.  With 128 text rows the
-            // two 16-lane groups of a warp hold the same columns and are folded first.
+            // so that lane j of a 16-lane group ends up with column j's maximum over the group.  With
+            // 128 text rows the two 16-lane groups of a warp hold the same columns and are folded first.
+            // In fp32 (15 shuffles a chunk, 16 more with 128 rows, instead of 8 and 8): see exact_max.
+            float* const dst = ph_stage + ((h & 1) * kAddWarps + q) * p.tk + half * p.cpl + (lane & 15);
+            const float fx = real_row ? f : 0.0f;
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+              if (c0 + x < ACH && c0 + x < total_chunks) {
+                float v[kChunk];
+#pragma unroll
+                for (int j = 0; j < kChunk; ++j) {
+                  v[j] = e[x][j] * fx;
+                  if (HALVES == 1) v[j] = fmaxf(v[j], __shfl_xor_sync(0xffffffffu, v[j], 16));
+                }
+#pragma unroll
+                for (int step = kChunk / 2; step >= 1; step >>= 1) {
+                  const bool upper = (lane & step) != 0;
+#pragma unroll
+                  for (int i = 0; i < step; ++i) {
+                    const float give = upper ? v[i] : v[i + step], keep = upper ? v[i + step] : v[i];
+                    v[i] = fmaxf(keep, __shfl_xor_sync(0xffffffffu, give, step));
+                  }
+                }
+                if (HALVES == 2 || lane < 16) dst[kChunk * (c0 + x)] = v[0];
+              }
+            }
+          } else if constexpr (PH == kPhPairs) {
+            // The same halving; the probabilities travel as fp16 pairs (two columns per register: half
+            // the shuffles, selects and maxima), scaled by 2^14 so that nothing above 4e-9 is subnormal;
+            // rounding them costs 2^-11 relative, a quarter of the score tolerance.
             float* const dst = ph_stage + ((h & 1) * kAddWarps + q) * p.tk + half * p.cpl + (lane & 15);
             auto hmax2 = [](uint32_t a, uint32_t b2) {
               uint32_t r;
@@ -1492,16 +1519,23 @@ namespace {
 
 using FusedKernel = void (*)(const CUtensorMap, const CUtensorMap, const FusedParams, const GatherMaps, const FilterTail);
 
-template <bool FILTER, bool PH>
+template <bool FILTER, int PH>
 FusedKernel pick_shape(int halves, int ach) {
   if (halves == 2) return ach > 5 ? score_fused_kernel<2, 10, FILTER, PH> : score_fused_kernel<2, 5, FILTER, PH>;
-  if (ach > 10) return score_fused_kernel<1, 11, FILTER, PH>;   // 176 columns per lane (one M=128 tile only)
+  if constexpr (PH != kPhExact) {   // (no grid plan is that wide)
+    if (ach > 10) return score_fused_kernel<1, 11, FILTER, PH>;   // 176 columns per lane (one M=128 tile only)
+  }
   return ach > 5 ? score_fused_kernel<1, 10, FILTER, PH> : score_fused_kernel<1, 5, FILTER, PH>;
 }
 
-FusedKernel pick_kernel(int halves, int ach, bool filter = false, bool per_head = false) {
-  if (filter) return per_head ? pick_shape<true, true>(halves, ach) : pick_shape<true, false>(halves, ach);
-  return per_head ? pick_shape<false, true>(halves, ach) : pick_shape<false, false>(halves, ach);
+template <bool FILTER>
+FusedKernel pick_reading(int halves, int ach, int ph) {
+  if (ph == kPhExact) return pick_shape<FILTER, kPhExact>(halves, ach);
+  return ph == kPhPairs ? pick_shape<FILTER, kPhPairs>(halves, ach) : pick_shape<FILTER, 0>(halves, ach);
+}
+
+FusedKernel pick_kernel(int halves, int ach, bool filter = false, int ph = 0) {
+  return filter ? pick_reading<true>(halves, ach, ph) : pick_reading<false>(halves, ach, ph);
 }
 
 // Clusters of `cluster` CTAs that can be resident at once (GPC boundaries make this less than
@@ -1554,6 +1588,10 @@ double gather_us(const Resolved& r, double ctas) {
   const double bytes = rows * r.B * (2.0 * r.hidden + 2.0 * 256.0 * r.H);
   return std::max(bytes / (33.0e3 * ctas), 2.0 * bytes / 7.0e6);
 }
+
+// Both passes of the two-pass kernel over the keys, on a full GPU (measured: 0.6 us per MB and 0.7 more
+// with 128 text rows).
+double two_pass_keys_us(const Resolved& r) { return 256.0e-6 * r.B * r.H * r.L * (0.6 + 0.7 * r.N / 128.0); }
 
 // Geometry of the fused kernel for a problem; false when the shape is outside what it covers.
 // row0 / n_rows: the text rows the launch covers (n_rows = 0: all of them).
@@ -1744,6 +1782,11 @@ bool plan_score_grid(const Resolved& r, int sm_count, int forced_ctas, FusedGeom
     if (score > best) {
       best = score;
       g.halves = halves; g.cluster = c; g.tk = tk; g.cpl = cpl; g.n_q = n_q; g.n_k = 0; g.split = 0; g.n_buf = n_buf;
+      // Per-head maxima.  Calls of so little work that the two-pass kernel's rate by itself would beat this plan
+      // get them in fp32, as that kernel gives them: a grid plan serves them only because a few heads leave
+      // that kernel's SMs idle, and its speed is no reason to round.  The others' travel as fp16 pairs (in fp32
+      // they take 8 % longer in the mean of 180 grid plans, up to 1.5 x with 160 keys per CTA and 71 heads).
+      g.exact_max = r.per_head_max && 0.9 * two_pass_keys_us(r) <= r.H * t_head + 12.0;
       g.ach = ach; g.groups = 1; g.n_slot = n_slot; g.gx = 1; g.resident = sm_count; g.row0 = 0; g.n_rows = r.N;
       g.est_us = static_cast<float>(r.H * t_head + 12.0 + gather_us(r, c * r.B));   // (+ filling and draining the longer chain)
       g.smem_bytes = smem_bytes;
@@ -1825,7 +1868,7 @@ cudaError_t launch_fused_common(const mustdrop_plan& plan, const FusedGeometry& 
   p.scale_log2e = r.scale_log2e;
   p.inv_heads = 1.0f / static_cast<float>(r.H);
 
-  FusedKernel kernel = pick_kernel(geo.halves, geo.ach, tail != nullptr, r.per_head_max != 0);
+  FusedKernel kernel = pick_kernel(geo.halves, geo.ach, tail != nullptr, r.per_head_max ? (geo.exact_max ? kPhExact : kPhPairs) : 0);
   cudaError_t e = ensure_kernel_attributes(reinterpret_cast<const void*>(kernel), true);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};

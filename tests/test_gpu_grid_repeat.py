@@ -104,3 +104,25 @@ def test_score_and_filter_calls_share_a_grid_plan_s_workspace():
             assert torch.equal(a, b)
         fresh.close()
     f.close()
+
+
+@pytest.mark.parametrize("n_vis,n_txt,ctas", [(300, 21, 2), (333, 64, 7), (500, 65, 6), (700, 128, 6), (1000, 40, 4)])
+def test_per_head_maxima_of_a_small_grid_plan_are_fp32(n_vis, n_txt, ctas):
+    """Grid plans take small calls from the two-pass kernel, whose per-head maxima are fp32.  The two kernels'
+    sums run in other orders: 1e-5 covers both (a maximum rounded to 11 bits is off by up to 5e-4)."""
+    w = small(batch=2, n_vis=n_vis, n_txt=n_txt, n_heads=3, hidden=384, key_cnt=0, budget=50, vis_start=3)
+    per_head = dict(flags=md.MUSTDROP_FLAG_PER_HEAD_MAX)
+    x = inputs(w, 77)
+    got = []
+    for force in (dict(debug_score_variant=md.MUSTDROP_DEBUG_VARIANT_GRID, debug_cluster=ctas),
+                  dict(debug_score_variant=md.MUSTDROP_DEBUG_VARIANT_TWO_PASS)):
+        f = md.Filter(cfg(w, **per_head, **force))
+        assert ("grid plan" in f.description) == (len(got) == 0)
+        f.score(x[0], x[1])
+        scored = f.i.clone()
+        f.filter(*x)
+        torch.cuda.synchronize()
+        assert f.device_status() == (0, 0) and torch.equal(scored, f.i)
+        got.append(scored)
+        f.close()
+    assert ((got[0] - got[1]).abs() <= 1e-5 * got[1].abs()).all()
