@@ -26,6 +26,9 @@ inline bool valid_plan(const mustdrop_plan_t* p) { return p != nullptr && p->mag
 
 inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// Keys that the largest cluster of the fused kernel holds: 16 CTAs of 320, of 176 with more than 64 text rows.
+inline int32_t max_cluster_keys(int32_t n_txt) { return 16 * (n_txt <= 64 ? 320 : 176); }
+
 }  // namespace
 
 namespace mustdrop {
@@ -159,28 +162,35 @@ mustdrop_status_t mustdrop_filter_plan(const mustdrop_config_t* c, mustdrop_plan
     const bool allow_fused = c->debug_score_variant != MUSTDROP_DEBUG_VARIANT_TWO_PASS;
     const bool force_split = c->debug_score_variant == MUSTDROP_DEBUG_VARIANT_ROW_SPLIT;
     const bool force_grid = c->debug_score_variant == MUSTDROP_DEBUG_VARIANT_GRID;
-    // the two-pass kernel's measured rate, less where heads x requests leave SMs without a CTA (one request
-    // of 8 heads, 4124 keys and 78 text rows: 175 us, 59 as a grid plan; the factor is bounded because a
-    // handful of heads is also where the grid plan's own start counts), and its second pass's walk over the
-    // heads
-    double idle = static_cast<double>(p->sm_count) / (r.B * r.H);
-    idle = idle < 1.0 ? 1.0 : (idle > 2.0 ? 2.0 : idle);
-    const double two_pass_us =
-        mustdrop::two_pass_keys_us(r) * idle + 3.0 * r.H + mustdrop::gather_us(r, p->sm_count);
+    // The separate launches around the two-pass kernel: four starts; a CTA's walk over all keys of a head
+    // (which sets the time where few heads x requests leave SMs idle: one request of 3 heads, 1483 keys and
+    // 111 text rows takes 74 us, as a grid plan 28) and, in the second pass, over all heads; what full SMs take
+    // for the keys; selection and copies, which start a CTA a row and tensor.
+    const double rows = 0.6 + 0.7 * r.N / 128.0;
+    const double tiles = std::ceil(r.B * std::ceil(r.M / 64.0) / p->sm_count);
+    const double two_pass_us = 14.0 + 0.42 * mustdrop::two_pass_keys_us(r) + r.L * (0.0133 + 0.0125 * rows) +
+                               r.H * (1.55 + 0.68 * rows * tiles) + 2.9e-3 * r.M + 4.0e-3 * r.B * mustdrop::gathered_rows(r) +
+                               mustdrop::gathered_bytes(r) / 8.8e6;
     double chosen_us = two_pass_us;
     p->row_split = 0;
+    bool tight = false;
     if (allow_fused && !force_split && !force_grid && plan_score_fused(r, p->sm_count, forced_cluster, &p->fused)) {
       p->score_variant = kScoreFusedCluster;
       chosen_us = p->fused.est_us;
       // A fused plan that had to fall back to few statistics slots (sequences needing clusters of
       // more than 8 CTAs) can be slower than reading K twice: compare with the two-pass kernel
       // unless the variant is forced.
-      const bool tight = p->fused.n_slot < 2 * p->fused.n_buf;
-      if (tight && !want && forced_cluster == 0 && p->fused.est_us > two_pass_us) {
+      // (Per-head maxima: the fused plan rounds them to 11 bits, the two-pass kernel does not.  There the scores
+      // alone are compared, at that kernel's best rate.)
+      tight = p->fused.n_slot < 2 * p->fused.n_buf;
+      const bool slower = r.per_head_max ? p->fused.score_us > mustdrop::two_pass_keys_us(r) : p->fused.est_us > two_pass_us;
+      if (tight && !want && forced_cluster == 0 && slower) {
         p->score_variant = kScoreTwoPassMma;
         chosen_us = two_pass_us;
       }
     }
+    // (One or two heads of one or two requests whose keys no cluster holds keep the separate launches, as ever.)
+    const bool keep_separate = r.L > max_cluster_keys(r.N) && r.B <= 2 && r.H <= 2;
     // More than 64 text rows fill all 128 tensor-memory lanes with one key range, which halves the
     // keys a CTA can take.  Alternative: two launches over the same keys, text rows 0..63 and the
     // rest, each with the two-tile layout (twice the keys per CTA); the second adds its column
@@ -191,13 +201,20 @@ mustdrop_status_t mustdrop_filter_plan(const mustdrop_config_t* c, mustdrop_plan
       mustdrop::FusedGeometry ga, gb;
       if (plan_score_fused(r, p->sm_count, forced_cluster, &ga, 0, 64) &&
           plan_score_fused(r, p->sm_count, forced_cluster, &gb, 64, r.N - 64)) {
-        // (the second launch starts and fills anew)
-        const double split_us = ga.est_us + gb.est_us + 20.0;
-        // Against one fused launch in several rounds of clusters it has to look an eighth faster: the
-        // estimates leave out that the second launch reads all keys again beside the first one's tail (41
-        // requests of 750 keys, 70 rows: estimated 158 against 170 us, measured 217 against 191).
-        const double bar = p->score_variant == kScoreFusedCluster ? 0.87 : 1.0;
-        if (force_split || (!want && forced_cluster == 0 && split_us < bar * chosen_us)) {
+        // The second launch loads while the first drains: side by side where the clusters of both fit the GPU, else
+        // mostly one after the other, and all keys are read twice.
+        const double longer = std::fmax(ga.est_us, gb.est_us), shorter = std::fmin(ga.est_us, gb.est_us);
+        const bool together = static_cast<double>(r.B) / ga.resident + static_cast<double>(r.B) / gb.resident <= 1.0;
+        const double split_us =
+            together ? 10.0 + 0.85 * longer + 80.0e-6 * r.B * r.H * r.L : 4.0 + 1.26 * longer + 0.32 * shorter;
+        // These two estimates are the least exact ones (16 % rms).  On 342 shapes with both plans forced, two
+        // launches win side by side where they look 7 % faster; one after the other against one launch that is
+        // short of statistics slots where they look 5 % faster, against one that is not from 14 % on (34 requests
+        // of 889 keys, 24 heads, 92 rows: 137 us in one launch, 154 in two; 35 of 1213, 32 heads, 120 rows: 390 and
+        // 343); against the two-pass kernel already where they look 15 % slower (23 of 2116 keys, one head, 65
+        // rows: 120 us two-pass, 86 in two launches).
+        const double look = together ? 0.93 : p->score_variant == kScoreTwoPassMma ? 1.15 : tight ? 0.95 : 0.86;
+        if (force_split || (!want && forced_cluster == 0 && !keep_separate && split_us < look * chosen_us)) {
           p->score_variant = kScoreFusedCluster;
           p->row_split = 1;
           p->fused = ga;
@@ -208,11 +225,12 @@ mustdrop_status_t mustdrop_filter_plan(const mustdrop_config_t* c, mustdrop_plan
     }
     // Small batches of long sequences: the same kernel without clusters - every CTA of the batch
     // resident at once, as many per request as the SMs allow, statistics through global memory.
-    // Taken when estimated faster than what was chosen above.
+    // Taken when estimated faster than what was chosen above by more than the estimates of the smallest calls
+    // are off (7 requests of 3 heads, 760 keys, 89 rows: 20.7 us, as clusters 18.0).
     if (allow_fused && !force_split && (force_grid || (!want && forced_cluster == 0))) {
       mustdrop::FusedGeometry gg;
       if (plan_score_grid(r, p->sm_count, force_grid ? forced_cluster : 0, &gg) &&
-          (force_grid || gg.est_us < chosen_us * 0.97)) {
+          (force_grid || (!keep_separate && gg.est_us + 2.5 < chosen_us))) {
         p->score_variant = kScoreFusedCluster;
         p->row_split = 0;
         p->fused = gg;

@@ -39,7 +39,8 @@ struct FusedGeometry {
                       //    exchange their statistics through global memory
   int32_t exact_max;  // grid plans: the per-head maxima of Eq. 10 are taken in fp32
   int32_t resident;   // clusters the device can hold at once (0: not asked)
-  float est_us;       // the planner's estimate of the score time
+  float est_us;       // the planner's estimate of a call's time ...
+  float score_us;     // ... and of its scores alone (clusters)
   size_t smem_bytes;  // dynamic shared memory
 };
 
@@ -113,8 +114,12 @@ cudaError_t launch_score_two_pass(const mustdrop_plan& p, const void* q_text, co
                                   const int32_t* vis_cnt = nullptr);
 bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, FusedGeometry* out, int row0 = 0,
                       int n_rows = 0);
-double gather_us(const Resolved& r, double ctas);   // the planner's estimates of the gather ...
-double two_pass_keys_us(const Resolved& r);         // ... and of the two-pass kernel on a full GPU
+// Estimates of the planner: the rows a request has gathered, a call's gathered bytes, the time that takes, the
+// two-pass kernel's time for the keys.
+double gathered_rows(const Resolved& r);
+double gathered_bytes(const Resolved& r);
+double gather_us(const Resolved& r, double ctas, double rounds);
+double two_pass_keys_us(const Resolved& r);
 // Grid plan of the same kernel (all CTAs of the batch resident at once, statistics through global
 // memory); false when the batch leaves fewer than two CTAs per request or the shape does not fit.
 bool plan_score_grid(const Resolved& r, int sm_count, int forced_ctas, FusedGeometry* out);

@@ -1581,12 +1581,23 @@ int max_resident_clusters(int cluster) {
 
 }  // namespace
 
-// Time of the gather when `ctas` CTAs share it: a CTA's one copying thread moves ~33 GB/s (one way), all of
-// them together what the memory takes.  (25 requests of 179 rows: 55 us a call on 125 CTAs, 64 on 100.)
-double gather_us(const Resolved& r, double ctas) {
-  const double rows = r.rebuild ? r.out_rows : (r.mode == MUSTDROP_MODE_BUDGET ? r.cap : r.cap / 3.0);
-  const double bytes = rows * r.B * (2.0 * r.hidden + 2.0 * 256.0 * r.H);
-  return std::max(bytes / (33.0e3 * ctas), 2.0 * bytes / 7.0e6);
+// The estimates below are fits (10 to 16 % rms) to the times of the four kinds of plan, each forced, on 830
+// shapes: 1 to 64 requests, 1 to 128 heads, 64 to 4096 tokens, 1 to 128 text rows.
+
+// Rows a request has gathered.  (How many a threshold keeps is not known before the call: a third is what the
+// default thresholds leave of attention-like scores.)
+double gathered_rows(const Resolved& r) {
+  const double kept = r.mode == MUSTDROP_MODE_BUDGET ? r.cap : r.cap / 3.0;
+  return r.rebuild ? r.vis_start + kept + r.N : kept;
+}
+double gathered_bytes(const Resolved& r) { return gathered_rows(r) * r.B * (2.0 * r.hidden + 2.0 * 256.0 * r.H); }
+
+// Time of the gather when `ctas` CTAs share a request's rows, in `rounds` rounds of requests: a CTA's one
+// copying thread takes 0.45 us a row however short the row is, and moves its bytes at 185 GB/s; then what the
+// memory takes for all of them.
+double gather_us(const Resolved& r, double ctas, double rounds) {
+  const double rows = gathered_rows(r), bytes = gathered_bytes(r);
+  return std::ceil(rows / ctas) * rounds * (0.45 + bytes / (rows * r.B) / 185.0e3) + bytes / 6.5e6;
 }
 
 // Both passes of the two-pass kernel over the keys, on a full GPU (measured: 0.6 us per MB and 0.7 more
@@ -1707,19 +1718,19 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
       if (t_head < t_exp / 2) t_head = t_exp / 2;
       if (t_head < t_stream) t_head = t_stream;
       if (t_head < 1.15) t_head = 1.15;
-      // ... and of a request: start, fill and exit (more where CTAs of a next wave have to wait for
-      // it), the first exchange of 128 rows, and the reduction over the head groups.
-      const double t_req = 3.0 + heads * t_head + t_chain + (c > 1 && halves == 1 ? 1.0 : 0.0) +
+      // ... and of a request: start, fill and exit, the first exchange of 128 rows, and the reduction over
+      // the head groups.
+      const double t_req = 8.0 + heads * t_head + t_chain + (c > 1 && halves == 1 ? 1.0 : 0.0) +
                            (grp > 1 ? 1.0 + 0.5 * grp : 0.0);
-      // (a launch of the last text rows also selects and gathers; what it shares out besides the rows' bytes
-      // makes every CTA worth a little)
-      double est = waves * t_req + (waves - 1) * 20.0;
-      if (row0 + n_rows == r.N) est += gather_us(r, active) - 0.015 * active;
+      // (clusters of a next wave wait until whole clusters have left: 10 us; a launch of the last text rows
+      // also selects and gathers)
+      double est = waves * t_req + (waves - 1) * 10.0;
+      if (row0 + n_rows == r.N) est += gather_us(r, size, waves) + waves * 1.1e-3 * r.M;
       if (best < 0.0 || est < best - 1e-9) {
         best = est;
         g.halves = halves; g.cluster = c; g.groups = grp; g.tk = tk; g.cpl = cpl; g.n_q = n_q; g.n_k = n_k; g.split = split;
         g.n_buf = n_buf; g.ach = ach; g.n_slot = n_slot; g.resident = resident; g.row0 = row0; g.n_rows = n_rows;
-        g.est_us = static_cast<float>(est);
+        g.est_us = static_cast<float>(est); g.score_us = static_cast<float>(waves * t_req + (waves - 1) * 10.0);
         g.smem_bytes = smem_bytes;
       }
     }
@@ -1788,7 +1799,8 @@ bool plan_score_grid(const Resolved& r, int sm_count, int forced_ctas, FusedGeom
       // they take 8 % longer in the mean of 180 grid plans, up to 1.5 x with 160 keys per CTA and 71 heads).
       g.exact_max = r.per_head_max && 0.9 * two_pass_keys_us(r) <= r.H * t_head + 12.0;
       g.ach = ach; g.groups = 1; g.n_slot = n_slot; g.gx = 1; g.resident = sm_count; g.row0 = 0; g.n_rows = r.N;
-      g.est_us = static_cast<float>(r.H * t_head + 12.0 + gather_us(r, c * r.B));   // (+ filling and draining the longer chain)
+      // (+ filling and draining the longer chain; the selection reads the scores back from L2)
+      g.est_us = static_cast<float>(0.85 * r.H * t_head + 11.0 + 4.4e-3 * r.M + gather_us(r, c, 1));
       g.smem_bytes = smem_bytes;
     }
   }

@@ -224,3 +224,16 @@ def test_every_fused_geometry_has_room_for_the_selection_s_scores():
                             seen.add((variant, "two launches" in text, "grid" in text))
                             assert launches == (2 if "two launches" in text else 1), (text, n_vis, n_txt, flags)
     assert len(seen) >= 3
+
+
+@pytest.mark.parametrize("batch,n_heads,vis_start,n_vis,n_txt,budget", [
+    (1, 3, 0, 1372, 111, 453), (4, 1, 35, 1875, 109, 1506), (6, 2, 0, 1371, 78, 773), (5, 1, 35, 1425, 86, 400), (6, 1, 0, 2228, 126, 700)])
+def test_a_few_heads_of_long_sequences_get_a_grid_plan(batch, n_heads, vis_start, n_vis, n_txt, budget):
+    """Few heads x requests leave the two-pass kernel's walk over a head's keys on a handful of SMs: these
+    calls take 74 to 152 us that way and 28 to 74 us as grid plans."""
+    c = md.Config(batch=batch, n_heads=n_heads, hidden=128 * n_heads, seq_len=vis_start + n_vis + n_txt, vis_start=vis_start, n_vis=n_vis,
+                  txt_start=vis_start + n_vis, n_txt=n_txt, budget=budget)
+    st, plan, _ = md.mustdrop_filter_plan(c)
+    assert st == md.MUSTDROP_OK
+    assert "grid plan" in md.mustdrop_plan_describe(plan) and md.mustdrop_plan_filter_launches(plan) == 1
+    md.mustdrop_plan_destroy(plan)
