@@ -1,20 +1,22 @@
 // Importance scores in ONE pass over the keys (Eq. 1, Eq. 8, Eq. 10), sm_100a only.
 //
-// A thread-block cluster owns one request and splits its L keys over its CTAs; each CTA loops
-// over the heads.  Warp roles inside a CTA (16 warps):
+// A thread-block cluster owns one request: `groups` groups of C CTAs, each group with a share of the heads
+// (one group has them all); the CTAs of a group split the L keys, and each loops over the group's heads.
+// Warp roles inside a CTA (16 warps):
 //   TMA warp      stages the CTA's K rows and the head's text queries in shared memory;
 //   MMA warp      one thread issues tcgen05 MMAs (bf16 in, fp32 logits in tensor memory);
-//   8 exp warps   read the logits with text queries on the TMEM lanes (a thread owns one text row
-//                 and a run of key columns, so row maxima and sums are in-thread), write the
-//                 exponentials back to tensor memory and send their (max, sum) pairs to every
-//                 CTA of the cluster with asynchronous distributed-shared-memory stores that
-//                 count on the receiver's mbarrier;
+//   8 exp warps   two groups of four that alternate heads: read the logits with text queries on the TMEM
+//                 lanes (a thread owns one text row and a run of key columns, so row maxima and sums are
+//                 in-thread), write the exponentials back to tensor memory and send their (stabiliser,
+//                 sum) pairs to every CTA of the group with asynchronous distributed-shared-memory
+//                 stores that count on the receiver's mbarrier;
 //   4 add warps   once all pairs of a head have arrived, normalise the exponentials and add them
 //                 into per-thread head sums that live in registers for the whole kernel.
 // Three to eight tensor-memory buffers (as many as the columns per head allow) keep the MMA, exp
 // and add stages of consecutive heads in flight.
-// After the last head the head mean is reduced over the text rows into G (column sum) and
-// I (column max).  K is read once; nothing goes through global scratch.
+// After the last head the add warps stage the head sums in shared memory and the exp warps reduce them -
+// over the groups, through distributed shared memory, and over the text rows - into G (column sum) and I
+// (column max).  K is read once; nothing goes through global scratch (grid plans: the statistics do).
 //
 // Lane layouts.  N <= 64: two M=64 MMAs per head write the two halves of the CTA's key range
 // to the lower and upper 16 lanes of every 32-lane TMEM quadrant, so all 128 lanes carry one of
@@ -40,7 +42,7 @@
 namespace mustdrop {
 namespace {
 
-constexpr int kExpWarps = 8;                // warps 0-7: 4 TMEM lane quadrants x 2 column groups
+constexpr int kExpWarps = 8;                // warps 0-7: 4 TMEM lane quadrants x 2 groups that alternate heads
 constexpr int kColGroups = 2;
 constexpr int kPhPairs = 1, kPhExact = 2;    // per-head maxima (Eq. 10): how they travel between the lanes
 constexpr float kPhScale = 16384.0f;        // ... as fp16 pairs: times 2^14
@@ -80,7 +82,7 @@ struct FusedParams {
   // Statistics exchange through global memory instead of distributed shared memory ("grid" plans:
   // the CTAs of a request are ordinary CTAs of the grid, any number of them, all resident at once).
   int32_t gx;                         // 1: grid plan (cluster = CTAs per request, launched without a cluster)
-  float2* gx_stats;                   // [B][H][CTAs per request][rows][pairs] (stabiliser, sum)
+  float2* gx_stats;                   // [B][H][CTAs per request][rows] (stabiliser, sum)
   uint32_t* gx_cnt;                   // [B*H] CTAs that published a head, [B] scores stored, [B] CTAs that left; zero between calls
   int32_t per_head;                   // 1: i_out = head mean of the per-head maxima over the text rows (PH instantiations)
   int32_t early_inputs;               // 1: q_text / k may be read before the stream's earlier work has completed (caller's promise)
@@ -416,7 +418,7 @@ struct __align__(8) Barriers {
   uint64_t sfull[kMaxSlots];    // all CTAs' (max, sum) pairs of a head have arrived
   uint64_t fin;                  // add warps meet before staging the head sums
   uint64_t ph;                   // add warps meet once per head (per-head maxima of Eq. 10)
-  uint64_t gsent[kMaxBufs];      // grid plans: exp warps -> publishing thread: this CTA's pairs of a head are in global memory
+  uint64_t gsent[kMaxBufs];      // grid plans: exp warps -> publishing warp: this CTA's pairs of a head are in its shared memory
   uint64_t gfull[kMaxGatherSlots];   // filter tail: a gathered row has landed in its slot
 };
 
@@ -907,9 +909,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       asm volatile("cp.async.wait_all;" ::: "memory");   // no copy of this warp is in flight when the CTA leaves
     } else if (warp == kMmaWarp + 2 && p.gx) {
       // ---------------- publishing warp (grid plans) ----------------
-      // Once all exp warps of this CTA have left their pairs of a head in shared memory: merge the
-      // pairs of each row into one, store it to global memory, then one fence and one counted
-      // release for the CTA - the round trip of the fence is off the exp warps' path.
+      // Once the exp warps of this CTA have left a head's pairs, one per row, in shared memory: copy them to
+      // global memory, then one counted release for the CTA - its round trip is off the exp warps' path.
       pdl_wait();   // global memory of the workspace: not before the stream's earlier work is done
       for (int h = 0; h < n_heads; ++h) {
         const int buf = h % p.n_buf;
@@ -1088,8 +1089,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       }
       if (HALVES == 2) lsum += __shfl_xor_sync(0xffffffffu, lsum, 16);
       if (p.gx) {
-        // grid plan: the pair stays in this CTA's shared memory; the publishing warp merges the CTA's
-        // pairs of a row and sends one pair per row on its way through global memory
+        // grid plan: the pair stays in this CTA's shared memory; the publishing warp sends it on its way
+        // through global memory
         if (sender) own_pairs[buf * NROWS + row] = make_float2(mx, lsum);
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&bars.gsent[buf]));
@@ -1688,7 +1689,7 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
     // A group loops over fewer heads, which costs one reduction of the groups' head sums through
     // distributed shared memory at the end; spending the CTAs on more key ranges per head instead (a
     // larger c) makes every head narrower, but a head costs ~1.2 us however narrow it is.  One
-    // request of 608 keys: 47.6 us as 16 key ranges, 25.2 as 4 x 4; 16 requests, budget 192: 76.1 us
+    // request of 608 keys: 47.6 us as 16 key ranges, 25.2 as 8 groups x 2; 16 requests, budget 192: 76.1 us
     // as 6, 64.3 as 2 groups x 3.  (Not with a forced cluster size or a tight window.)
     const int max_s = forced_cluster > 0 || is_tight ? 1 : kMaxCluster / c;
     for (int grp = 1; grp <= max_s && grp <= r.H; ++grp) {
@@ -1868,11 +1869,12 @@ cudaError_t launch_fused_common(const mustdrop_plan& plan, const FusedGeometry& 
   p.early_inputs = (combine || (r.inputs_ready && vis_cnt == nullptr)) ? 1 : 0;
   p.release_late = plan.row_split && !combine ? 1 : 0;
   p.wait_cycles = r.wait_cycles > 0 ? r.wait_cycles : kWaitCycles;
-  // The gather reads the kept tokens' keys a second time.  Where the keys of the requests that are
-  // resident at once are not far beyond L2 they stay there with normal priority (16 requests of 640
-  // keys, budget 192: 64.1 -> 57.1 us a call; 8 of 2944: 83.3 -> 82.7; two waves of 33 requests of 704
-  // keys and 40 heads: 245 -> 242); beyond twice its size they leave first, so that they do not push
-  // out what other kernels keep there (64 requests of 640 keys: 105.4, with normal priority 107.4).
+  // The gather reads the kept tokens' keys a second time, a row at a time.  Where the keys of the requests that
+  // are resident at once are not far beyond L2 they stay there with normal priority; beyond twice its size
+  // they leave first, so that they do not push out what other kernels keep there.  First out against kept, on
+  // buffers that no recent call has touched (7 to 9 sets in turn, over 4 x L2 of keys; with three sets the same):
+  // 16 requests of 640 keys, budget 192: 63.8 and 56.6 us a call; 24 with per-head maxima: 84.0 and 76.7; 12 as
+  // three calls, 144: 48.8 and 47.3; 8 of 2144: 88.3 and 87.1; 64 of 640 (320 MB): 105.1 and 106.8.
   const int64_t at_once = geo.resident > 0 && geo.resident < r.B && !geo.gx ? geo.resident : r.B;
   // Not where less than an eighth is gathered (18 of 551 keys, budget 29 of 406: 56.8 us, first out 55.3),
   // and not where two launches share the text rows (51 of 1389 keys, 8 heads: 208.8, first out 193.1).

@@ -1,11 +1,5 @@
 // Dual criteria, key set and selection: one CTA per request (Eq. 9, Eq. 10; Sec. 3.3 key set).
 //
-// The per-token score is computed in fp32 with one rounding per operation (no fused
-// multiply-add, IEEE division), because it decides which indices are kept.  Budget mode is a
-// radix select over the order-preserving integer image of the score, followed by an
-// index-ordered emit, so kept indices come out ascending and equal scores resolve to the
-// lower index.
-//
 // The work of a request is in select_body.cuh; this file is the stand-alone kernel around it.
 #include "select_body.cuh"
 

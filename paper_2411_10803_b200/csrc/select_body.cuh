@@ -3,8 +3,9 @@
 // request) and by the single-launch filter kernel (the first eight warps of every CTA of the
 // request).
 //
-// The per-token score is computed in fp32 with one rounding per operation (no fused
-// multiply-add, IEEE division), because it decides which indices are kept.  Budget mode is a
+// The per-token score is computed in fp32 with one rounding per operation (the quotients are correctly
+// rounded: corrected reciprocal products where that is exact, IEEE division elsewhere), because it decides
+// which indices are kept.  Budget mode is a
 // radix select over the order-preserving integer image of the score, followed by an
 // index-ordered emit, so kept indices come out ascending and equal scores resolve to the
 // lower index.
@@ -16,9 +17,9 @@
 // tokens, where the size of the code counts, four strips a trip (their loads overlap) beyond; a
 // digit's bins are scanned by every warp for itself (no barrier), and once the cut bin holds at
 // most 64 tokens - nearly always after one digit or two - they are ranked against each other directly;
-// the kept set is a bitmap whose words are ballots, so positions come from popcounts.  The filter of
-// 8 requests of 2880 tokens takes 83.9 us a call this way, 93.4 with up to 16 consecutive tokens in
-// each thread's registers.
+// the kept set is a bitmap whose words are ballots, so positions come from popcounts.  From the
+// last barrier before it to the list, in the filter kernel: 4.5 us for 576 tokens, 7.4 for 1369, 11.8 for 2880 (with
+// up to 16 consecutive tokens in each thread's registers 4.6, 6.7 and 14.1).
 #pragma once
 
 #include "mustdrop_internal.h"
