@@ -209,11 +209,11 @@ mustdrop_status_t mustdrop_filter_plan(const mustdrop_config_t* c, mustdrop_plan
             together ? 10.0 + 0.85 * longer + 80.0e-6 * r.B * r.H * r.L : 4.0 + 1.26 * longer + 0.32 * shorter;
         // These two estimates are the least exact ones (16 % rms).  On 342 shapes with both plans forced, two
         // launches win side by side where they look 7 % faster; one after the other against one launch that is
-        // short of statistics slots where they look 5 % faster, against one that is not from 14 % on (34 requests
-        // of 889 keys, 24 heads, 92 rows: 137 us in one launch, 154 in two; 35 of 1213, 32 heads, 120 rows: 390 and
-        // 343); against the two-pass kernel already where they look 15 % slower (23 of 2116 keys, one head, 65
+        // short of statistics slots where they look 5 % faster, against one that is not from a quarter on (34
+        // requests of 889 keys, 24 heads, 92 rows: 137 us in one launch, 154 in two; 35 of 1213, 32 heads, 120 rows:
+        // 390 and 343); against the two-pass kernel already where they look 15 % slower (23 of 2116 keys, one head, 65
         // rows: 120 us two-pass, 86 in two launches).
-        const double look = together ? 0.93 : p->score_variant == kScoreTwoPassMma ? 1.15 : tight ? 0.95 : 0.86;
+        const double look = together ? 0.93 : p->score_variant == kScoreTwoPassMma ? 1.15 : tight ? 0.95 : 0.74;
         if (force_split || (!want && forced_cluster == 0 && !keep_separate && split_us < look * chosen_us)) {
           p->score_variant = kScoreFusedCluster;
           p->row_split = 1;
@@ -226,11 +226,16 @@ mustdrop_status_t mustdrop_filter_plan(const mustdrop_config_t* c, mustdrop_plan
     // Small batches of long sequences: the same kernel without clusters - every CTA of the batch
     // resident at once, as many per request as the SMs allow, statistics through global memory.
     // Taken when estimated faster than what was chosen above by more than the estimates of the smallest calls
-    // are off (7 requests of 3 heads, 760 keys, 89 rows: 20.7 us, as clusters 18.0).
+    // are off (7 requests of 3 heads, 760 keys, 89 rows: 20.7 us, as clusters 18.0), and than clusters with a
+    // full set of statistics slots by 5 % (280 shapes with both forced: where the estimates are 5 to 8 % apart
+    // the grid plan takes 0.99 of the time in the mean, where less than 5 %, 1.04; 18 requests of 1476 keys, 40
+    // heads: 142 against 146 us estimated, 173 against 164 measured).
+    const bool full_slots = p->score_variant == kScoreFusedCluster && !p->row_split && !tight;
     if (allow_fused && !force_split && (force_grid || (!want && forced_cluster == 0))) {
       mustdrop::FusedGeometry gg;
       if (plan_score_grid(r, p->sm_count, force_grid ? forced_cluster : 0, &gg) &&
-          (force_grid || (!keep_separate && gg.est_us + 2.5 < chosen_us))) {
+          (force_grid || (!keep_separate && gg.est_us + 2.5 < chosen_us &&
+                           gg.est_us < (full_slots ? 0.95 : 1.0) * chosen_us))) {
         p->score_variant = kScoreFusedCluster;
         p->row_split = 0;
         p->fused = gg;

@@ -237,3 +237,16 @@ def test_a_few_heads_of_long_sequences_get_a_grid_plan(batch, n_heads, vis_start
     assert st == md.MUSTDROP_OK
     assert "grid plan" in md.mustdrop_plan_describe(plan) and md.mustdrop_plan_filter_launches(plan) == 1
     md.mustdrop_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("batch,n_heads,vis_start,n_vis,n_txt,budget", [
+    (18, 40, 35, 1408, 33, 461),     # 164 us on clusters; as a grid plan, which looks 3 % faster, 173
+    (34, 24, 0, 797, 92, 115)])      # 137 us; the text rows in two launches, which look a sixth faster: 154
+def test_another_kind_of_plan_has_to_look_clearly_faster_than_clusters(batch, n_heads, vis_start, n_vis, n_txt, budget):
+    c = md.Config(batch=batch, n_heads=n_heads, hidden=128 * n_heads, seq_len=vis_start + n_vis + n_txt, vis_start=vis_start, n_vis=n_vis,
+                  txt_start=vis_start + n_vis, n_txt=n_txt, budget=budget)
+    st, plan, _ = md.mustdrop_filter_plan(c)
+    assert st == md.MUSTDROP_OK
+    text = md.mustdrop_plan_describe(plan)
+    assert "cluster" in text and "two launches" not in text, text
+    md.mustdrop_plan_destroy(plan)
