@@ -1729,6 +1729,10 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
       // fewest of 420 shapes came out slower than under the estimate before, at the same mean.)
       double est = waves * t_req + (waves - 1) * 10.0;
       if (row0 + n_rows == r.N) est += gather_us(r, size, waves) + waves * 1.1e-3 * r.M - 0.05 * active;
+      // Clusters of five: 24 fit three to a processing cluster; the places of a 25th and 26th are whole only once
+      // the call before has left altogether.  Calls in a row of 25 and 26 requests of 948 keys, 32 heads: 81 and
+      // 103 us where one alone takes 70 (24 requests: 65); as clusters of four 71.
+      if (size == 5 && r.B > 24 && r.B <= resident) est *= 1.0 + 0.2 * (r.B - 24);
       if (best < 0.0 || est < best - 1e-9) {
         best = est;
         g.halves = halves; g.cluster = c; g.groups = grp; g.tk = tk; g.cpl = cpl; g.n_q = n_q; g.n_k = n_k; g.split = split;

@@ -250,3 +250,13 @@ def test_another_kind_of_plan_has_to_look_clearly_faster_than_clusters(batch, n_
     text = md.mustdrop_plan_describe(plan)
     assert "cluster" in text and "two launches" not in text, text
     md.mustdrop_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("batch", [25, 26])
+def test_clusters_of_five_leave_their_last_places_free(batch):
+    """25 and 26 clusters of five fit the GPU, but calls in a row wait for the last places (up to 103 us where
+    a call alone takes 70); clusters of four take 71."""
+    c = md.Config(batch=batch, n_heads=32, hidden=4096, seq_len=948, vis_start=35, n_vis=894, txt_start=929, n_txt=19, budget=61)
+    st, plan, _ = md.mustdrop_filter_plan(c)
+    assert st == md.MUSTDROP_OK and "cluster 5," not in md.mustdrop_plan_describe(plan)
+    md.mustdrop_plan_destroy(plan)
