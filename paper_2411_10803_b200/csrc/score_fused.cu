@@ -14,6 +14,7 @@
 //                 into per-thread head sums that live in registers for the whole kernel.
 // Three to eight tensor-memory buffers (as many as the columns per head allow) keep the MMA, exp
 // and add stages of consecutive heads in flight.
+// (Tiles of 176 columns keep the last 16 of them apart: kExtra.)
 // After the last head the add warps stage the head sums in shared memory and the exp warps reduce them -
 // over the groups, through distributed shared memory, and over the text rows - into G (column sum) and I
 // (column max).  K is read once; nothing goes through global scratch (grid plans: the statistics do).
@@ -56,10 +57,13 @@ constexpr int kChunk = 16;                  // TMEM columns per tcgen05.ld / st
 constexpr int kMaxCluster = 16;               // beyond 8 the cluster size is non-portable (opt-in per kernel)
 constexpr int kMaxQBufs = 4;                  // shared-memory ring of text-query tiles (one per head)
 constexpr int kMaxKBufs = 8;                  // shared-memory ring of key half-tiles (HALVES per head)
-constexpr int kMinBufs = 3;                 // tensor-memory buffers: MMA, exp and add stages in flight (two for 176-column tiles) ...
+constexpr int kMinBufs = 3;                 // tensor-memory buffers: MMA, exp and add stages in flight (176-column tiles: two at least) ...
 constexpr int kMaxBufs = 8;                 // ... more when the columns per head allow, to hide the per-head latency chain
 constexpr int kMaxSlots = 2 * kMaxBufs;     // statistics slots = 2 x buffers: a peer's exp warps run at most that far ahead of our add warps
 constexpr int kTmemCols = 512;
+constexpr int kExtraCols = 16;              // 176-column tiles: the last chunk of a head has a place of its own (see kExtra) ...
+constexpr int kExtraAt = kTmemCols - 2 * kExtraCols;   // ... of which there are two, behind three buffers of 160 columns
+constexpr size_t kExtraBytes = kExtraCols * 128 * 4;   // ... and its exponentials lie in shared memory, per buffer
 constexpr int kMaxGatherSlots = 8;         // rows in flight per CTA in the gather tail of the filter kernel
 constexpr size_t kMinSmem = 116 * 1024;     // least dynamic shared memory of a CTA, so that two (each wanting all of tensor memory) never share an SM
 constexpr int kKeptListBytes = kMaxVis * 4; // the request's kept indices, at the start of dynamic shared memory
@@ -415,6 +419,7 @@ struct __align__(8) Barriers {
   uint64_t tfull[kMaxBufs];      // MMA -> exp warps: logits of a head are in tensor memory
   uint64_t eready[kMaxBufs];     // exp -> add warps: exponentials of a head are in tensor memory
   uint64_t tempty[kMaxBufs];     // add warps -> MMA: tensor-memory buffer free
+  uint64_t xempty[2];            // exp warps -> MMA: place of a head's last chunk free (176-column tiles)
   uint64_t sfull[kMaxSlots];    // all CTAs' (max, sum) pairs of a head have arrived
   uint64_t fin;                  // add warps meet before staging the head sums
   uint64_t ph;                   // add warps meet once per head (per-head maxima of Eq. 10)
@@ -530,6 +535,14 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
   // stores - runs under the other group's loop.  (Splitting every head's chunks over the two warps
   // instead left those 0.7 us per head on the path of every head: 7 % of a step at the target point.)
   constexpr bool kRealloc = ACH > 5;             // move registers from the other warpgroups to the add warps
+  // 176-column tiles.  A buffer is held from a head's MMAs until its sums - 4.7 us of MMAs, exponentials,
+  // exchange and sums - and tensor memory has room for two of 176 columns: 2.36 us a head.  So the buffers
+  // hold the first 160 columns only, which makes three of them, and the last 16 columns' logits go to one of two
+  // places behind: the exp warps take them into registers as soon as they get to the head, and leave their
+  // exponentials in shared memory.  64 requests of 704 keys, 128 rows, 40 heads: 240.1 -> 216.1 us a call (the
+  // exp warps are what a head waits for then).
+  constexpr bool kExtra = ACH > 10;
+  constexpr int kBufChunks = kExtra ? 10 : ACH;  // (at most) chunks of a head in its buffer
 
   extern __shared__ __align__(1024) unsigned char smem_dyn[];
   __shared__ Barriers bars;
@@ -569,6 +582,9 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
   float* const ph_stage = reinterpret_cast<float*>(stats + static_cast<size_t>(p.n_slot) * slot_pairs);
   // grid plans only: [n_buf][rows] the pairs of this CTA's own exp warps, per tensor-memory buffer
   float2* const own_pairs = reinterpret_cast<float2*>(ph_stage + (PH ? 2 * kAddWarps * p.tk : 0));
+  // 176-column tiles only: [n_buf][4][rows] exponentials of the last 16 columns, four to a vector
+  float4* const extra_exps = reinterpret_cast<float4*>(own_pairs);
+  const uint32_t buf_cols = kExtra ? static_cast<uint32_t>(kBufChunks * kChunk) : static_cast<uint32_t>(p.cpl);
 
   __shared__ SelectShared sel_sh;       // (FILTER: cleared and the key set marked long before the scores are complete)
   if constexpr (FILTER) select_clear(sel_sh, threadIdx.x, kThreads);
@@ -582,6 +598,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       mbar_init(smem_u32(&bars.eready[s]), kExpWarps / kColGroups);   // (the four warps of the head's group)
       mbar_init(smem_u32(&bars.tempty[s]), kAddWarps);
     }
+    for (int s = 0; s < 2; ++s) mbar_init(smem_u32(&bars.xempty[s]), kExpWarps / kColGroups);
     // (grid plans: the 32 lanes of the fetch warp each arrive once their copies have landed)
     for (int s = 0; s < kMaxSlots; ++s) mbar_init(smem_u32(&bars.sfull[s]), p.gx ? 32 : 1);
     mbar_init(smem_u32(&bars.fin), kAddThreads);
@@ -780,8 +797,23 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
 #endif
     } else if (warp == kMmaWarp && lane == 0) {
       // ---------------- MMA issuer ----------------
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(p.cpl >> 3) << 17) |
-                             (static_cast<uint32_t>(NROWS >> 4) << 24);
+      const uint32_t idesc_any = (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(NROWS >> 4) << 24);
+      const uint32_t idesc = idesc_any | ((buf_cols >> 3) << 17);
+      // The last 16 columns of head h (keys from row 160 of the tile on), once the exp warps have taken those of
+      // head h - 2 out of their place.
+      auto extra_mma = [&](int h, uint32_t q_src, uint32_t k_src, uint32_t slab_bytes) {
+        if constexpr (kExtra) {
+          if (!mbar_wait(smem_u32(&bars.xempty[h & 1]), (static_cast<uint32_t>(h >> 1) & 1u) ^ 1u, abort_flag, wait_limit)) return false;
+          tc_fence_after();
+#pragma unroll
+          for (int ks = 0; ks < 8; ++ks) {
+            const uint32_t slab = ks >> 2, koff = (ks & 3) * 32u;
+            tc_mma(tmem_base + static_cast<uint32_t>(kExtraAt + (h & 1) * kExtraCols), smem_desc(q_src + slab * (NROWS * 128u) + koff),
+                   smem_desc(k_src + slab * slab_bytes + buf_cols * 128u + koff), idesc_any | ((kExtraCols >> 3) << 17), ks > 0 ? 1u : 0u);
+          }
+        }
+        return true;
+      };
       int committed = -1;   // last head whose MMAs were committed to its tfull barrier
       if (p.split) {
         int k_used = 0;
@@ -804,13 +836,17 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             tc_fence_after();
             const uint32_t k_src = k_base + ki * kh_bytes;
             // the second M=64 tile goes to the upper 16 lanes of every TMEM quadrant
-            const uint32_t d = tmem_base + static_cast<uint32_t>(buf * p.cpl) + (hv ? (16u << 16) : 0u);
+            const uint32_t d = tmem_base + static_cast<uint32_t>(buf) * buf_cols + (hv ? (16u << 16) : 0u);
   #pragma unroll
             for (int ks = 0; ks < 8; ++ks) {
               const uint32_t slab = ks >> 2, koff = (ks & 3) * 32u;
               const uint64_t ad = smem_desc(q_src + slab * (NROWS * 128u) + koff);
               const uint64_t bd = smem_desc(k_src + slab * (p.cpl * 128u) + koff);
               tc_mma(d, ad, bd, idesc, ks > 0 ? 1u : 0u);
+            }
+            if (!extra_mma(h, q_src, k_src, static_cast<uint32_t>(p.cpl) * 128u)) {
+              ok = false;
+              break;
             }
             tc_commit(smem_u32(&bars.empty[ki]));   // this half-tile may be refilled once its MMAs are done
             ++k_used;
@@ -835,7 +871,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
   #pragma unroll
           for (int hv = 0; hv < HALVES; ++hv) {
             // the second M=64 tile goes to the upper 16 lanes of every TMEM quadrant
-            const uint32_t d = tmem_base + static_cast<uint32_t>(buf * p.cpl) + (hv ? (16u << 16) : 0u);
+            const uint32_t d = tmem_base + static_cast<uint32_t>(buf) * buf_cols + (hv ? (16u << 16) : 0u);
   #pragma unroll
             for (int ks = 0; ks < 8; ++ks) {
               const uint32_t slab = ks >> 2, koff = (ks & 3) * 32u;
@@ -844,6 +880,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
               tc_mma(d, ad, bd, idesc, ks > 0 ? 1u : 0u);
             }
           }
+          if (!extra_mma(h, q_src, k_src, static_cast<uint32_t>(p.tk) * 128u)) break;
           tc_commit(smem_u32(&bars.empty[s]));
           tc_commit(smem_u32(&bars.tfull[buf]));
           committed = h;
@@ -939,14 +976,14 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     }
   } else if (warp < kExpWarps) {
     // ---------------- exp warps ----------------
-    if (kRealloc) asm volatile("setmaxnreg.dec.sync.aligned.u32 112;");
+    if (kRealloc) asm volatile("setmaxnreg.dec.sync.aligned.u32 120;");
     const int q = warp & 3, g = warp >> 2;
     const int half = (HALVES == 2) ? (lane >> 4) : 0;
     const int row = (HALVES == 2) ? (16 * q + (lane & 15)) : (32 * q + lane);
     const uint32_t lane_addr = static_cast<uint32_t>(32 * q) << 16;
     const int total_chunks = p.cpl / kChunk;
-    // chunks g, g+2, ... of every head, or all chunks of every second head (uniform per warp)
-    const int my_chunks = total_chunks;
+    // all chunks of every second head (uniform per warp)
+    const int my_chunks = kExtra ? kBufChunks : total_chunks;   // (... in its buffer)
     auto chunk_of = [&](int t) { return t; };
     const int key_lane0 = static_cast<int>(rank) * p.tk + half * p.cpl;        // key of this lane's column 0
     int lim = p.causal ? (txt_start + p.row0 + row + 1) : Lb;                  // keys below lim are visible
@@ -968,7 +1005,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     }
     // chunk c (columns 16c .. 16c + 15) is partly visible to a lane only if 16c < lim < 16c + 16
     const int mix_lo = lim_lo / kChunk;
-    const int mix_hi = (lim_hi + kChunk - 1) / kChunk;
+    const int mix_hi = min((lim_hi + kChunk - 1) / kChunk, my_chunks);
     const bool sender = (half == 0);           // with two halves, lanes s and s+16 share a row: the lower one sends
     const uint32_t pair_idx = rank * NROWS + row;                              // this thread's pair in a slot
 
@@ -993,7 +1030,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         mbar_expect_tx(smem_u32(&bars.sfull[slot]), slot_pairs * 8u);
       }
       tc_fence_after();
-      const uint32_t tbuf = tmem_base + static_cast<uint32_t>(buf * p.cpl) + lane_addr;
+      const uint32_t tbuf = tmem_base + static_cast<uint32_t>(buf) * buf_cols + lane_addr;
       const uint32_t slot_addr = smem_u32(&stats[slot * slot_pairs + pair_idx]);
       const uint32_t bar_addr = smem_u32(&bars.sfull[slot]);
       // The thread's chunks go through a loop of one chunk per trip whose only taken branch is the
@@ -1014,9 +1051,16 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       constexpr float kSumLimit = 1.0995116e12f;   // 2^40
       constexpr float kHidden = -3.0e38f;           // logit of a column the lane must not see (finite: 0 * kHidden = 0)
       float z[kChunk], e[kChunk];
+      [[maybe_unused]] float zx[kChunk];   // kExtra: the logits of the last 16 columns
       tc_ld16(tbuf + kChunk * chunk_of(0), z);
+      if constexpr (kExtra) tc_ld16(tmem_base + static_cast<uint32_t>(kExtraAt + (h & 1) * kExtraCols) + lane_addr, zx);
       float mx = -INFINITY, sub = 0.0f;
       tc_wait_ld();
+      if constexpr (kExtra) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bars.xempty[h & 1]));
+      }
       if (mix_lo < mix_hi) {
         // Chunks partly visible to some lane of this warp (the causal triangle, the end of the
         // sequence: one or two per head, and only in the CTA that holds them): the logits of the
@@ -1082,7 +1126,45 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         tc_st16_if(ok, tbuf + kChunk * c, e);
         stored += ok ? 1 : 0;
       }
-      if (stored < my_chunks) {   // rare
+      if constexpr (kExtra) {
+        // the last 16 columns, from registers: like a chunk of the loop, but for the place of its exponentials
+        const int nvis = lim - kChunk * kBufChunks;
+#pragma unroll
+        for (int j = 0; j < kChunk; ++j) zx[j] = j < nvis ? zx[j] : kHidden;
+        auto exps = [&]() {
+          const float sc = nvis > 0 ? p.scale_log2e : 0.0f, ns = nvis > 0 ? -sub : -INFINITY;
+          const uint64_t sc2 = pack2(sc, sc), ns2 = pack2(ns, ns);
+          uint64_t part2[2] = {0ull, 0ull};
+#pragma unroll
+          for (int j = 0; j < kChunk; j += 2) {
+            unpack2(fma2(pack2(zx[j], zx[j + 1]), sc2, ns2), e[j], e[j + 1]);
+            e[j] = ex2(e[j]);
+            e[j + 1] = ex2(e[j + 1]);
+            part2[(j >> 1) & 1] = add2(part2[(j >> 1) & 1], pack2(e[j], e[j + 1]));
+          }
+          float part[4];
+          unpack2(part2[0], part[0], part[1]);
+          unpack2(part2[1], part[2], part[3]);
+          return nvis > 0 ? (part[0] + part[1]) + (part[2] + part[3]) : 0.0f;
+        };
+        float psum = exps();
+        if (!ok || __any_sync(0xffffffffu, !(psum < kSumLimit))) {   // rare: as in redo_rest
+          const RedoResult r = redo_rest(tbuf, kChunk, stored, my_chunks, lim, kChunk, p.scale_log2e, false, mx, lsum);
+          float cm = -INFINITY;
+#pragma unroll
+          for (int j = 0; j < kChunk; ++j) cm = fmaxf(cm, j < nvis ? zx[j] : -INFINITY);
+          mx = fmaxf(r.mx, cm * p.scale_log2e);
+          sub = (mx == -INFINITY) ? 0.0f : mx;
+          const float fac = (mx == r.mx || r.mx == -INFINITY) ? 1.0f : ex2(r.mx - mx);
+          if (__any_sync(0xffffffffu, fac != 1.0f)) rescale_stored(tbuf, kChunk, my_chunks, fac);
+          lsum = r.l * fac;
+          psum = exps();
+        }
+        lsum += psum;
+        float4* const to = extra_exps + static_cast<size_t>(buf) * (kExtraCols / 4) * NROWS + row;
+#pragma unroll
+        for (int j = 0; j < kChunk; j += 4) to[(j / 4) * NROWS] = make_float4(e[j], e[j + 1], e[j + 2], e[j + 3]);
+      } else if (stored < my_chunks) {   // rare
         const RedoResult r = redo_rest(tbuf, kChunk, stored, my_chunks, lim, kChunk, p.scale_log2e, HALVES == 2, mx, lsum);
         mx = r.mx;
         lsum = r.l;
@@ -1302,14 +1384,23 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.eready[buf]), bph, abort_flag, wait_limit))) break;
       if (tid_a == 0) MD_TRACE(h, 6);
       tc_fence_after();
-      const uint32_t tbuf = tmem_base + static_cast<uint32_t>(buf * p.cpl) + lane_addr;
+      const uint32_t tbuf = tmem_base + static_cast<uint32_t>(buf) * buf_cols + lane_addr;
 #pragma unroll
       for (int c0 = 0; c0 < ACH; c0 += 2) {
         if (c0 < total_chunks) {
           float e[2][kChunk];
-          tc_ld16(tbuf + kChunk * c0, e[0]);
-          if (c0 + 1 < ACH && c0 + 1 < total_chunks) tc_ld16(tbuf + kChunk * (c0 + 1), e[1]);
-          tc_wait_ld();
+          if (kExtra && c0 == kBufChunks) {
+            const float4* const from = extra_exps + static_cast<size_t>(buf) * (kExtraCols / 4) * NROWS + row;
+#pragma unroll
+            for (int j = 0; j < kChunk; j += 4) {
+              const float4 v = from[(j / 4) * NROWS];
+              e[0][j] = v.x; e[0][j + 1] = v.y; e[0][j + 2] = v.z; e[0][j + 3] = v.w;
+            }
+          } else {
+            tc_ld16(tbuf + kChunk * c0, e[0]);
+            if (c0 + 1 < ACH && c0 + 1 < total_chunks) tc_ld16(tbuf + kChunk * (c0 + 1), e[1]);
+            tc_wait_ld();
+          }
           const uint64_t f_2 = pack2(f, f);
 #pragma unroll
           for (int j = 0; j < kChunk; j += 2) acc[c0][j >> 1] = fma2(pack2(e[0][j], e[0][j + 1]), f_2, acc[c0][j >> 1]);
@@ -1629,7 +1720,8 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
     // slot size in pairs per row and CTA.  The kernel sends ONE pair per row; wide tiles keep the room for
     // two that they had when the two exp warps of a quadrant shared a head: the cost model's constants and
     // every measured plan choice rest on the stage / buffer / slot counts that this sizing gives.
-    const int epr = ach <= 5 ? 1 : kColGroups;
+    // (Not the 176-column tiles, whose third buffer's slots and exponentials need the room.)
+    const int epr = ach <= 5 || ach > 10 ? 1 : kColGroups;
     // Shared memory.  Whole stages first (a head's query tile and keys recycled together): as many
     // tensor-memory buffers as the columns allow (3..8), fewer if their statistics slots (2 x
     // buffers x cluster x rows x pairs x 8 bytes) would leave no room for 2 stages; four stages
@@ -1642,9 +1734,11 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
     const size_t ph_bytes = r.per_head_max ? static_cast<size_t>(2 * kAddWarps) * tk * sizeof(float) : 0;
     const size_t avail = 227 * 1024 - 4096 /* static */ - 1024 /* alignment */ - ph_bytes;
     auto slots_bytes = [&](int n_slot) { return static_cast<size_t>(n_slot) * c * nrows * epr * 8; };
-    int n_buf = kTmemCols / cpl;
+    const bool extra_cols = cpl > 10 * kChunk;               // 176-column tiles: buffers of 160, exponentials of the rest in shared memory
+    int n_buf = extra_cols ? kExtraAt / (10 * kChunk) : kTmemCols / cpl;
     if (n_buf > kMaxBufs) n_buf = kMaxBufs;
-    const int min_bufs = cpl > 10 * kChunk ? 2 : kMinBufs;   // 176-column tiles: two buffers is all that fits
+    const int min_bufs = extra_cols ? 2 : kMinBufs;
+    const size_t x_bytes = extra_cols ? kExtraBytes : 0;     // per buffer
     if (n_buf < min_bufs) continue;
     const int max_buf = n_buf;
     size_t extra = 0;
@@ -1655,20 +1749,20 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
       // per head is spread over them)
       int best_q = 0, best_buf = 0;
       for (int nb = max_buf; nb >= min_bufs; --nb) {
-        const size_t e = slots_bytes(2 * nb);
+        const size_t e = slots_bytes(2 * nb) + nb * x_bytes;
         if (e + 2 * stage > avail) continue;
         int q = static_cast<int>((avail - e) / stage);
         if (q > 4) q = 4;
         if (q > best_q) { best_q = q; best_buf = nb; }
       }
       n_q = best_q;
-      if (best_q >= 2) { n_buf = best_buf; n_slot = 2 * n_buf; extra = slots_bytes(n_slot); }
+      if (best_q >= 2) { n_buf = best_buf; n_slot = 2 * n_buf; extra = slots_bytes(n_slot) + n_buf * x_bytes; }
     }
     if (n_q < 2) {                                 // tight windows
       n_buf = max_buf;
       int best_d = 0;
       for (int d = 2; d >= 1 && best_d == 0; --d) {
-        const size_t e = slots_bytes(2 * d);
+        const size_t e = slots_bytes(2 * d) + n_buf * x_bytes;
         if (e + 2 * stage <= avail) {              // whole stages
           best_d = d; split = 0; extra = e; n_slot = 2 * d;
           n_q = static_cast<int>((avail - e) / stage);
