@@ -982,8 +982,6 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     const int row = (HALVES == 2) ? (16 * q + (lane & 15)) : (32 * q + lane);
     const uint32_t lane_addr = static_cast<uint32_t>(32 * q) << 16;
     const int total_chunks = p.cpl / kChunk;
-    // all chunks of every second head (uniform per warp)
-    const int my_chunks = kExtra ? kBufChunks : total_chunks;   // (... in its buffer)
     auto chunk_of = [&](int t) { return t; };
     const int key_lane0 = static_cast<int>(rank) * p.tk + half * p.cpl;        // key of this lane's column 0
     int lim = p.causal ? (txt_start + p.row0 + row + 1) : Lb;                  // keys below lim are visible
@@ -995,14 +993,14 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     // and the lane's sum of that chunk is dropped), or in part: the chunks partly visible to some
     // lane of the warp - [mix_lo, mix_hi), one or two per head and only in the CTA that holds the
     // causal triangle or the end of the sequence - get their hidden logits overwritten before the loop.
+    // Chunks that no lane of the warp sees are left out altogether, by the loop's bound: the CTA with the text keys
+    // is the last one of every head, and the others wait for its pairs.  (40 heads of 704 keys under 128 rows: 216.2 ->
+    // 198.0 us a call with the mask's loop over the mixed chunks alone; 8 x 2048, 96 rows: 86.9 -> 85.1.)
     const bool partial = lim > 0 && lim < p.cpl;
-    int lim_lo = partial ? lim : (1 << 30), lim_hi = partial ? lim : 0;
-#pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) {
-      const int a = __shfl_xor_sync(0xffffffffu, lim_lo, d), c = __shfl_xor_sync(0xffffffffu, lim_hi, d);
-      lim_lo = a < lim_lo ? a : lim_lo;
-      lim_hi = c > lim_hi ? c : lim_hi;
-    }
+    const int lim_lo = __reduce_min_sync(0xffffffffu, partial ? lim : (1 << 30));
+    const int lim_hi = __reduce_max_sync(0xffffffffu, partial ? lim : 0);
+    const int seen = (min(max(__reduce_max_sync(0xffffffffu, lim), 0), p.cpl) + kChunk - 1) / kChunk;
+    const int my_chunks = min(seen, kExtra ? kBufChunks : total_chunks);   // chunks of every second head, in its buffer
     // chunk c (columns 16c .. 16c + 15) is partly visible to a lane only if 16c < lim < 16c + 16
     const int mix_lo = lim_lo / kChunk;
     const int mix_hi = min((lim_hi + kChunk - 1) / kChunk, my_chunks);
@@ -1067,9 +1065,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         // hidden columns are overwritten in tensor memory with a huge negative number before the
         // loop, so that the loop itself carries no per-column mask.
 #pragma unroll 1
-        for (int t = 0; t < my_chunks; ++t) {
+        for (int t = mix_lo; t < mix_hi; ++t) {
           const int c = chunk_of(t);
-          if (c < mix_lo || c >= mix_hi) continue;
           const int nvis = lim - kChunk * c;
           if (t > 0) {
             tc_ld16(tbuf + kChunk * c, e);
@@ -1126,7 +1123,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         tc_st16_if(ok, tbuf + kChunk * c, e);
         stored += ok ? 1 : 0;
       }
-      if constexpr (kExtra) {
+      if (kExtra && seen > kBufChunks) {
         // the last 16 columns, from registers: like a chunk of the loop, but for the place of its exponentials
         const int nvis = lim - kChunk * kBufChunks;
 #pragma unroll
