@@ -799,12 +799,14 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       // ---------------- MMA issuer ----------------
       const uint32_t idesc_any = (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(NROWS >> 4) << 24);
       const uint32_t idesc = idesc_any | ((buf_cols >> 3) << 17);
-      // The last 16 columns of head h (keys from row 160 of the tile on), once the exp warps have taken those of
-      // head h - 2 out of their place.
+      // 176-column tiles: the place of head h's last 16 columns, free once the exp warps have taken those of head h - 2
+      // out of it (waited for before the head's first MMA: a wait that runs out leaves no MMA behind that no barrier
+      // tells about), and their MMAs (keys from row 160 of the tile on).
+      auto extra_free = [&](int h) {
+        return !kExtra || mbar_wait(smem_u32(&bars.xempty[h & 1]), (static_cast<uint32_t>(h >> 1) & 1u) ^ 1u, abort_flag, wait_limit);
+      };
       auto extra_mma = [&](int h, uint32_t q_src, uint32_t k_src, uint32_t slab_bytes) {
         if constexpr (kExtra) {
-          if (!mbar_wait(smem_u32(&bars.xempty[h & 1]), (static_cast<uint32_t>(h >> 1) & 1u) ^ 1u, abort_flag, wait_limit)) return false;
-          tc_fence_after();
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks) {
             const uint32_t slab = ks >> 2, koff = (ks & 3) * 32u;
@@ -812,7 +814,6 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                    smem_desc(k_src + slab * slab_bytes + buf_cols * 128u + koff), idesc_any | ((kExtraCols >> 3) << 17), ks > 0 ? 1u : 0u);
           }
         }
-        return true;
       };
       int committed = -1;   // last head whose MMAs were committed to its tfull barrier
       if (p.split) {
@@ -823,7 +824,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           const uint32_t bph = static_cast<uint32_t>(h / p.n_buf) & 1u;
           if (!mbar_wait(smem_u32(&bars.qfull[qi]), static_cast<uint32_t>(h / p.n_q) & 1u, abort_flag, wait_limit)) break;
           MD_TRACE(h, 1);
-          if (!mbar_wait(smem_u32(&bars.tempty[buf]), bph ^ 1u, abort_flag, wait_limit)) break;
+          if (!mbar_wait(smem_u32(&bars.tempty[buf]), bph ^ 1u, abort_flag, wait_limit) || !extra_free(h)) break;
           MD_TRACE(h, 2);
           const uint32_t q_src = stage_base + qi * q_bytes;
   #pragma unroll
@@ -844,10 +845,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
               const uint64_t bd = smem_desc(k_src + slab * (p.cpl * 128u) + koff);
               tc_mma(d, ad, bd, idesc, ks > 0 ? 1u : 0u);
             }
-            if (!extra_mma(h, q_src, k_src, static_cast<uint32_t>(p.cpl) * 128u)) {
-              ok = false;
-              break;
-            }
+            extra_mma(h, q_src, k_src, static_cast<uint32_t>(p.cpl) * 128u);
             tc_commit(smem_u32(&bars.empty[ki]));   // this half-tile may be refilled once its MMAs are done
             ++k_used;
           }
@@ -863,7 +861,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           const uint32_t bph = static_cast<uint32_t>(h / p.n_buf) & 1u;
           if (!mbar_wait(smem_u32(&bars.full[s]), ph, abort_flag, wait_limit)) break;
           MD_TRACE(h, 1);
-          if (!mbar_wait(smem_u32(&bars.tempty[buf]), bph ^ 1u, abort_flag, wait_limit)) break;
+          if (!mbar_wait(smem_u32(&bars.tempty[buf]), bph ^ 1u, abort_flag, wait_limit) || !extra_free(h)) break;
           MD_TRACE(h, 2);
           tc_fence_after();
           const uint32_t q_src = stage_base + s * stage_bytes;
@@ -880,7 +878,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
               tc_mma(d, ad, bd, idesc, ks > 0 ? 1u : 0u);
             }
           }
-          if (!extra_mma(h, q_src, k_src, static_cast<uint32_t>(p.tk) * 128u)) break;
+          extra_mma(h, q_src, k_src, static_cast<uint32_t>(p.tk) * 128u);
           tc_commit(smem_u32(&bars.empty[s]));
           tc_commit(smem_u32(&bars.tfull[buf]));
           committed = h;
