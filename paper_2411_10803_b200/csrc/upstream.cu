@@ -12,6 +12,10 @@
 // cluster's barriers, which all images of a batch reach at about the same time.
 #include <cuda_bf16.h>
 
+#include <map>
+#include <mutex>
+#include <utility>
+
 #include "mustdrop_internal.h"
 
 namespace mustdrop {
@@ -110,7 +114,9 @@ struct MergeParams {
 
 __device__ __forceinline__ int quotient(int x, uint32_t inv) { return static_cast<int>((static_cast<uint32_t>(x) * inv) >> 20); }
 
-__global__ void __launch_bounds__(kThreads, 4) spatial_merge_kernel(MergeParams p) {
+constexpr int kMergeCtas = 3;   // CTAs of the merge on an SM: registers for 128 bytes in flight per lane
+
+__global__ void __launch_bounds__(kThreads, kMergeCtas) spatial_merge_kernel(MergeParams p) {
   __shared__ unsigned char merged_flag[kMaxSlots / 4];
   __shared__ __align__(16) uint32_t emit[kWords];   // slots that emit a token: all of an unmerged window, the first of a merged one
   __shared__ int first_row[kWords];                 // output row of a word's first emitting slot
@@ -135,17 +141,29 @@ __global__ void __launch_bounds__(kThreads, 4) spatial_merge_kernel(MergeParams 
     const uint4* r3 = r2 + p.vecs;
     uint64_t acc[10] = {};   // |0|^2 |1|^2 |2|^2 |3|^2 01 | 02 03 12 13 23
 #pragma unroll 1
-    for (int x = lane; x < p.vecs; x += 32) {
-      const uint4 a = r0[x], c = r1[x], e = r2[x], f = r3[x];
-      const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, cw[4] = {c.x, c.y, c.z, c.w};
-      const uint32_t ew[4] = {e.x, e.y, e.z, e.w}, fw[4] = {f.x, f.y, f.z, f.w};
+    for (int x = lane; x < p.vecs; x += 64) {   // (two vectors of all four tokens in flight)
+      uint4 t[2][4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint64_t v0 = pack2(bf16_lo(aw[q]), bf16_hi(aw[q])), v1 = pack2(bf16_lo(cw[q]), bf16_hi(cw[q]));
-        const uint64_t v2 = pack2(bf16_lo(ew[q]), bf16_hi(ew[q])), v3 = pack2(bf16_lo(fw[q]), bf16_hi(fw[q]));
-        fma2(acc[0], v0, v0); fma2(acc[1], v1, v1); fma2(acc[2], v2, v2); fma2(acc[3], v3, v3);
-        fma2(acc[4], v0, v1); fma2(acc[5], v0, v2); fma2(acc[6], v0, v3);
-        fma2(acc[7], v1, v2); fma2(acc[8], v1, v3); fma2(acc[9], v2, v3);
+      for (int u = 0; u < 2; ++u) {
+        const int at = x + 32 * u;
+        const bool in = at < p.vecs;
+        t[u][0] = in ? r0[at] : make_uint4(0, 0, 0, 0);
+        t[u][1] = in ? r1[at] : make_uint4(0, 0, 0, 0);
+        t[u][2] = in ? r2[at] : make_uint4(0, 0, 0, 0);
+        t[u][3] = in ? r3[at] : make_uint4(0, 0, 0, 0);
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const uint32_t aw[4] = {t[u][0].x, t[u][0].y, t[u][0].z, t[u][0].w}, cw[4] = {t[u][1].x, t[u][1].y, t[u][1].z, t[u][1].w};
+        const uint32_t ew[4] = {t[u][2].x, t[u][2].y, t[u][2].z, t[u][2].w}, fw[4] = {t[u][3].x, t[u][3].y, t[u][3].z, t[u][3].w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint64_t v0 = pack2(bf16_lo(aw[q]), bf16_hi(aw[q])), v1 = pack2(bf16_lo(cw[q]), bf16_hi(cw[q]));
+          const uint64_t v2 = pack2(bf16_lo(ew[q]), bf16_hi(ew[q])), v3 = pack2(bf16_lo(fw[q]), bf16_hi(fw[q]));
+          fma2(acc[0], v0, v0); fma2(acc[1], v1, v1); fma2(acc[2], v2, v2); fma2(acc[3], v3, v3);
+          fma2(acc[4], v0, v1); fma2(acc[5], v0, v2); fma2(acc[6], v0, v3);
+          fma2(acc[7], v1, v2); fma2(acc[8], v1, v3); fma2(acc[9], v2, v3);
+        }
       }
     }
     // sums over the lanes: the half-warps exchange five sums for five, then each reduces its own five
@@ -238,19 +256,27 @@ __global__ void __launch_bounds__(kThreads, 4) spatial_merge_kernel(MergeParams 
     const uint4* r3 = r2 + p.vecs;
     uint4* dst = out + static_cast<size_t>(row_of(s)) * p.vecs;
 #pragma unroll 1
-    for (int v = lane; v < p.vecs; v += 32) {
-      const uint4 a = r0[v], c = r1[v], e = r2[v], f = r3[v];
-      const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, cw[4] = {c.x, c.y, c.z, c.w};
-      const uint32_t ew[4] = {e.x, e.y, e.z, e.w}, fw[4] = {f.x, f.y, f.z, f.w};
-      uint32_t ow[4];
+    for (int v0 = lane; v0 < p.vecs; v0 += 64) {
+      uint4 t[2][4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float lo = ((bf16_lo(aw[q]) + bf16_lo(cw[q])) + (bf16_lo(ew[q]) + bf16_lo(fw[q]))) * 0.25f;
-        const float hi = ((bf16_hi(aw[q]) + bf16_hi(cw[q])) + (bf16_hi(ew[q]) + bf16_hi(fw[q]))) * 0.25f;
-        const __nv_bfloat16 bl = __float2bfloat16_rn(lo), bh = __float2bfloat16_rn(hi);
-        ow[q] = static_cast<uint32_t>(__bfloat16_as_ushort(bl)) | (static_cast<uint32_t>(__bfloat16_as_ushort(bh)) << 16);
+      for (int u = 0; u < 2; ++u) {
+        const int at = min(v0 + 32 * u, p.vecs - 1);
+        t[u][0] = r0[at]; t[u][1] = r1[at]; t[u][2] = r2[at]; t[u][3] = r3[at];
       }
-      __stcs(dst + v, make_uint4(ow[0], ow[1], ow[2], ow[3]));
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const uint32_t aw[4] = {t[u][0].x, t[u][0].y, t[u][0].z, t[u][0].w}, cw[4] = {t[u][1].x, t[u][1].y, t[u][1].z, t[u][1].w};
+        const uint32_t ew[4] = {t[u][2].x, t[u][2].y, t[u][2].z, t[u][2].w}, fw[4] = {t[u][3].x, t[u][3].y, t[u][3].z, t[u][3].w};
+        uint32_t ow[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float lo = ((bf16_lo(aw[q]) + bf16_lo(cw[q])) + (bf16_lo(ew[q]) + bf16_lo(fw[q]))) * 0.25f;
+          const float hi = ((bf16_hi(aw[q]) + bf16_hi(cw[q])) + (bf16_hi(ew[q]) + bf16_hi(fw[q]))) * 0.25f;
+          const __nv_bfloat16 bl = __float2bfloat16_rn(lo), bh = __float2bfloat16_rn(hi);
+          ow[q] = static_cast<uint32_t>(__bfloat16_as_ushort(bl)) | (static_cast<uint32_t>(__bfloat16_as_ushort(bh)) << 16);
+        }
+        if (v0 + 32 * u < p.vecs) __stcs(dst + v0 + 32 * u, make_uint4(ow[0], ow[1], ow[2], ow[3]));
+      }
     }
   }
 }
@@ -552,6 +578,35 @@ cudaError_t launch_cluster(Kernel kernel, int batch, int cluster, size_t smem, c
   return cudaLaunchKernelEx(&cfg, kernel, p);
 }
 
+// Clusters of `cluster` CTAs of the merge that the current device holds at once (processing-cluster boundaries make
+// this less than its SMs would hold); asked once per device and size.
+inline int resident_merge_clusters(int cluster) {
+  static std::mutex mu;
+  static std::map<std::pair<int, int>, int> known;   // (device, cluster size)
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess) {
+    std::lock_guard<std::mutex> lock(mu);
+    const auto it = known.find({dev, cluster});
+    if (it != known.end()) return it->second;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(cluster));
+    cfg.blockDim = dim3(kThreads);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(cluster);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, spatial_merge_kernel, &cfg) == cudaSuccess && n > 0) {
+      known[{dev, cluster}] = n;
+      return n;
+    }
+  }
+  (void)cudaGetLastError();
+  return kMergeCtas * 148 / cluster;                 // no device to ask
+}
+
 inline mustdrop_status_t finish(cudaError_t e) {
   if (e == cudaSuccess) return MUSTDROP_OK;
   set_last_cuda_error(e);
@@ -581,8 +636,15 @@ extern "C" mustdrop_status_t mustdrop_spatial_merge(int32_t batch, int32_t grid,
   p.inv_grid = ((1u << 20) + grid - 1) / grid;
   p.inv_half = ((1u << 20) + grid / 2 - 1) / (grid / 2);
   const int n_win = (grid / 2) * (grid / 2);
-  int cluster = 8;                                   // no more CTAs than there are rounds of windows for them
-  while (cluster > 1 && (cluster - 1) * kWarps >= n_win) cluster >>= 1;
+  // CTAs per image: the fewest rounds of windows in a row, over the waves of clusters that the GPU holds at once; then
+  // the most CTAs.  (64 images of 144 windows: clusters of six, three full rounds each, leave some for a second
+  // wave; 42.7 -> 36.5 us together with the loads in flight.)
+  int cluster = 1, best = 1 << 30;
+  for (int c = 1; c <= 8 && (c - 1) * kWarps < n_win; ++c) {
+    const int at_once = resident_merge_clusters(c);
+    const int rounds = (batch + at_once - 1) / at_once * ((n_win + c * kWarps - 1) / (c * kWarps));
+    if (rounds <= best) { best = rounds; cluster = c; }
+  }
   return finish(launch_cluster(spatial_merge_kernel, batch, cluster, 0, static_cast<cudaStream_t>(cuda_stream), p));
 }
 
