@@ -304,7 +304,13 @@ struct KeySetParams {
 // CTA's tokens, their maximum and the sum of their exponentials; one exchange of these statistics
 // over the cluster normalises all heads.  (Sharing the heads put six CTA-wide barriers into every
 // head and left the partial sums of all tokens to be exchanged: 36 us for 64 images of 576 tokens,
-// 16 heads x 64, where reading the keys takes 11.5 us; now 30.)
+// 16 heads x 64, where reading the keys takes 11.5 us.)
+// VPL, FLY: head dimensions of up to 96: a token's row is read by four lanes, VPL = 1, 2 or 3 vectors of 16 bytes
+// each, and a warp takes eight tokens a step, FLY steps a trip.  (A lane per vector and a power of two of lanes to a
+// token leaves 5 to 7 of 16 lanes idle at 72, 80 and 88 dimensions, and takes three or four shuffles for two or four tokens
+// instead of two for eight: 49 images of 1936 tokens, 16 x 80: 120.4 -> 67.7 us, 64 of 576: 45.8 -> 33.9; memory takes
+// 37.4 and 14.5.)  VPL = 0: larger ones, a lane per vector.
+template <int VPL, int FLY>
 __global__ void __launch_bounds__(kThreads, 4) key_set_kernel(KeySetParams p) {
   __shared__ __align__(16) float a[kMaxSlots];      // CTA 0: head-mean attention; the others: of their own tokens
   __shared__ __align__(16) uint32_t words[kWords];
@@ -333,45 +339,63 @@ __global__ void __launch_bounds__(kThreads, 4) key_set_kernel(KeySetParams p) {
   pdl_wait();
   const float inv_h = 1.0f / static_cast<float>(p.H);
   const int own = kParts * p.part, t0 = rank * own, n_own = max(0, min(own, M - t0));   // this CTA's tokens
-  // Coalesced rows: a group of `grp` lanes (the power of two >= D/8) reads one token's row as
-  // 16-byte vectors, a warp takes 32/grp consecutive tokens per step, five steps in flight (with 32 warps on
-  // an SM: eight in flight, a second trip for the ninth step of 36 tokens, took 36 us instead of 30).
-  int grp = 1;
-  while (grp < dv) grp <<= 1;
+  constexpr int kVec = VPL > 0 ? VPL : 1;
+  int grp = VPL > 0 ? 4 : 1;                        // lanes that share a token's row
+  if constexpr (VPL == 0) {
+    while (grp < dv) grp <<= 1;
+  }
   const int sub = lane & (grp - 1), tok = lane / grp, per_warp = 32 / grp;
   float* const mine = a + t0;                       // (at the place where CTA 0 wants them)
 
   for (int hb = 0; hb < p.H; hb += p.block) {
     const int nh = min(p.block, p.H - hb), units = nh * kParts;
+    // A unit's trips: the next trip's loads - of the next unit, behind a unit's last - go out before this one's
+    // products.  (Five steps of a vector each without loads ahead: 20 us until the last logit of 64 images of 576
+    // tokens, 16 heads x 64, where memory takes 11.6; the kernel 30.8 us, with loads ahead 28.5.)
+    const uint4* const k_img = p.k + (static_cast<size_t>(b) * p.H + hb) * M * dv;
+    auto fetch = [&](int u, int base, uint4 (&kv)[FLY][kVec]) {
+      const int first = (u % kParts) * p.part, n = max(0, min(p.part, n_own - first));
+      const uint4* const rows = k_img + (static_cast<size_t>(u / kParts) * M + t0 + first) * dv + sub;
+#pragma unroll
+      for (int x = 0; x < FLY; ++x) {
+        const int j = base + x * per_warp + tok;
+#pragma unroll
+        for (int v = 0; v < kVec; ++v) {
+          kv[x][v] = make_uint4(0, 0, 0, 0);
+          if (u < units && j < n && sub + v * grp < dv) kv[x][v] = rows[static_cast<size_t>(j) * dv + v * grp];
+        }
+      }
+    };
+    uint4 kv[FLY][kVec], next[FLY][kVec];
+    fetch(warp, 0, kv);
     for (int u = warp; u < units; u += kWarps) {
       const int h = hb + u / kParts, first = (u % kParts) * p.part, n = max(0, min(p.part, n_own - first));
-      uint4 qw = make_uint4(0, 0, 0, 0);
-      if (sub < dv) qw = reinterpret_cast<const uint4*>(p.q_cls)[(static_cast<size_t>(b) * p.H + h) * dv + sub];
-      const float qv[8] = {bf16_lo(qw.x), bf16_hi(qw.x), bf16_lo(qw.y), bf16_hi(qw.y),
-                           bf16_lo(qw.z), bf16_hi(qw.z), bf16_lo(qw.w), bf16_hi(qw.w)};
-      const uint4* const rows = p.k + ((static_cast<size_t>(b) * p.H + h) * M + t0 + first) * dv;
+      uint4 qw[kVec];
+#pragma unroll
+      for (int v = 0; v < kVec; ++v) {
+        qw[v] = make_uint4(0, 0, 0, 0);
+        if (sub + v * grp < dv) qw[v] = reinterpret_cast<const uint4*>(p.q_cls)[(static_cast<size_t>(b) * p.H + h) * dv + sub + v * grp];
+      }
       float* const z = logits + u * p.part;
       float mx = -INFINITY;
-      constexpr int kFly = 5;
-      for (int base = 0; base < n; base += kFly * per_warp) {   // warp-uniform trip count
-        uint4 kv[kFly];
+      for (int base = 0;; base += FLY * per_warp) {   // warp-uniform trip count, at least one
+        const bool last = base + FLY * per_warp >= n;
+        fetch(last ? u + kWarps : u, last ? 0 : base + FLY * per_warp, next);
 #pragma unroll
-        for (int x = 0; x < kFly; ++x) {
+        for (int x = 0; x < FLY; ++x) {
           const int j = base + x * per_warp + tok;
-          kv[x] = make_uint4(0, 0, 0, 0);
-          if (j < n && sub < dv) kv[x] = rows[static_cast<size_t>(j) * dv + sub];
-        }
+          float da = 0.0f;
 #pragma unroll
-        for (int x = 0; x < kFly; ++x) {
-          const int j = base + x * per_warp + tok;
-          float da = bf16_lo(kv[x].x) * qv[0];
-          da = fmaf(bf16_hi(kv[x].x), qv[1], da);
-          da = fmaf(bf16_lo(kv[x].y), qv[2], da);
-          da = fmaf(bf16_hi(kv[x].y), qv[3], da);
-          da = fmaf(bf16_lo(kv[x].z), qv[4], da);
-          da = fmaf(bf16_hi(kv[x].z), qv[5], da);
-          da = fmaf(bf16_lo(kv[x].w), qv[6], da);
-          da = fmaf(bf16_hi(kv[x].w), qv[7], da);
+          for (int v = 0; v < kVec; ++v) {
+            da = fmaf(bf16_lo(kv[x][v].x), bf16_lo(qw[v].x), da);
+            da = fmaf(bf16_hi(kv[x][v].x), bf16_hi(qw[v].x), da);
+            da = fmaf(bf16_lo(kv[x][v].y), bf16_lo(qw[v].y), da);
+            da = fmaf(bf16_hi(kv[x][v].y), bf16_hi(qw[v].y), da);
+            da = fmaf(bf16_lo(kv[x][v].z), bf16_lo(qw[v].z), da);
+            da = fmaf(bf16_hi(kv[x][v].z), bf16_hi(qw[v].z), da);
+            da = fmaf(bf16_lo(kv[x][v].w), bf16_lo(qw[v].w), da);
+            da = fmaf(bf16_hi(kv[x][v].w), bf16_hi(qw[v].w), da);
+          }
           for (int d = grp >> 1; d >= 1; d >>= 1) da += __shfl_xor_sync(0xffffffffu, da, d);   // over the group's lanes (fixed tree)
           if (j < n) {
             da *= p.scale_log2e;
@@ -379,6 +403,11 @@ __global__ void __launch_bounds__(kThreads, 4) key_set_kernel(KeySetParams p) {
             mx = fmaxf(mx, da);
           }
         }
+#pragma unroll
+        for (int x = 0; x < FLY; ++x)
+#pragma unroll
+          for (int v = 0; v < kVec; ++v) kv[x][v] = next[x][v];
+        if (last) break;
       }
 #pragma unroll
       for (int d = 16; d >= 1; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
@@ -674,7 +703,16 @@ extern "C" mustdrop_status_t mustdrop_key_set(int32_t batch, int32_t n_heads, in
   if (p.block > n_heads) p.block = n_heads;
   if (p.block < 1) p.block = 1;
   const size_t smem = p.block * per_head;
-  cudaError_t e = ensure_kernel_attributes(reinterpret_cast<const void*>(key_set_kernel), false);
+  // Four lanes to a token's row, but for 33 to 64 dimensions where the batch fills the GPU and a warp's unit is several
+  // trips long: there memory is the limit, and the kernel with a lane per vector, whose loads run ahead without
+  // spilling, is ahead (64 images of 576 tokens, 16 x 64: merge and key set 66.8 us with it, 70.9 with four lanes; 27 of 256
+  // tokens: 34.7 and 30.6; one of 576: 30.4 and 27.3).
+  const bool streams = batch * cluster >= 296 && p.part > 16;
+  auto* const kernel = head_dim <= 32                ? key_set_kernel<1, 3>
+                       : head_dim <= 64 && !streams ? key_set_kernel<2, 2>
+                       : head_dim > 64 && head_dim <= 96 ? key_set_kernel<3, 1>
+                                                         : key_set_kernel<0, 3>;
+  cudaError_t e = ensure_kernel_attributes(reinterpret_cast<const void*>(kernel), false);
   if (e != cudaSuccess) return finish(e);
-  return finish(launch_cluster(key_set_kernel, batch, cluster, smem, static_cast<cudaStream_t>(cuda_stream), p));
+  return finish(launch_cluster(kernel, batch, cluster, smem, static_cast<cudaStream_t>(cuda_stream), p));
 }
