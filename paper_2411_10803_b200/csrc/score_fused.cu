@@ -1716,7 +1716,7 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
     // two that they had when the two exp warps of a quadrant shared a head: the cost model's constants and
     // every measured plan choice rest on the stage / buffer / slot counts that this sizing gives.
     // (Not the 176-column tiles, whose third buffer's slots and exponentials need the room.)
-    const int epr = ach <= 5 || ach > 10 ? 1 : kColGroups;
+    const int epr = ach <= 5 ? 1 : kColGroups;
     // Shared memory.  Whole stages first (a head's query tile and keys recycled together): as many
     // tensor-memory buffers as the columns allow (3..8), fewer if their statistics slots (2 x
     // buffers x cluster x rows x pairs x 8 bytes) would leave no room for 2 stages; four stages
@@ -1744,14 +1744,15 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
       // per head is spread over them)
       int best_q = 0, best_buf = 0;
       for (int nb = max_buf; nb >= min_bufs; --nb) {
-        const size_t e = slots_bytes(2 * nb) + nb * x_bytes;
+        const size_t e = slots_bytes(2 * nb) / (extra_cols ? kColGroups : 1) + nb * x_bytes;
         if (e + 2 * stage > avail) continue;
+        if (extra_cols && nb == 2 && slots_bytes(2 * nb) + 2 * stage > avail) continue;   // (... and no more of two than ever)
         int q = static_cast<int>((avail - e) / stage);
         if (q > 4) q = 4;
         if (q > best_q) { best_q = q; best_buf = nb; }
       }
       n_q = best_q;
-      if (best_q >= 2) { n_buf = best_buf; n_slot = 2 * n_buf; extra = slots_bytes(n_slot) + n_buf * x_bytes; }
+      if (best_q >= 2) { n_buf = best_buf; n_slot = 2 * n_buf; extra = slots_bytes(n_slot) / (extra_cols ? kColGroups : 1) + n_buf * x_bytes; }
     }
     if (n_q < 2) {                                 // tight windows
       n_buf = max_buf;
@@ -1822,6 +1823,10 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
       // the call before has left altogether.  Calls in a row of 25 and 26 requests of 948 keys, 32 heads: 81 and
       // 103 us where one alone takes 70 (24 requests: 65); as clusters of four 71.
       if (size == 5 && r.B > 24 && r.B <= resident) est *= 1.0 + 0.2 * (r.B - 24);
+      // Tiles of 176 columns with a third buffer look faster than they are: the chunk that is kept apart takes some of it
+      // back (28 requests of 1035 keys, 8 heads, 83 rows: 96.9 us in such tiles, 88.3 in two launches, which looked a
+      // few per cent slower).  37 of 862 shapes move to them with this: 1.077 x faster in the mean, 0.965 to 1.35.
+      if (extra_cols && n_buf > 2) est *= 1.06;
       if (best < 0.0 || est < best - 1e-9) {
         best = est;
         g.halves = halves; g.cluster = c; g.groups = grp; g.tk = tk; g.cpl = cpl; g.n_q = n_q; g.n_k = n_k; g.split = split;
