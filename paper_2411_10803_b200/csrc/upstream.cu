@@ -386,15 +386,16 @@ __global__ void __launch_bounds__(kThreads, 4) key_set_kernel(KeySetParams p) {
           const int j = base + x * per_warp + tok;
           float da = 0.0f;
 #pragma unroll
-          for (int v = 0; v < kVec; ++v) {
-            da = fmaf(bf16_lo(kv[x][v].x), bf16_lo(qw[v].x), da);
-            da = fmaf(bf16_hi(kv[x][v].x), bf16_hi(qw[v].x), da);
-            da = fmaf(bf16_lo(kv[x][v].y), bf16_lo(qw[v].y), da);
-            da = fmaf(bf16_hi(kv[x][v].y), bf16_hi(qw[v].y), da);
-            da = fmaf(bf16_lo(kv[x][v].z), bf16_lo(qw[v].z), da);
-            da = fmaf(bf16_hi(kv[x][v].z), bf16_hi(qw[v].z), da);
-            da = fmaf(bf16_lo(kv[x][v].w), bf16_lo(qw[v].w), da);
-            da = fmaf(bf16_hi(kv[x][v].w), bf16_hi(qw[v].w), da);
+          for (int v = 0; v < kVec; ++v) {   // (a sum per vector: chains of eight terms, as with a lane per vector)
+            float dv8 = bf16_lo(kv[x][v].x) * bf16_lo(qw[v].x);
+            dv8 = fmaf(bf16_hi(kv[x][v].x), bf16_hi(qw[v].x), dv8);
+            dv8 = fmaf(bf16_lo(kv[x][v].y), bf16_lo(qw[v].y), dv8);
+            dv8 = fmaf(bf16_hi(kv[x][v].y), bf16_hi(qw[v].y), dv8);
+            dv8 = fmaf(bf16_lo(kv[x][v].z), bf16_lo(qw[v].z), dv8);
+            dv8 = fmaf(bf16_hi(kv[x][v].z), bf16_hi(qw[v].z), dv8);
+            dv8 = fmaf(bf16_lo(kv[x][v].w), bf16_lo(qw[v].w), dv8);
+            dv8 = fmaf(bf16_hi(kv[x][v].w), bf16_hi(qw[v].w), dv8);
+            da = v == 0 ? dv8 : da + dv8;
           }
           for (int d = grp >> 1; d >= 1; d >>= 1) da += __shfl_xor_sync(0xffffffffu, da, d);   // over the group's lanes (fixed tree)
           if (j < n) {
