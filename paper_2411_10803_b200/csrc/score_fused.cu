@@ -1715,8 +1715,10 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
     // slot size in pairs per row and CTA.  The kernel sends ONE pair per row; wide tiles keep the room for
     // two that they had when the two exp warps of a quadrant shared a head: the cost model's constants and
     // every measured plan choice rest on the stage / buffer / slot counts that this sizing gives.
-    // (Not the 176-column tiles, whose third buffer's slots and exponentials need the room.)
-    const int epr = ach <= 5 ? 1 : kColGroups;
+    // (Not the 176-column tiles, whose third buffer's slots and exponentials need the room: without it no cluster of
+    // 12 to 16 CTAs would hold them.)
+    const bool extra_cols = cpl > 10 * kChunk;               // 176-column tiles: buffers of 160, exponentials of the rest in shared memory
+    const int epr = ach <= 5 || extra_cols ? 1 : kColGroups;
     // Shared memory.  Whole stages first (a head's query tile and keys recycled together): as many
     // tensor-memory buffers as the columns allow (3..8), fewer if their statistics slots (2 x
     // buffers x cluster x rows x pairs x 8 bytes) would leave no room for 2 stages; four stages
@@ -1729,7 +1731,6 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
     const size_t ph_bytes = r.per_head_max ? static_cast<size_t>(2 * kAddWarps) * tk * sizeof(float) : 0;
     const size_t avail = 227 * 1024 - 4096 /* static */ - 1024 /* alignment */ - ph_bytes;
     auto slots_bytes = [&](int n_slot) { return static_cast<size_t>(n_slot) * c * nrows * epr * 8; };
-    const bool extra_cols = cpl > 10 * kChunk;               // 176-column tiles: buffers of 160, exponentials of the rest in shared memory
     int n_buf = extra_cols ? kExtraAt / (10 * kChunk) : kTmemCols / cpl;
     if (n_buf > kMaxBufs) n_buf = kMaxBufs;
     const int min_bufs = extra_cols ? 2 : kMinBufs;
@@ -1744,20 +1745,22 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
       // per head is spread over them)
       int best_q = 0, best_buf = 0;
       for (int nb = max_buf; nb >= min_bufs; --nb) {
-        const size_t e = slots_bytes(2 * nb) / (extra_cols ? kColGroups : 1) + nb * x_bytes;
+        const size_t e = slots_bytes(2 * nb) + nb * x_bytes;
         if (e + 2 * stage > avail) continue;
-        if (extra_cols && nb == 2 && slots_bytes(2 * nb) + 2 * stage > avail) continue;   // (... and no more of two than ever)
+        // (two buffers of 176 columns only where they fit with room for two pairs: the larger clusters that one pair
+        // lets in are slower than the plans that they replace - 19 requests of 2106 keys: 233 -> 260 us)
+        if (extra_cols && nb == 2 && kColGroups * slots_bytes(2 * nb) + 2 * stage > avail) continue;
         int q = static_cast<int>((avail - e) / stage);
         if (q > 4) q = 4;
         if (q > best_q) { best_q = q; best_buf = nb; }
       }
       n_q = best_q;
-      if (best_q >= 2) { n_buf = best_buf; n_slot = 2 * n_buf; extra = slots_bytes(n_slot) / (extra_cols ? kColGroups : 1) + n_buf * x_bytes; }
+      if (best_q >= 2) { n_buf = best_buf; n_slot = 2 * n_buf; extra = slots_bytes(n_slot) + n_buf * x_bytes; }
     }
     if (n_q < 2) {                                 // tight windows
       n_buf = max_buf;
       int best_d = 0;
-      for (int d = 2; d >= 1 && best_d == 0; --d) {
+      for (int d = extra_cols ? 1 : 2; d >= 1 && best_d == 0; --d) {   // (176 columns: two slots, as they always had there)
         const size_t e = slots_bytes(2 * d) + n_buf * x_bytes;
         if (e + 2 * stage <= avail) {              // whole stages
           best_d = d; split = 0; extra = e; n_slot = 2 * d;

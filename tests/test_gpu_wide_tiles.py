@@ -31,6 +31,24 @@ def test_wide_tiles_match_the_oracle(cluster, n_vis, n_txt, n_heads, path, monke
                               key_cnt=5, budget=n_vis // 3), path=path)
 
 
+# every cluster size holds tiles of 176 keys under more than 64 rows, with both readings of Eq. 10: the keys that
+# fill them have a plan of one launch (seven and eight CTAs: two buffers; nine and more: two statistics slots)
+@pytest.mark.parametrize("flags", [0, md.MUSTDROP_FLAG_PER_HEAD_MAX])
+@pytest.mark.parametrize("cluster,n_txt", [(6, 65), (7, 128), (8, 100), (9, 128), (11, 70), (12, 66), (14, 128), (16, 65), (16, 128)])
+def test_wide_tiles_in_large_clusters(cluster, n_txt, flags):
+    w = small(batch=2, n_vis=cluster * 176 - n_txt, n_txt=n_txt, n_heads=5, hidden=640, vis_start=0)
+    d = synth.make_batch(w, with_values=False)
+    f = md.Filter(cfg(w, flags=flags, debug_score_variant=md.MUSTDROP_DEBUG_VARIANT_FUSED, debug_cluster=cluster))
+    assert "cluster %d," % cluster in f.description and "176 keys per CTA" in f.description
+    f.score(to_dev_bf16(d["q_text"]), to_dev_bf16(d["k"]))
+    torch.cuda.synchronize()
+    assert f.device_status() == (0, 0)
+    G, I = (oracle.score_per_head if flags else oracle.score)(d["q_text"], d["k"], w.vis_start, w.n_vis, w.txt_start)
+    assert_scores_close(f.g.cpu().numpy(), G, "G")
+    assert_scores_close(f.i.cpu().numpy(), I, "I")
+    f.close()
+
+
 @pytest.mark.parametrize("flags", [0, md.MUSTDROP_FLAG_PER_HEAD_MAX])
 @pytest.mark.parametrize("jump", [0, 150, 161, 170])
 def test_logits_that_leave_the_range_in_the_last_columns(jump, flags):
