@@ -1829,6 +1829,8 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
       // Tiles of 176 columns with a third buffer look faster than they are: the chunk that is kept apart takes some of it
       // back (28 requests of 1035 keys, 8 heads, 83 rows: 96.9 us in such tiles, 88.3 in two launches, which looked a
       // few per cent slower).  37 of 862 shapes move to them with this: 1.077 x faster in the mean, 0.965 to 1.35.
+      // (With few slots as well: without it 12 of 3000 shapes - one head of 2500 to 2700 keys - would leave grid plans
+      // for clusters of sixteen, 29.6 -> 34.5 us, and forced cluster plans take 3 % longer in the mean of 290.)
       if (extra_cols && n_buf > 2) est *= 1.06;
       if (best < 0.0 || est < best - 1e-9) {
         best = est;
