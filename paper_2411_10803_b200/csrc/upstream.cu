@@ -12,9 +12,7 @@
 // cluster's barriers, which all images of a batch reach at about the same time.
 #include <cuda_bf16.h>
 
-#include <map>
-#include <mutex>
-#include <utility>
+#include <atomic>
 
 #include "mustdrop_internal.h"
 
@@ -608,33 +606,39 @@ cudaError_t launch_cluster(Kernel kernel, int batch, int cluster, size_t smem, c
   return cudaLaunchKernelEx(&cfg, kernel, p);
 }
 
+// What the calls ask a device once.  Plain words, to which every thread would store the same: the C entries take no
+// lock and allocate nothing (a container's insertion may throw).
+constexpr int kMaxDevices = 64, kMaxMergeCluster = 8;
+struct DeviceFacts {
+  std::atomic<int> merge_clusters[kMaxMergeCluster + 1];   // clusters of the merge held at once, by their size (0: not asked yet)
+};
+inline DeviceFacts& facts_of(int dev) {
+  static DeviceFacts known[kMaxDevices + 1];               // (the last one: devices beyond, asked on every call)
+  return known[dev >= 0 && dev < kMaxDevices ? dev : kMaxDevices];
+}
+
 // Clusters of `cluster` CTAs of the merge that the current device holds at once (processing-cluster boundaries make
-// this less than its SMs would hold); asked once per device and size.
-inline int resident_merge_clusters(int cluster) {
-  static std::mutex mu;
-  static std::map<std::pair<int, int>, int> known;   // (device, cluster size)
-  int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess) {
-    std::lock_guard<std::mutex> lock(mu);
-    const auto it = known.find({dev, cluster});
-    if (it != known.end()) return it->second;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(cluster));
-    cfg.blockDim = dim3(kThreads);
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = static_cast<unsigned>(cluster);
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, spatial_merge_kernel, &cfg) == cudaSuccess && n > 0) {
-      known[{dev, cluster}] = n;
-      return n;
-    }
+// this less than its SMs would hold).
+inline int resident_merge_clusters(int dev, int cluster) {
+  std::atomic<int>& known = facts_of(dev).merge_clusters[cluster];
+  int n = known.load(std::memory_order_relaxed);
+  if (n > 0) return n;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(cluster));
+  cfg.blockDim = dim3(kThreads);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(cluster);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaOccupancyMaxActiveClusters(&n, spatial_merge_kernel, &cfg) != cudaSuccess || n < 1) {
+    (void)cudaGetLastError();
+    return 1;                                              // no answer (the launch will tell): as if one fitted
   }
-  (void)cudaGetLastError();
-  return kMergeCtas * 148 / cluster;                 // no device to ask
+  if (dev >= 0 && dev < kMaxDevices) known.store(n, std::memory_order_relaxed);
+  return n;
 }
 
 inline mustdrop_status_t finish(cudaError_t e) {
@@ -669,9 +673,10 @@ extern "C" mustdrop_status_t mustdrop_spatial_merge(int32_t batch, int32_t grid,
   // CTAs per image: the fewest rounds of windows in a row, over the waves of clusters that the GPU holds at once; then
   // the most CTAs.  (64 images of 144 windows: clusters of six, three full rounds each, leave some for a second
   // wave; 42.7 -> 36.5 us together with the loads in flight.)
-  int cluster = 1, best = 1 << 30;
-  for (int c = 1; c <= 8 && (c - 1) * kWarps < n_win; ++c) {
-    const int at_once = resident_merge_clusters(c);
+  int dev = -1, cluster = 1, best = 1 << 30;
+  if (cudaGetDevice(&dev) != cudaSuccess) (void)cudaGetLastError();
+  for (int c = 1; c <= kMaxMergeCluster && (c - 1) * kWarps < n_win; ++c) {
+    const int at_once = resident_merge_clusters(dev, c);
     const int rounds = (batch + at_once - 1) / at_once * ((n_win + c * kWarps - 1) / (c * kWarps));
     if (rounds <= best) { best = rounds; cluster = c; }
   }
