@@ -15,12 +15,14 @@
 #include <atomic>
 
 #include "mustdrop_internal.h"
+#include "vision_plan.h"
 
 namespace mustdrop {
 namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
+static_assert(kWarps == kVisionWarps, "the layout rules count the warps of a CTA");
 constexpr int kMaxSlots = 4096;            // tokens per image
 constexpr int kWords = kMaxSlots / 32;     // words of a token bitmap
 
@@ -608,7 +610,7 @@ cudaError_t launch_cluster(Kernel kernel, int batch, int cluster, size_t smem, c
 
 // What the calls ask a device once.  Plain words, to which every thread would store the same: the C entries take no
 // lock and allocate nothing (a container's insertion may throw).
-constexpr int kMaxDevices = 64, kMaxMergeCluster = 8;
+constexpr int kMaxDevices = 64;
 struct DeviceFacts {
   std::atomic<int> merge_clusters[kMaxMergeCluster + 1];   // clusters of the merge held at once, by their size (0: not asked yet)
 };
@@ -670,16 +672,10 @@ extern "C" mustdrop_status_t mustdrop_spatial_merge(int32_t batch, int32_t grid,
   p.inv_grid = ((1u << 20) + grid - 1) / grid;
   p.inv_half = ((1u << 20) + grid / 2 - 1) / (grid / 2);
   const int n_win = (grid / 2) * (grid / 2);
-  // CTAs per image: the fewest rounds of windows in a row, over the waves of clusters that the GPU holds at once; then
-  // the most CTAs.  (64 images of 144 windows: clusters of six, three full rounds each, leave some for a second
-  // wave; 42.7 -> 36.5 us together with the loads in flight.)
-  int dev = -1, cluster = 1, best = 1 << 30;
+  int dev = -1, resident[kMaxMergeCluster + 1] = {};
   if (cudaGetDevice(&dev) != cudaSuccess) (void)cudaGetLastError();
-  for (int c = 1; c <= kMaxMergeCluster && (c - 1) * kWarps < n_win; ++c) {
-    const int at_once = resident_merge_clusters(dev, c);
-    const int rounds = (batch + at_once - 1) / at_once * ((n_win + c * kWarps - 1) / (c * kWarps));
-    if (rounds <= best) { best = rounds; cluster = c; }
-  }
+  for (int c = 1; c <= kMaxMergeCluster; ++c) resident[c] = resident_merge_clusters(dev, c);
+  const int cluster = merge_cluster(batch, n_win, resident);
   return finish(launch_cluster(spatial_merge_kernel, batch, cluster, 0, static_cast<cudaStream_t>(cuda_stream), p));
 }
 

@@ -1,0 +1,30 @@
+// How the vision-encoding calls are laid out on the GPU: rules on sizes alone, host code without CUDA.
+#pragma once
+
+namespace mustdrop {
+
+constexpr int kVisionWarps = 8;        // warps of a CTA of these kernels
+constexpr int kMaxMergeCluster = 8;
+
+// CTAs per image of the spatial merge: the fewest rounds of windows (one per warp) in a row, over the waves of clusters
+// that the GPU holds at once; of the same number of rounds the one with the fewest waves, whose CTAs start together; then
+// the most CTAs.  resident[c]: clusters of c CTAs held at once.  (64 images of 144 windows: clusters of six, three full
+// rounds in one wave; 42.7 -> 36.4 us together with the loads in flight.  96 of 36 windows x 512 channels: four CTAs,
+// two rounds in one wave, 10.5 us; five, one round in each of two waves, 13.5.  One of 144 x 1024: eight CTAs 13.7 us,
+// six, which take three rounds too, 15.1.)
+inline int merge_cluster(int batch, int n_win, const int* resident) {
+  int cluster = 1;
+  long best = -1, best_waves = 0;
+  for (int c = 1; c <= kMaxMergeCluster && (c - 1) * kVisionWarps < n_win; ++c) {
+    const long waves = (batch + resident[c] - 1) / resident[c];
+    const long rounds = waves * ((n_win + c * kVisionWarps - 1) / (c * kVisionWarps));
+    if (best < 0 || rounds < best || (rounds == best && waves <= best_waves)) {
+      best = rounds;
+      best_waves = waves;
+      cluster = c;
+    }
+  }
+  return cluster;
+}
+
+}  // namespace mustdrop

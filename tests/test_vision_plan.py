@@ -1,0 +1,47 @@
+"""The layout rules of the vision-encoding calls (host code without CUDA), compiled by themselves: the choices
+that timings of both sides of each line are written beside."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2411_10803_b200", "csrc")
+SOURCE = """
+#include "vision_plan.h"
+extern "C" int merge_cluster(int batch, int n_win, const int* resident) {
+  return mustdrop::merge_cluster(batch, n_win, resident);
+}
+"""
+# clusters of 1 .. 8 CTAs that a B200 holds at once with three CTAs of the merge on an SM
+THREE_ON_AN_SM = (444, 222, 142, 104, 82, 71, 56, 48)
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    if shutil.which("g++") is None:
+        pytest.skip("needs g++")
+    d = tmp_path_factory.mktemp("vision_plan")
+    (d / "rules.cpp").write_text(SOURCE)
+    so = str(d / "rules.so")
+    subprocess.check_call(["g++", "-std=c++17", "-shared", "-fPIC", "-Wall", "-Werror", "-I", CSRC, "-o", so, str(d / "rules.cpp")])
+    return ctypes.CDLL(so)
+
+
+def merge_cluster(rules, batch, n_win, resident=THREE_ON_AN_SM):
+    return rules.merge_cluster(batch, n_win, (ctypes.c_int * 9)(0, *resident))
+
+
+@pytest.mark.parametrize("batch,n_win,cluster", [
+    (96, 36, 4), (111, 36, 3), (74, 64, 5), (74, 49, 5), (157, 25, 2),   # as many rounds: the fewest waves
+    (64, 144, 6), (37, 81, 8), (1, 144, 8), (100, 64, 4), (40, 49, 7),   # fewest rounds, then the most CTAs
+    (1, 1, 1), (19, 1, 1), (16, 9, 2), (65535, 576, 1),
+])
+def test_ctas_per_image_of_the_merge(rules, batch, n_win, cluster):
+    assert merge_cluster(rules, batch, n_win) == cluster
+
+
+def test_the_merge_is_laid_out_without_an_answer_about_the_device(rules):
+    # (nothing known: one cluster at a time, whatever its size)
+    assert merge_cluster(rules, 5, 144, (1,) * 8) == 8
