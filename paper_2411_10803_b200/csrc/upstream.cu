@@ -114,9 +114,10 @@ struct MergeParams {
 
 __device__ __forceinline__ int quotient(int x, uint32_t inv) { return static_cast<int>((static_cast<uint32_t>(x) * inv) >> 20); }
 
-constexpr int kMergeCtas = 3;   // CTAs of the merge on an SM: registers for 128 bytes in flight per lane
-
-__global__ void __launch_bounds__(kThreads, kMergeCtas) spatial_merge_kernel(MergeParams p) {
+// FLY: vectors of each of a window's four tokens that a lane has in flight.  Two take the registers of a fourth CTA on
+// the SM, which rows of 32 vectors or fewer would give away for nothing.
+template <int FLY>
+__global__ void __launch_bounds__(kThreads, FLY == 2 ? 3 : 4) spatial_merge_kernel(MergeParams p) {
   __shared__ unsigned char merged_flag[kMaxSlots / 4];
   __shared__ __align__(16) uint32_t emit[kWords];   // slots that emit a token: all of an unmerged window, the first of a merged one
   __shared__ int first_row[kWords];                 // output row of a word's first emitting slot
@@ -141,10 +142,10 @@ __global__ void __launch_bounds__(kThreads, kMergeCtas) spatial_merge_kernel(Mer
     const uint4* r3 = r2 + p.vecs;
     uint64_t acc[10] = {};   // |0|^2 |1|^2 |2|^2 |3|^2 01 | 02 03 12 13 23
 #pragma unroll 1
-    for (int x = lane; x < p.vecs; x += 64) {   // (two vectors of all four tokens in flight)
-      uint4 t[2][4];
+    for (int x = lane; x < p.vecs; x += 32 * FLY) {
+      uint4 t[FLY][4];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
+      for (int u = 0; u < FLY; ++u) {
         const int at = x + 32 * u;
         const bool in = at < p.vecs;
         t[u][0] = in ? r0[at] : make_uint4(0, 0, 0, 0);
@@ -153,7 +154,7 @@ __global__ void __launch_bounds__(kThreads, kMergeCtas) spatial_merge_kernel(Mer
         t[u][3] = in ? r3[at] : make_uint4(0, 0, 0, 0);
       }
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
+      for (int u = 0; u < FLY; ++u) {
         const uint32_t aw[4] = {t[u][0].x, t[u][0].y, t[u][0].z, t[u][0].w}, cw[4] = {t[u][1].x, t[u][1].y, t[u][1].z, t[u][1].w};
         const uint32_t ew[4] = {t[u][2].x, t[u][2].y, t[u][2].z, t[u][2].w}, fw[4] = {t[u][3].x, t[u][3].y, t[u][3].z, t[u][3].w};
 #pragma unroll
@@ -256,15 +257,15 @@ __global__ void __launch_bounds__(kThreads, kMergeCtas) spatial_merge_kernel(Mer
     const uint4* r3 = r2 + p.vecs;
     uint4* dst = out + static_cast<size_t>(row_of(s)) * p.vecs;
 #pragma unroll 1
-    for (int v0 = lane; v0 < p.vecs; v0 += 64) {
-      uint4 t[2][4];
+    for (int v0 = lane; v0 < p.vecs; v0 += 32 * FLY) {
+      uint4 t[FLY][4];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
+      for (int u = 0; u < FLY; ++u) {
         const int at = min(v0 + 32 * u, p.vecs - 1);
         t[u][0] = r0[at]; t[u][1] = r1[at]; t[u][2] = r2[at]; t[u][3] = r3[at];
       }
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
+      for (int u = 0; u < FLY; ++u) {
         const uint32_t aw[4] = {t[u][0].x, t[u][0].y, t[u][0].z, t[u][0].w}, cw[4] = {t[u][1].x, t[u][1].y, t[u][1].z, t[u][1].w};
         const uint32_t ew[4] = {t[u][2].x, t[u][2].y, t[u][2].z, t[u][2].w}, fw[4] = {t[u][3].x, t[u][3].y, t[u][3].z, t[u][3].w};
         uint32_t ow[4];
@@ -612,17 +613,19 @@ cudaError_t launch_cluster(Kernel kernel, int batch, int cluster, size_t smem, c
 // lock and allocate nothing (a container's insertion may throw).
 constexpr int kMaxDevices = 64;
 struct DeviceFacts {
-  std::atomic<int> merge_clusters[kMaxMergeCluster + 1];   // clusters of the merge held at once, by their size (0: not asked yet)
+  std::atomic<int> merge_clusters[2][kMaxMergeCluster + 1];   // clusters of the merge held at once, by FLY and size (0: not asked yet)
 };
 inline DeviceFacts& facts_of(int dev) {
   static DeviceFacts known[kMaxDevices + 1];               // (the last one: devices beyond, asked on every call)
   return known[dev >= 0 && dev < kMaxDevices ? dev : kMaxDevices];
 }
 
-// Clusters of `cluster` CTAs of the merge that the current device holds at once (processing-cluster boundaries make
+using MergeKernel = void (*)(MergeParams);
+
+// Clusters of `cluster` CTAs of a merge kernel that the current device holds at once (processing-cluster boundaries make
 // this less than its SMs would hold).
-inline int resident_merge_clusters(int dev, int cluster) {
-  std::atomic<int>& known = facts_of(dev).merge_clusters[cluster];
+inline int resident_merge_clusters(int dev, MergeKernel kernel, int fly, int cluster) {
+  std::atomic<int>& known = facts_of(dev).merge_clusters[fly - 1][cluster];
   int n = known.load(std::memory_order_relaxed);
   if (n > 0) return n;
   cudaLaunchConfig_t cfg = {};
@@ -635,7 +638,7 @@ inline int resident_merge_clusters(int dev, int cluster) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaOccupancyMaxActiveClusters(&n, spatial_merge_kernel, &cfg) != cudaSuccess || n < 1) {
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
     (void)cudaGetLastError();
     return 1;                                              // no answer (the launch will tell): as if one fitted
   }
@@ -674,9 +677,11 @@ extern "C" mustdrop_status_t mustdrop_spatial_merge(int32_t batch, int32_t grid,
   const int n_win = (grid / 2) * (grid / 2);
   int dev = -1, resident[kMaxMergeCluster + 1] = {};
   if (cudaGetDevice(&dev) != cudaSuccess) (void)cudaGetLastError();
-  for (int c = 1; c <= kMaxMergeCluster; ++c) resident[c] = resident_merge_clusters(dev, c);
+  const int fly = merge_fly(p.vecs);
+  const MergeKernel kernel = fly == 2 ? spatial_merge_kernel<2> : spatial_merge_kernel<1>;
+  for (int c = 1; c <= kMaxMergeCluster; ++c) resident[c] = resident_merge_clusters(dev, kernel, fly, c);
   const int cluster = merge_cluster(batch, n_win, resident);
-  return finish(launch_cluster(spatial_merge_kernel, batch, cluster, 0, static_cast<cudaStream_t>(cuda_stream), p));
+  return finish(launch_cluster(kernel, batch, cluster, 0, static_cast<cudaStream_t>(cuda_stream), p));
 }
 
 extern "C" mustdrop_status_t mustdrop_key_set(int32_t batch, int32_t n_heads, int32_t head_dim, int32_t n_tokens,

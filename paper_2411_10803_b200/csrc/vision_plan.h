@@ -6,6 +6,12 @@ namespace mustdrop {
 constexpr int kVisionWarps = 8;        // warps of a CTA of these kernels
 constexpr int kMaxMergeCluster = 8;
 
+// Vectors of each of a window's four tokens that a lane of the spatial merge has in flight, for rows of `vecs` vectors: a
+// second one only where a row has more than the warp's 32 (62 images of 22 x 22 tokens x 96 channels: 13.2 us with one
+// and four CTAs on an SM, 16.4 with two and three; 3 of 48 x 48 x 256: 26.6 and 28.5; 8 of 16 x 16 x 320: 7.7 both; 3 of
+// 36 x 36 x 496: 20.5 and 19.0).
+inline int merge_fly(int vecs) { return vecs > 32 ? 2 : 1; }
+
 // CTAs per image of the spatial merge: the fewest rounds of windows (one per warp) in a row, over the waves of clusters
 // that the GPU holds at once; of the same number of rounds the one with the fewest waves, whose CTAs start together; then
 // the most CTAs.  resident[c]: clusters of c CTAs held at once.  (64 images of 144 windows: clusters of six, three full

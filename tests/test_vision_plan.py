@@ -10,6 +10,7 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2411_10803_b200", "csrc")
 SOURCE = """
 #include "vision_plan.h"
+extern "C" int merge_fly(int vecs) { return mustdrop::merge_fly(vecs); }
 extern "C" int merge_cluster(int batch, int n_win, const int* resident) {
   return mustdrop::merge_cluster(batch, n_win, resident);
 }
@@ -45,3 +46,7 @@ def test_ctas_per_image_of_the_merge(rules, batch, n_win, cluster):
 def test_the_merge_is_laid_out_without_an_answer_about_the_device(rules):
     # (nothing known: one cluster at a time, whatever its size)
     assert merge_cluster(rules, 5, 144, (1,) * 8) == 8
+
+
+def test_a_second_vector_in_flight_needs_rows_that_have_one(rules):
+    assert [rules.merge_fly(v) for v in (1, 2, 12, 32, 33, 64, 173)] == [1, 1, 1, 1, 2, 2, 2]
