@@ -306,12 +306,13 @@ struct KeySetParams {
 // over the cluster normalises all heads.  (Sharing the heads put six CTA-wide barriers into every
 // head and left the partial sums of all tokens to be exchanged: 36 us for 64 images of 576 tokens,
 // 16 heads x 64, where reading the keys takes 11.5 us.)
-// VPL, FLY: head dimensions of up to 96: a token's row is read by four lanes, VPL = 1, 2 or 3 vectors of 16 bytes
-// each, and a warp takes eight tokens a step, FLY steps a trip.  (A lane per vector and a power of two of lanes to a
-// token leaves 5 to 7 of 16 lanes idle at 72, 80 and 88 dimensions, and takes three or four shuffles for two or four tokens
-// instead of two for eight: 49 images of 1936 tokens, 16 x 80: 120.4 -> 67.7 us, 64 of 576: 45.8 -> 33.9; memory takes
-// 37.4 and 14.5.)  VPL = 0: larger ones, a lane per vector.
-template <int VPL, int FLY>
+// LANES, VPL, FLY: a token's row is read by LANES = 4 or 8 lanes, VPL vectors of 16 bytes each, and a warp takes 32 / LANES
+// tokens a step, FLY steps a trip.  (A lane per vector and a power of two of lanes to a token leaves 5 to 7 of 16 lanes idle
+// at 72, 80 and 88 dimensions, and takes three or four shuffles for two or four tokens instead of two for eight:
+// 49 images of 1936 tokens, 16 x 80: 120.4 -> 67.7 us, 64 of 576: 45.8 -> 33.9; memory takes 37.4 and 14.5.)  LANES = 0: a
+// lane per vector, VPL = 1.
+// AHEAD: a trip's loads go out before the products of the trip before, which takes the registers of as many loads again.
+template <int LANES, int VPL, int FLY, bool AHEAD>
 __global__ void __launch_bounds__(kThreads, 4) key_set_kernel(KeySetParams p) {
   __shared__ __align__(16) float a[kMaxSlots];      // CTA 0: head-mean attention; the others: of their own tokens
   __shared__ __align__(16) uint32_t words[kWords];
@@ -340,9 +341,8 @@ __global__ void __launch_bounds__(kThreads, 4) key_set_kernel(KeySetParams p) {
   pdl_wait();
   const float inv_h = 1.0f / static_cast<float>(p.H);
   const int own = kParts * p.part, t0 = rank * own, n_own = max(0, min(own, M - t0));   // this CTA's tokens
-  constexpr int kVec = VPL > 0 ? VPL : 1;
-  int grp = VPL > 0 ? 4 : 1;                        // lanes that share a token's row
-  if constexpr (VPL == 0) {
+  int grp = LANES > 0 ? LANES : 1;                  // lanes that share a token's row
+  if constexpr (LANES == 0) {
     while (grp < dv) grp <<= 1;
   }
   const int sub = lane & (grp - 1), tok = lane / grp, per_warp = 32 / grp;
@@ -350,30 +350,31 @@ __global__ void __launch_bounds__(kThreads, 4) key_set_kernel(KeySetParams p) {
 
   for (int hb = 0; hb < p.H; hb += p.block) {
     const int nh = min(p.block, p.H - hb), units = nh * kParts;
-    // A unit's trips: the next trip's loads - of the next unit, behind a unit's last - go out before this one's
+    // A unit's trips.  With AHEAD the next trip's loads - of the next unit, behind a unit's last - go out before this one's
     // products.  (Five steps of a vector each without loads ahead: 20 us until the last logit of 64 images of 576
     // tokens, 16 heads x 64, where memory takes 11.6; the kernel 30.8 us, with loads ahead 28.5.)
     const uint4* const k_img = p.k + (static_cast<size_t>(b) * p.H + hb) * M * dv;
-    auto fetch = [&](int u, int base, uint4 (&kv)[FLY][kVec]) {
+    auto fetch = [&](int u, int base, uint4 (&kv)[FLY][VPL]) {
       const int first = (u % kParts) * p.part, n = max(0, min(p.part, n_own - first));
       const uint4* const rows = k_img + (static_cast<size_t>(u / kParts) * M + t0 + first) * dv + sub;
 #pragma unroll
       for (int x = 0; x < FLY; ++x) {
         const int j = base + x * per_warp + tok;
 #pragma unroll
-        for (int v = 0; v < kVec; ++v) {
+        for (int v = 0; v < VPL; ++v) {
           kv[x][v] = make_uint4(0, 0, 0, 0);
           if (u < units && j < n && sub + v * grp < dv) kv[x][v] = rows[static_cast<size_t>(j) * dv + v * grp];
         }
       }
     };
-    uint4 kv[FLY][kVec], next[FLY][kVec];
-    fetch(warp, 0, kv);
+    uint4 kv[FLY][VPL];
+    [[maybe_unused]] uint4 next[FLY][VPL];
+    if constexpr (AHEAD) fetch(warp, 0, kv);
     for (int u = warp; u < units; u += kWarps) {
       const int h = hb + u / kParts, first = (u % kParts) * p.part, n = max(0, min(p.part, n_own - first));
-      uint4 qw[kVec];
+      uint4 qw[VPL];
 #pragma unroll
-      for (int v = 0; v < kVec; ++v) {
+      for (int v = 0; v < VPL; ++v) {
         qw[v] = make_uint4(0, 0, 0, 0);
         if (sub + v * grp < dv) qw[v] = reinterpret_cast<const uint4*>(p.q_cls)[(static_cast<size_t>(b) * p.H + h) * dv + sub + v * grp];
       }
@@ -381,13 +382,14 @@ __global__ void __launch_bounds__(kThreads, 4) key_set_kernel(KeySetParams p) {
       float mx = -INFINITY;
       for (int base = 0;; base += FLY * per_warp) {   // warp-uniform trip count, at least one
         const bool last = base + FLY * per_warp >= n;
-        fetch(last ? u + kWarps : u, last ? 0 : base + FLY * per_warp, next);
+        if constexpr (AHEAD) fetch(last ? u + kWarps : u, last ? 0 : base + FLY * per_warp, next);
+        else fetch(u, base, kv);
 #pragma unroll
         for (int x = 0; x < FLY; ++x) {
           const int j = base + x * per_warp + tok;
           float da = 0.0f;
 #pragma unroll
-          for (int v = 0; v < kVec; ++v) {   // (a sum per vector: chains of eight terms, as with a lane per vector)
+          for (int v = 0; v < VPL; ++v) {   // (a sum per vector: chains of eight terms, as with a lane per vector)
             float dv8 = bf16_lo(kv[x][v].x) * bf16_lo(qw[v].x);
             dv8 = fmaf(bf16_hi(kv[x][v].x), bf16_hi(qw[v].x), dv8);
             dv8 = fmaf(bf16_lo(kv[x][v].y), bf16_lo(qw[v].y), dv8);
@@ -408,7 +410,8 @@ __global__ void __launch_bounds__(kThreads, 4) key_set_kernel(KeySetParams p) {
 #pragma unroll
         for (int x = 0; x < FLY; ++x)
 #pragma unroll
-          for (int v = 0; v < kVec; ++v) kv[x][v] = next[x][v];
+          for (int v = 0; v < VPL; ++v)
+            if constexpr (AHEAD) kv[x][v] = next[x][v];
         if (last) break;
       }
 #pragma unroll
@@ -621,6 +624,7 @@ inline DeviceFacts& facts_of(int dev) {
 }
 
 using MergeKernel = void (*)(MergeParams);
+using KeySetKernel = void (*)(KeySetParams);
 
 // Clusters of `cluster` CTAs of a merge kernel that the current device holds at once (processing-cluster boundaries make
 // this less than its SMs would hold).
@@ -710,15 +714,15 @@ extern "C" mustdrop_status_t mustdrop_key_set(int32_t batch, int32_t n_heads, in
   if (p.block > n_heads) p.block = n_heads;
   if (p.block < 1) p.block = 1;
   const size_t smem = p.block * per_head;
-  // Four lanes to a token's row, but for 33 to 64 dimensions where the batch fills the GPU and a warp's unit is several
-  // trips long: there memory is the limit, and the kernel with a lane per vector, whose loads run ahead without
-  // spilling, is ahead (64 images of 576 tokens, 16 x 64: merge and key set 66.8 us with it, 70.9 with four lanes; 27 of 256
-  // tokens: 34.7 and 30.6; one of 576: 30.4 and 27.3).
-  const bool streams = batch * cluster >= 296 && p.part > 16;
-  auto* const kernel = head_dim <= 32                ? key_set_kernel<1, 3>
-                       : head_dim <= 64 && !streams ? key_set_kernel<2, 2>
-                       : head_dim > 64 && head_dim <= 96 ? key_set_kernel<3, 1>
-                                                         : key_set_kernel<0, 3>;
+  KeySetKernel kernel = nullptr;
+  switch (key_rows(head_dim, p.part, batch * cluster)) {
+    case KeyRows::kLanePerVector3Ahead: kernel = key_set_kernel<0, 1, 3, true>; break;
+    case KeyRows::kFour1x3Ahead: kernel = key_set_kernel<4, 1, 3, true>; break;
+    case KeyRows::kFour2x2Ahead: kernel = key_set_kernel<4, 2, 2, true>; break;
+    case KeyRows::kFour3x1Ahead: kernel = key_set_kernel<4, 3, 1, true>; break;
+    case KeyRows::kEight2x2: kernel = key_set_kernel<8, 2, 2, false>; break;
+    case KeyRows::kEight4x1Ahead: kernel = key_set_kernel<8, 4, 1, true>; break;
+  }
   cudaError_t e = ensure_kernel_attributes(reinterpret_cast<const void*>(kernel), false);
   if (e != cudaSuccess) return finish(e);
   return finish(launch_cluster(kernel, batch, cluster, smem, static_cast<cudaStream_t>(cuda_stream), p));

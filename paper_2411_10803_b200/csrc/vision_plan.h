@@ -33,4 +33,31 @@ inline int merge_cluster(int batch, int n_win, const int* resident) {
   return cluster;
 }
 
+// How the key set reads a token's row: a lane per vector of 16 bytes, or four or eight lanes with so many vectors each;
+// steps of the warp's 32 lanes over its tokens in a trip; whether a trip's loads go out ahead of the trip before.
+enum class KeyRows {
+  kLanePerVector3Ahead,
+  kFour1x3Ahead,
+  kFour2x2Ahead,
+  kFour3x1Ahead,
+  kEight2x2,
+  kEight4x1Ahead,
+};
+
+// part: tokens of a warp's unit of work (half of a CTA's); ctas: CTAs of the call.
+inline KeyRows key_rows(int head_dim, int part, int ctas) {
+  // Four lanes to a token's row, but for 33 to 64 dimensions where the batch fills the GPU and a warp's unit is several
+  // trips long: there memory is the limit, and the kernel with a lane per vector, whose loads run ahead without
+  // spilling, is ahead (64 images of 576 tokens, 16 x 64: merge and key set 66.8 us with it, 70.9 with four lanes; 27 of 256
+  // tokens: 34.7 and 30.6; one of 576: 30.4 and 27.3).
+  if (head_dim <= 32) return KeyRows::kFour1x3Ahead;
+  if (head_dim <= 64) return ctas >= 296 && part > 16 ? KeyRows::kLanePerVector3Ahead : KeyRows::kFour2x2Ahead;
+  if (head_dim <= 96) return KeyRows::kFour3x1Ahead;
+  // Eight lanes.  A lane per vector with three steps ahead made calls of 20 to 120 tokens a unit slower than five steps
+  // without had been (us for five steps, three ahead, eight lanes: 4 images of 300 tokens, 12 x 104 dimensions: 14.9, 16.2,
+  // 11.2; 15 of 2007, 16 x 104: 103, 114, 66; 64 of 576, 16 x 128: 44.8, 45.0, 42.8; 64 of 576, 16 x 160: 80.9, 82.5, 51.7;
+  // 12 of 1936, 12 x 256: 136, 118, 86).
+  return head_dim <= 128 ? KeyRows::kEight2x2 : KeyRows::kEight4x1Ahead;
+}
+
 }  // namespace mustdrop

@@ -11,12 +11,16 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 SOURCE = """
 #include "vision_plan.h"
 extern "C" int merge_fly(int vecs) { return mustdrop::merge_fly(vecs); }
+extern "C" int key_rows(int head_dim, int part, int ctas) { return static_cast<int>(mustdrop::key_rows(head_dim, part, ctas)); }
 extern "C" int merge_cluster(int batch, int n_win, const int* resident) {
   return mustdrop::merge_cluster(batch, n_win, resident);
 }
 """
 # clusters of 1 .. 8 CTAs that a B200 holds at once with three CTAs of the merge on an SM
 THREE_ON_AN_SM = (444, 222, 142, 104, 82, 71, 56, 48)
+
+
+(LANE_PER_VECTOR3_AHEAD, FOUR1X3_AHEAD, FOUR2X2_AHEAD, FOUR3X1_AHEAD, EIGHT2X2, EIGHT4X1_AHEAD) = range(6)   # enum KeyRows
 
 
 @pytest.fixture(scope="module")
@@ -50,3 +54,10 @@ def test_the_merge_is_laid_out_without_an_answer_about_the_device(rules):
 
 def test_a_second_vector_in_flight_needs_rows_that_have_one(rules):
     assert [rules.merge_fly(v) for v in (1, 2, 12, 32, 33, 64, 173)] == [1, 1, 1, 1, 2, 2, 2]
+
+
+@pytest.mark.parametrize("part", [1, 5, 20, 36, 127])
+@pytest.mark.parametrize("ctas", [8, 296, 512])
+def test_eight_lanes_share_rows_of_more_than_96_dimensions(rules, part, ctas):
+    assert [rules.key_rows(d, part, ctas) for d in (96, 104, 128, 136, 256)] == [FOUR3X1_AHEAD, EIGHT2X2, EIGHT2X2, EIGHT4X1_AHEAD,
+                                                                               EIGHT4X1_AHEAD]
