@@ -716,8 +716,10 @@ extern "C" mustdrop_status_t mustdrop_key_set(int32_t batch, int32_t n_heads, in
   const size_t smem = p.block * per_head;
   KeySetKernel kernel = nullptr;
   switch (key_rows(head_dim, p.part, batch * cluster)) {
+    case KeyRows::kLanePerVector5: kernel = key_set_kernel<0, 1, 5, false>; break;
     case KeyRows::kLanePerVector3Ahead: kernel = key_set_kernel<0, 1, 3, true>; break;
     case KeyRows::kFour1x3Ahead: kernel = key_set_kernel<4, 1, 3, true>; break;
+    case KeyRows::kFour1x5: kernel = key_set_kernel<4, 1, 5, false>; break;
     case KeyRows::kFour2x2Ahead: kernel = key_set_kernel<4, 2, 2, true>; break;
     case KeyRows::kFour3x1Ahead: kernel = key_set_kernel<4, 3, 1, true>; break;
     case KeyRows::kEight2x2: kernel = key_set_kernel<8, 2, 2, false>; break;

@@ -36,8 +36,10 @@ inline int merge_cluster(int batch, int n_win, const int* resident) {
 // How the key set reads a token's row: a lane per vector of 16 bytes, or four or eight lanes with so many vectors each;
 // steps of the warp's 32 lanes over its tokens in a trip; whether a trip's loads go out ahead of the trip before.
 enum class KeyRows {
+  kLanePerVector5,
   kLanePerVector3Ahead,
   kFour1x3Ahead,
+  kFour1x5,
   kFour2x2Ahead,
   kFour3x1Ahead,
   kEight2x2,
@@ -46,11 +48,22 @@ enum class KeyRows {
 
 // part: tokens of a warp's unit of work (half of a CTA's); ctas: CTAs of the call.
 inline KeyRows key_rows(int head_dim, int part, int ctas) {
+  if (head_dim <= 32) {
+    // Four lanes with a vector each, three steps ahead: 24 tokens a trip.  Up to 16 dimensions that leaves two or three of
+    // four lanes without a vector, which shows where a unit is more than one trip or, with one vector to a row, the
+    // batch fills the GPU (us for a lane per vector, four lanes; 12 images of 1936 tokens, 12 x 8: 14.2, 22.6; x 16: 17.8,
+    // 22.5; 24 of 576, 16 x 8: 14.1, 18.1; 96 of 256, 12 x 8: 18.2, 19.2; but x 16: 21.0, 19.4; 4 of 300, 12 x 16: 10.1,
+    // 9.2; x 8: 9.3, 9.2).
+    if (head_dim <= 16 && (part > 24 || (head_dim <= 8 && ctas >= 296))) return KeyRows::kLanePerVector5;
+    // Units that take two trips of three steps but one of five: five at once (24 images of 576 tokens, 16 x 24: 18.1 us
+    // with three ahead, 15.8 with five, 17.5 with a lane per vector; 40 of 400, 16 x 32: 18.0, 15.6, 17.2; longer ones are
+    // as fast with three ahead: 3 of 700, 16 x 32: 12.2, 13.7, 15.7).
+    return part > 24 && part <= 40 ? KeyRows::kFour1x5 : KeyRows::kFour1x3Ahead;
+  }
   // Four lanes to a token's row, but for 33 to 64 dimensions where the batch fills the GPU and a warp's unit is several
   // trips long: there memory is the limit, and the kernel with a lane per vector, whose loads run ahead without
   // spilling, is ahead (64 images of 576 tokens, 16 x 64: merge and key set 66.8 us with it, 70.9 with four lanes; 27 of 256
   // tokens: 34.7 and 30.6; one of 576: 30.4 and 27.3).
-  if (head_dim <= 32) return KeyRows::kFour1x3Ahead;
   if (head_dim <= 64) return ctas >= 296 && part > 16 ? KeyRows::kLanePerVector3Ahead : KeyRows::kFour2x2Ahead;
   if (head_dim <= 96) return KeyRows::kFour3x1Ahead;
   // Eight lanes.  A lane per vector with three steps ahead made calls of 20 to 120 tokens a unit slower than five steps

@@ -22,7 +22,8 @@ def _built():
 
 # four lanes to a row with one, two and three vectors each, eight with two and four, whole and short rows, and a lane per
 # vector: at 33 .. 64 where the batch fills the GPU and a warp has more than 16 tokens of a head (the last two)
-@pytest.mark.parametrize("B,H,D,M", [(1, 2, 8, 33), (1, 2, 32, 200), (2, 3, 40, 130), (1, 2, 64, 64), (1, 2, 64, 1030), (2, 3, 72, 129),
+@pytest.mark.parametrize("B,H,D,M", [(1, 2, 8, 33), (1, 2, 8, 700), (40, 2, 8, 100), (2, 3, 16, 577), (1, 2, 32, 200),
+                                     (1, 2, 24, 400), (2, 3, 32, 640), (1, 2, 32, 641), (2, 3, 40, 130), (1, 2, 64, 64), (1, 2, 64, 1030), (2, 3, 72, 129),
                                      (1, 2, 88, 577), (1, 2, 96, 257), (1, 2, 104, 100), (2, 3, 128, 777), (1, 2, 136, 300),
                                      (2, 3, 192, 250), (1, 2, 248, 1031), (1, 1, 256, 70), (37, 2, 64, 272),
                                      (38, 1, 48, 300)])

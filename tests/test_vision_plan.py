@@ -20,7 +20,8 @@ extern "C" int merge_cluster(int batch, int n_win, const int* resident) {
 THREE_ON_AN_SM = (444, 222, 142, 104, 82, 71, 56, 48)
 
 
-(LANE_PER_VECTOR3_AHEAD, FOUR1X3_AHEAD, FOUR2X2_AHEAD, FOUR3X1_AHEAD, EIGHT2X2, EIGHT4X1_AHEAD) = range(6)   # enum KeyRows
+(LANE_PER_VECTOR5, LANE_PER_VECTOR3_AHEAD, FOUR1X3_AHEAD, FOUR1X5, FOUR2X2_AHEAD, FOUR3X1_AHEAD, EIGHT2X2,
+ EIGHT4X1_AHEAD) = range(8)                                             # enum KeyRows
 
 
 @pytest.fixture(scope="module")
@@ -61,3 +62,12 @@ def test_a_second_vector_in_flight_needs_rows_that_have_one(rules):
 def test_eight_lanes_share_rows_of_more_than_96_dimensions(rules, part, ctas):
     assert [rules.key_rows(d, part, ctas) for d in (96, 104, 128, 136, 256)] == [FOUR3X1_AHEAD, EIGHT2X2, EIGHT2X2, EIGHT4X1_AHEAD,
                                                                                EIGHT4X1_AHEAD]
+
+
+@pytest.mark.parametrize("head_dim,part,ctas,rows", [
+    (8, 121, 96, LANE_PER_VECTOR5), (16, 121, 96, LANE_PER_VECTOR5), (8, 36, 192, LANE_PER_VECTOR5), (8, 16, 768, LANE_PER_VECTOR5),
+    (16, 16, 768, FOUR1X3_AHEAD), (16, 19, 32, FOUR1X3_AHEAD), (8, 19, 32, FOUR1X3_AHEAD), (8, 25, 32, LANE_PER_VECTOR5),
+    (24, 24, 192, FOUR1X3_AHEAD), (24, 25, 192, FOUR1X5), (32, 36, 8, FOUR1X5), (32, 40, 320, FOUR1X5), (32, 41, 320, FOUR1X3_AHEAD),
+])
+def test_rows_of_up_to_32_dimensions(rules, head_dim, part, ctas, rows):
+    assert rules.key_rows(head_dim, part, ctas) == rows
