@@ -616,11 +616,24 @@ cudaError_t launch_cluster(Kernel kernel, int batch, int cluster, size_t smem, c
 // lock and allocate nothing (a container's insertion may throw).
 constexpr int kMaxDevices = 64;
 struct DeviceFacts {
+  std::atomic<int> sms;
   std::atomic<int> merge_clusters[2][kMaxMergeCluster + 1];   // clusters of the merge held at once, by FLY and size (0: not asked yet)
 };
 inline DeviceFacts& facts_of(int dev) {
   static DeviceFacts known[kMaxDevices + 1];               // (the last one: devices beyond, asked on every call)
   return known[dev >= 0 && dev < kMaxDevices ? dev : kMaxDevices];
+}
+
+inline int sm_count(int dev) {
+  std::atomic<int>& known = facts_of(dev).sms;
+  int n = known.load(std::memory_order_relaxed);
+  if (n > 0) return n;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) {
+    (void)cudaGetLastError();
+    return 1;
+  }
+  if (dev >= 0 && dev < kMaxDevices) known.store(n, std::memory_order_relaxed);
+  return n;
 }
 
 using MergeKernel = void (*)(MergeParams);
@@ -714,12 +727,15 @@ extern "C" mustdrop_status_t mustdrop_key_set(int32_t batch, int32_t n_heads, in
   if (p.block > n_heads) p.block = n_heads;
   if (p.block < 1) p.block = 1;
   const size_t smem = p.block * per_head;
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) (void)cudaGetLastError();
   KeySetKernel kernel = nullptr;
-  switch (key_rows(head_dim, p.part, batch * cluster)) {
+  switch (key_rows(head_dim, p.part, batch * cluster, sm_count(dev))) {
     case KeyRows::kLanePerVector5: kernel = key_set_kernel<0, 1, 5, false>; break;
     case KeyRows::kLanePerVector3Ahead: kernel = key_set_kernel<0, 1, 3, true>; break;
     case KeyRows::kFour1x3Ahead: kernel = key_set_kernel<4, 1, 3, true>; break;
     case KeyRows::kFour1x5: kernel = key_set_kernel<4, 1, 5, false>; break;
+    case KeyRows::kFour2x2: kernel = key_set_kernel<4, 2, 2, false>; break;
     case KeyRows::kFour2x2Ahead: kernel = key_set_kernel<4, 2, 2, true>; break;
     case KeyRows::kFour3x1Ahead: kernel = key_set_kernel<4, 3, 1, true>; break;
     case KeyRows::kEight2x2: kernel = key_set_kernel<8, 2, 2, false>; break;

@@ -40,31 +40,41 @@ enum class KeyRows {
   kLanePerVector3Ahead,
   kFour1x3Ahead,
   kFour1x5,
+  kFour2x2,
   kFour2x2Ahead,
   kFour3x1Ahead,
   kEight2x2,
   kEight4x1Ahead,
 };
 
-// part: tokens of a warp's unit of work (half of a CTA's); ctas: CTAs of the call.
-inline KeyRows key_rows(int head_dim, int part, int ctas) {
+// part: tokens of a warp's unit of work (half of a CTA's); ctas: CTAs of the call; sms: SMs of the device.
+inline KeyRows key_rows(int head_dim, int part, int ctas, int sms) {
+  const bool full = 2L * ctas >= 5L * sms;   // five CTAs and more on two SMs
   if (head_dim <= 32) {
     // Four lanes with a vector each, three steps ahead: 24 tokens a trip.  Up to 16 dimensions that leaves two or three of
     // four lanes without a vector, which shows where a unit is more than one trip or, with one vector to a row, the
     // batch fills the GPU (us for a lane per vector, four lanes; 12 images of 1936 tokens, 12 x 8: 14.2, 22.6; x 16: 17.8,
     // 22.5; 24 of 576, 16 x 8: 14.1, 18.1; 96 of 256, 12 x 8: 18.2, 19.2; but x 16: 21.0, 19.4; 4 of 300, 12 x 16: 10.1,
     // 9.2; x 8: 9.3, 9.2).
-    if (head_dim <= 16 && (part > 24 || (head_dim <= 8 && ctas >= 296))) return KeyRows::kLanePerVector5;
+    if (head_dim <= 16 && (part > 24 || (head_dim <= 8 && full))) return KeyRows::kLanePerVector5;
     // Units that take two trips of three steps but one of five: five at once (24 images of 576 tokens, 16 x 24: 18.1 us
     // with three ahead, 15.8 with five, 17.5 with a lane per vector; 40 of 400, 16 x 32: 18.0, 15.6, 17.2; longer ones are
     // as fast with three ahead: 3 of 700, 16 x 32: 12.2, 13.7, 15.7).
     return part > 24 && part <= 40 ? KeyRows::kFour1x5 : KeyRows::kFour1x3Ahead;
   }
-  // Four lanes to a token's row, but for 33 to 64 dimensions where the batch fills the GPU and a warp's unit is several
-  // trips long: there memory is the limit, and the kernel with a lane per vector, whose loads run ahead without
-  // spilling, is ahead (64 images of 576 tokens, 16 x 64: merge and key set 66.8 us with it, 70.9 with four lanes; 27 of 256
-  // tokens: 34.7 and 30.6; one of 576: 30.4 and 27.3).
-  if (head_dim <= 64) return ctas >= 296 && part > 16 ? KeyRows::kLanePerVector3Ahead : KeyRows::kFour2x2Ahead;
+  if (head_dim <= 64) {
+    // Four lanes with two vectors each, two steps at once; the form with loads ahead spills (16 x 64 dimensions, us for five
+    // steps of a lane per vector, two steps of four lanes ahead, at once: 24 images of 576 tokens: 25.1, 24.5, 20.2; 24 of 320:
+    // 17.3, 19.3, 15.8; 39 of 1731, 12 heads: 47.3, 38.2, 33.7; 40 of 320: 17.9, 20.1, 16.8).
+    if (!full) return KeyRows::kFour2x2;
+    // Where the batch fills the GPU and the merge's writes are still on their way, whole lines of 128 bytes in flight all
+    // the time are ahead: a lane per vector, three steps ahead (merge and key set of 64 images of 576 tokens x 1024 channels,
+    // 16 x 64 dimensions: 69.3 us for two steps ahead, 75 at once, 65.5; 48 images: 62.5, 61.9, 57.0; 44, where it is not
+    // full: 54.3, 52.6, 55.6).  But for units of one trip of four lanes (64 of 256 tokens: 43.2, 45.3, 45.3), and of one trip of
+    // five steps that three would take two for (96 of 320 tokens, the key set alone: 32.2 us with five steps, 34.0).
+    if (part <= 16) return KeyRows::kFour2x2Ahead;
+    return part <= 20 ? KeyRows::kLanePerVector5 : KeyRows::kLanePerVector3Ahead;
+  }
   if (head_dim <= 96) return KeyRows::kFour3x1Ahead;
   // Eight lanes.  A lane per vector with three steps ahead made calls of 20 to 120 tokens a unit slower than five steps
   // without had been (us for five steps, three ahead, eight lanes: 4 images of 300 tokens, 12 x 104 dimensions: 14.9, 16.2,

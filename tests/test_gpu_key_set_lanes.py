@@ -21,12 +21,12 @@ def _built():
 
 
 # four lanes to a row with one, two and three vectors each, eight with two and four, whole and short rows, and a lane per
-# vector: at 33 .. 64 where the batch fills the GPU and a warp has more than 16 tokens of a head (the last two)
-@pytest.mark.parametrize("B,H,D,M", [(1, 2, 8, 33), (1, 2, 8, 700), (40, 2, 8, 100), (2, 3, 16, 577), (1, 2, 32, 200),
-                                     (1, 2, 24, 400), (2, 3, 32, 640), (1, 2, 32, 641), (2, 3, 40, 130), (1, 2, 64, 64), (1, 2, 64, 1030), (2, 3, 72, 129),
+# vector: up to 16, and at 33 .. 64 where the batch fills the GPU (the last four)
+@pytest.mark.parametrize("B,H,D,M", [(1, 2, 8, 33), (1, 2, 8, 700), (40, 2, 8, 100), (2, 3, 16, 577), (1, 2, 24, 400), (1, 2, 32, 200),
+                                     (2, 3, 32, 640), (1, 2, 32, 641), (2, 3, 40, 130), (1, 2, 64, 64), (1, 2, 64, 1030), (2, 3, 72, 129),
                                      (1, 2, 88, 577), (1, 2, 96, 257), (1, 2, 104, 100), (2, 3, 128, 777), (1, 2, 136, 300),
-                                     (2, 3, 192, 250), (1, 2, 248, 1031), (1, 1, 256, 70), (37, 2, 64, 272),
-                                     (38, 1, 48, 300)])
+                                     (2, 3, 192, 250), (1, 2, 248, 1031), (1, 1, 256, 70), (37, 2, 64, 272), (38, 1, 48, 300),
+                                     (47, 2, 64, 256), (47, 1, 48, 300), (50, 2, 64, 330), (48, 1, 40, 577)])
 def test_key_set_at_the_change_overs(B, H, D, M):
     qb, kb, _ = synth.make_cls_attention(7, B, H, D, M, min(M, 4))
     a = torch.zeros((B, M), dtype=torch.float32, device="cuda")

@@ -11,7 +11,9 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 SOURCE = """
 #include "vision_plan.h"
 extern "C" int merge_fly(int vecs) { return mustdrop::merge_fly(vecs); }
-extern "C" int key_rows(int head_dim, int part, int ctas) { return static_cast<int>(mustdrop::key_rows(head_dim, part, ctas)); }
+extern "C" int key_rows(int head_dim, int part, int ctas, int sms) {
+  return static_cast<int>(mustdrop::key_rows(head_dim, part, ctas, sms));
+}
 extern "C" int merge_cluster(int batch, int n_win, const int* resident) {
   return mustdrop::merge_cluster(batch, n_win, resident);
 }
@@ -20,8 +22,8 @@ extern "C" int merge_cluster(int batch, int n_win, const int* resident) {
 THREE_ON_AN_SM = (444, 222, 142, 104, 82, 71, 56, 48)
 
 
-(LANE_PER_VECTOR5, LANE_PER_VECTOR3_AHEAD, FOUR1X3_AHEAD, FOUR1X5, FOUR2X2_AHEAD, FOUR3X1_AHEAD, EIGHT2X2,
- EIGHT4X1_AHEAD) = range(8)                                             # enum KeyRows
+(LANE_PER_VECTOR5, LANE_PER_VECTOR3_AHEAD, FOUR1X3_AHEAD, FOUR1X5, FOUR2X2, FOUR2X2_AHEAD, FOUR3X1_AHEAD, EIGHT2X2,
+ EIGHT4X1_AHEAD) = range(9)                                             # enum KeyRows
 
 
 @pytest.fixture(scope="module")
@@ -60,7 +62,7 @@ def test_a_second_vector_in_flight_needs_rows_that_have_one(rules):
 @pytest.mark.parametrize("part", [1, 5, 20, 36, 127])
 @pytest.mark.parametrize("ctas", [8, 296, 512])
 def test_eight_lanes_share_rows_of_more_than_96_dimensions(rules, part, ctas):
-    assert [rules.key_rows(d, part, ctas) for d in (96, 104, 128, 136, 256)] == [FOUR3X1_AHEAD, EIGHT2X2, EIGHT2X2, EIGHT4X1_AHEAD,
+    assert [rules.key_rows(d, part, ctas, 148) for d in (96, 104, 128, 136, 256)] == [FOUR3X1_AHEAD, EIGHT2X2, EIGHT2X2, EIGHT4X1_AHEAD,
                                                                                EIGHT4X1_AHEAD]
 
 
@@ -70,4 +72,14 @@ def test_eight_lanes_share_rows_of_more_than_96_dimensions(rules, part, ctas):
     (24, 24, 192, FOUR1X3_AHEAD), (24, 25, 192, FOUR1X5), (32, 36, 8, FOUR1X5), (32, 40, 320, FOUR1X5), (32, 41, 320, FOUR1X3_AHEAD),
 ])
 def test_rows_of_up_to_32_dimensions(rules, head_dim, part, ctas, rows):
-    assert rules.key_rows(head_dim, part, ctas) == rows
+    assert rules.key_rows(head_dim, part, ctas, 148) == rows
+
+
+@pytest.mark.parametrize("part,ctas,sms,rows", [
+    (36, 192, 148, FOUR2X2), (109, 312, 148, FOUR2X2), (20, 320, 148, FOUR2X2), (36, 369, 148, FOUR2X2), (36, 370, 148, LANE_PER_VECTOR3_AHEAD),
+    (36, 512, 148, LANE_PER_VECTOR3_AHEAD), (36, 512, 296, FOUR2X2), (16, 512, 148, FOUR2X2_AHEAD), (17, 512, 148, LANE_PER_VECTOR5),
+    (20, 768, 148, LANE_PER_VECTOR5), (21, 768, 148, LANE_PER_VECTOR3_AHEAD),
+])
+@pytest.mark.parametrize("head_dim", [40, 64])
+def test_rows_of_33_to_64_dimensions(rules, head_dim, part, ctas, sms, rows):
+    assert rules.key_rows(head_dim, part, ctas, sms) == rows
