@@ -1126,7 +1126,10 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         const int nvis = lim - kChunk * kBufChunks;
 #pragma unroll
         for (int j = 0; j < kChunk; ++j) zx[j] = j < nvis ? zx[j] : kHidden;
-        auto exps = [&]() {
+        float psum;
+        // (One copy of the chunk's code for both goes: a second behind the rare path made the kernel spill.)
+#pragma unroll 1
+        for (bool again = false;; again = true) {
           const float sc = nvis > 0 ? p.scale_log2e : 0.0f, ns = nvis > 0 ? -sub : -INFINITY;
           const uint64_t sc2 = pack2(sc, sc), ns2 = pack2(ns, ns);
           uint64_t part2[2] = {0ull, 0ull};
@@ -1140,10 +1143,9 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           float part[4];
           unpack2(part2[0], part[0], part[1]);
           unpack2(part2[1], part[2], part[3]);
-          return nvis > 0 ? (part[0] + part[1]) + (part[2] + part[3]) : 0.0f;
-        };
-        float psum = exps();
-        if (!ok || __any_sync(0xffffffffu, !(psum < kSumLimit))) {   // rare: as in redo_rest
+          psum = nvis > 0 ? (part[0] + part[1]) + (part[2] + part[3]) : 0.0f;
+          if (again || (ok && !__any_sync(0xffffffffu, !(psum < kSumLimit)))) break;
+          // rare: as in redo_rest
           const RedoResult r = redo_rest(tbuf, kChunk, stored, my_chunks, lim, kChunk, p.scale_log2e, false, mx, lsum);
           float cm = -INFINITY;
 #pragma unroll
@@ -1153,7 +1155,6 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           const float fac = (mx == r.mx || r.mx == -INFINITY) ? 1.0f : ex2(r.mx - mx);
           if (__any_sync(0xffffffffu, fac != 1.0f)) rescale_stored(tbuf, kChunk, my_chunks, fac);
           lsum = r.l * fac;
-          psum = exps();
         }
         lsum += psum;
         float4* const to = extra_exps + static_cast<size_t>(buf) * (kExtraCols / 4) * NROWS + row;
