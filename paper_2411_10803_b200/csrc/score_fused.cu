@@ -816,7 +816,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         }
       };
       int committed = -1;   // last head whose MMAs were committed to its tfull barrier
-      if (p.split) {
+      if (!kExtra && p.split) {   // (176-column tiles have one half: where its two rings fit, two whole stages do)
         int k_used = 0;
         bool ok = true;
         for (int h = 0; h < n_heads && ok; ++h) {
@@ -824,7 +824,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           const uint32_t bph = static_cast<uint32_t>(h / p.n_buf) & 1u;
           if (!mbar_wait(smem_u32(&bars.qfull[qi]), static_cast<uint32_t>(h / p.n_q) & 1u, abort_flag, wait_limit)) break;
           MD_TRACE(h, 1);
-          if (!mbar_wait(smem_u32(&bars.tempty[buf]), bph ^ 1u, abort_flag, wait_limit) || !extra_free(h)) break;
+          if (!mbar_wait(smem_u32(&bars.tempty[buf]), bph ^ 1u, abort_flag, wait_limit)) break;
           MD_TRACE(h, 2);
           const uint32_t q_src = stage_base + qi * q_bytes;
   #pragma unroll
@@ -845,7 +845,6 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
               const uint64_t bd = smem_desc(k_src + slab * (p.cpl * 128u) + koff);
               tc_mma(d, ad, bd, idesc, ks > 0 ? 1u : 0u);
             }
-            extra_mma(h, q_src, k_src, static_cast<uint32_t>(p.cpl) * 128u);
             tc_commit(smem_u32(&bars.empty[ki]));   // this half-tile may be refilled once its MMAs are done
             ++k_used;
           }
@@ -980,7 +979,6 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     const int row = (HALVES == 2) ? (16 * q + (lane & 15)) : (32 * q + lane);
     const uint32_t lane_addr = static_cast<uint32_t>(32 * q) << 16;
     const int total_chunks = p.cpl / kChunk;
-    auto chunk_of = [&](int t) { return t; };
     const int key_lane0 = static_cast<int>(rank) * p.tk + half * p.cpl;        // key of this lane's column 0
     int lim = p.causal ? (txt_start + p.row0 + row + 1) : Lb;                  // keys below lim are visible
     lim = (lim < Lb ? lim : Lb) - key_lane0;                                   // ... as a column count of this lane
@@ -1048,7 +1046,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       constexpr float kHidden = -3.0e38f;           // logit of a column the lane must not see (finite: 0 * kHidden = 0)
       float z[kChunk], e[kChunk];
       [[maybe_unused]] float zx[kChunk];   // kExtra: the logits of the last 16 columns
-      tc_ld16(tbuf + kChunk * chunk_of(0), z);
+      tc_ld16(tbuf, z);
       if constexpr (kExtra) tc_ld16(tmem_base + static_cast<uint32_t>(kExtraAt + (h & 1) * kExtraCols) + lane_addr, zx);
       float mx = -INFINITY, sub = 0.0f;
       tc_wait_ld();
@@ -1064,15 +1062,14 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         // loop, so that the loop itself carries no per-column mask.
 #pragma unroll 1
         for (int t = mix_lo; t < mix_hi; ++t) {
-          const int c = chunk_of(t);
-          const int nvis = lim - kChunk * c;
+          const int nvis = lim - kChunk * t;
           if (t > 0) {
-            tc_ld16(tbuf + kChunk * c, e);
+            tc_ld16(tbuf + kChunk * t, e);
             tc_wait_ld();
           }
 #pragma unroll
           for (int j = 0; j < kChunk; ++j) e[j] = (j < nvis) ? (t > 0 ? e[j] : z[j]) : kHidden;
-          tc_st16(tbuf + kChunk * c, e);
+          tc_st16(tbuf + kChunk * t, e);
           if (t == 0) {
 #pragma unroll
             for (int j = 0; j < kChunk; ++j) z[j] = e[j];
@@ -1082,9 +1079,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       }
       if (my_chunks > 0) {   // stabiliser from the first chunk
         float c4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-        const int nvis = lim - kChunk * chunk_of(0);
 #pragma unroll
-        for (int j = 0; j < kChunk; ++j) c4[j & 3] = fmaxf(c4[j & 3], (j < nvis) ? z[j] : -INFINITY);
+        for (int j = 0; j < kChunk; ++j) c4[j & 3] = fmaxf(c4[j & 3], (j < lim) ? z[j] : -INFINITY);
         mx = fmaxf(fmaxf(c4[0], c4[1]), fmaxf(c4[2], c4[3])) * p.scale_log2e;   // log2 units; scale > 0 keeps the order
         if (HALVES == 2) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));  // one stabiliser per row
         sub = (mx == -INFINITY) ? 0.0f : mx;   // (first chunk all masked: so are the later ones)
@@ -1094,15 +1090,14 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       float lsum = 0.0f;
 #pragma unroll 1
       for (int t = 0; t < my_chunks; ++t) {
-        const int c = chunk_of(t);
-        const int nvis = lim - kChunk * c;                   // visible columns of this lane in this chunk
+        const int nvis = lim - kChunk * t;                   // visible columns of this lane in this chunk
         const float sc = nvis > 0 ? p.scale_log2e : 0.0f;    // nothing visible: exponent 0 * z - inf
         const float ns = nvis > 0 ? -sub : -INFINITY;
         tc_wait_ld();
         const uint64_t sc2 = pack2(sc, sc), ns2 = pack2(ns, ns);
 #pragma unroll
         for (int j = 0; j < kChunk; j += 2) unpack2(fma2(pack2(z[j], z[j + 1]), sc2, ns2), e[j], e[j + 1]);
-        if (t + 1 < my_chunks) tc_ld16(tbuf + kChunk * chunk_of(t + 1), z);
+        if (t + 1 < my_chunks) tc_ld16(tbuf + kChunk * (t + 1), z);
         uint64_t part2[2] = {0ull, 0ull};   // (two packed zeros)
 #pragma unroll
         for (int j = 0; j < kChunk; j += 2) {
@@ -1118,7 +1113,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         const float psum = nvis > 0 ? (part[0] + part[1]) + (part[2] + part[3]) : 0.0f;
         ok = ok && !__any_sync(0xffffffffu, !(psum < kSumLimit));   // (the first chunk's sum is at most 16)
         lsum += ok ? psum : 0.0f;
-        tc_st16_if(ok, tbuf + kChunk * c, e);
+        tc_st16_if(ok, tbuf + kChunk * t, e);
         stored += ok ? 1 : 0;
       }
       if (kExtra && seen > kBufChunks) {
@@ -1766,7 +1761,7 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
         if (e + 2 * stage <= avail) {              // whole stages
           best_d = d; split = 0; extra = e; n_slot = 2 * d;
           n_q = static_cast<int>((avail - e) / stage);
-        } else if (e + 2 * q_tile + (halves + 1) * k_half <= avail) {   // split rings
+        } else if (!extra_cols && e + 2 * q_tile + (halves + 1) * k_half <= avail) {   // split rings
           best_d = d; split = 1; extra = e; n_slot = 2 * d;
           n_q = 2;
           n_k = static_cast<int>((avail - e - 2 * q_tile) / k_half);
