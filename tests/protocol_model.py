@@ -9,6 +9,7 @@ role, joined by the barriers
     eready            the exponentials of a head are in the buffer
     tempty            the buffer is free again
     sfull             every CTA's (max, sum) pair of a head has arrived in a slot    (n_slot slots)
+    xempty            the place of a head's last columns is free again               (176-column tiles: 2 places)
 with the phase-parity waits, the transaction counts of the asynchronous statistics stores, the
 hand-over (an exp group hands a head's exponentials to the add role at once; ``handover="late"``
 models the alternative - only when the group has got to its NEXT head, two heads on - which ends
@@ -17,6 +18,12 @@ in time-outs with two buffers: that next head needs the very same buffer), the
 slots) and the bounded waits: a wait that runs out raises the CTA's abort flag, every other wait
 of that CTA then returns at once, the CTA records a time-out, tells its peers before the exit
 barrier of the cluster, and the request is marked invalid (kept_cnt = -1).
+
+Tiles of 176 columns (``extra=True``): the logits of a head's last columns go to one of two places of
+their own, and the exp role gives a place back as soon as it has taken them into registers - behind its
+wait for ``tfull``, and under the tight rule behind the wait for the add role as well; the MMA role
+waits for the place that head h - 2 used.  ``keep_place=True``: the exp role gives it back only at its
+next head, two heads on, whose MMAs wait for it - every wait runs out.
 
 Grid plans (``grid=True``): the CTAs of the request are no cluster; the exp role leaves its pair in
 the CTA's own memory and arrives on ``gsent``; a publishing role stores the pair to (modelled)
@@ -90,6 +97,8 @@ class Cta:
         self.eready = [Mbarrier(1) for _ in range(geo["n_buf"])]
         self.tempty = [Mbarrier(1) for _ in range(geo["n_buf"])]
         self.sfull = [Mbarrier(1) for _ in range(geo["n_slot"])]
+        self.xempty = [Mbarrier(1) for _ in range(2)]
+        self.place = [None] * 2             # head whose last columns' logits lie there
         self.gsent = [Mbarrier(1) for _ in range(geo["n_buf"])]     # grid plans: exp role -> publishing role
         self.own_pair = [None] * geo["n_buf"]
         self.stats = [[None] * geo["C"] for _ in range(geo["n_slot"])]   # head whose pair sits there
@@ -110,11 +119,11 @@ class Cta:
 
 
 class Cluster:
-    """One request: C CTAs x 4 roles.  fault = (rank, role, head, what) makes that role skip one
-    arrive ("full", "tfull", "eready", "tempty", "empty") or one statistics store ("stats")."""
+    """One request: C CTAs x 5 roles.  fault = (rank, role, head, what) makes that role skip one
+    arrive ("full", "tfull", "eready", "tempty", "empty", "xempty") or one statistics store ("stats")."""
 
     def __init__(self, C=2, H=12, n_q=2, n_buf=3, n_slot=None, tight=0, limit=0.25, fault=None, jitter=None,
-                 grid=False, handover="auto", lanes_meet=True):
+                 grid=False, handover="auto", lanes_meet=True, extra=False, keep_place=False):
         n_slot = (min(n_buf, 4) if grid else 2 * n_buf) if n_slot is None else n_slot
         self.grid = grid
         self.g_lock = threading.Lock()
@@ -124,6 +133,7 @@ class Cluster:
         # "auto": what the kernel does (at once); "late": one head of the group later
         self.eager = handover == "auto"
         self.limit, self.fault, self.jitter, self.lanes_meet = limit, fault, jitter or {}, lanes_meet
+        self.extra, self.keep_place = extra, keep_place
         self.ctas = [Cta(self, r, self.geo) for r in range(C)]
         self.errors = []
         self.cluster_abort = False
@@ -159,6 +169,8 @@ class Cluster:
                 return
             if not c.wait(c.tempty[buf], ((h // g["n_buf"]) & 1) ^ 1, self.limit):
                 return
+            if self.extra and not c.wait(c.xempty[h & 1], ((h >> 1) & 1) ^ 1, self.limit):
+                return
             self._pause(c.rank, "mma")
             if c.stage_head[s] != h:
                 raise ProtocolError("MMA of head %d found head %s staged" % (h, c.stage_head[s]))
@@ -166,6 +178,10 @@ class Cluster:
                 if c.buf_state[buf][0] != "free":
                     raise ProtocolError("buffer %d overwritten while %s" % (buf, c.buf_state[buf],))
                 c.buf_state[buf] = ("logits", h)
+                if self.extra:
+                    if c.place[h & 1] is not None:
+                        raise ProtocolError("place %d overwritten before head %s was taken" % (h & 1, c.place[h & 1]))
+                    c.place[h & 1] = h
             c.stage_head[s] = None
             if not self._skips(c.rank, "mma", h, "empty"):
                 c.empty[s].arrive()
@@ -186,6 +202,14 @@ class Cluster:
                 return
             if not self.grid:
                 c.sfull[slot].arrive(expect_tx=g["C"])    # arm: every CTA will send one pair
+            if self.extra:
+                self._pause(c.rank, "take")
+                with c.guard:
+                    if c.place[h & 1] != h:
+                        raise ProtocolError("exp role of head %d found the last columns of head %s" % (h, c.place[h & 1]))
+                    c.place[h & 1] = None
+                if not self.keep_place and not self._skips(c.rank, "exp", h, "xempty"):
+                    c.xempty[h & 1].arrive()
             if last is not None:                          # late hand-over of the group's previous head
                 if not self._skips(c.rank, "exp", last, "eready"):
                     c.eready[last % g["n_buf"]].arrive()

@@ -10,14 +10,17 @@ GEOMETRIES = [
     dict(C=2, n_q=2, n_buf=3),                       # the 7B batch-64 plan
     dict(C=4, n_q=4, n_buf=6),
     dict(C=5, n_q=2, n_buf=3),
-    dict(C=4, n_q=2, n_buf=2),                       # 176-column tiles: two buffers only
+    dict(C=4, n_q=2, n_buf=2),                       # the least number of buffers
+    dict(C=4, n_q=2, n_buf=3, extra=True),           # 176-column tiles: three buffers and a full set of slots,
+    dict(C=8, n_q=2, n_buf=2, extra=True),           # ... two where three buffers' slots do not fit,
+    dict(C=10, n_q=2, n_buf=3, n_slot=2, tight=1, extra=True),   # ... three and two slots in clusters of nine and more
     dict(C=8, n_q=3, n_buf=8),
     dict(C=10, n_q=2, n_buf=3, n_slot=4, tight=2),   # large clusters: few slots, the exp role held near the add role
     dict(C=12, n_q=2, n_buf=3, n_slot=2, tight=1),
 ]
 
 
-@pytest.mark.parametrize("geo", GEOMETRIES, ids=lambda g: "C%d_q%d_b%d_s%s" % (g["C"], g["n_q"], g["n_buf"], g.get("n_slot", "2b")))
+@pytest.mark.parametrize("geo", GEOMETRIES, ids=lambda g: "C%d_q%d_b%d_s%s%s" % (g["C"], g["n_q"], g["n_buf"], g.get("n_slot", "2b"), "_x" if g.get("extra") else ""))
 def test_protocol_completes_and_keeps_its_invariants(geo):
     cl = Cluster(H=13, limit=5.0, **geo)
     assert cl.run(), "a role never came back"
@@ -48,6 +51,22 @@ def test_a_late_hand_over_needs_a_third_buffer(n_buf, ends):
         assert all(c.status == TIMEOUT for c in cl.ctas)
 
 
+@pytest.mark.parametrize("geo", [dict(n_buf=2), dict(n_buf=3), dict(n_buf=3, n_slot=2, tight=1)],
+                         ids=lambda g: "b%d_s%s" % (g["n_buf"], g.get("n_slot", "2b")))
+@pytest.mark.parametrize("slow", [(0, "add"), (1, "take"), (0, "mma"), (1, "exp"), (1, "tma")])
+def test_the_place_of_the_last_columns_tolerates_a_slow_role(geo, slow):
+    cl = Cluster(C=3, H=11, n_q=2, limit=5.0, extra=True, jitter={slow: 0.01}, **geo)
+    assert cl.run() and cl.errors == []
+    assert all(c.added == list(range(11)) for c in cl.ctas) and cl.kept_cnt == 11
+
+
+def test_a_place_that_is_kept_times_out_everywhere():
+    cl = Cluster(C=2, H=9, n_q=2, n_buf=3, limit=0.3, extra=True, keep_place=True)
+    assert cl.run(join_limit=10.0), "a role hung instead of giving up"
+    assert cl.errors == [] and cl.kept_cnt == -1
+    assert all(c.status == TIMEOUT for c in cl.ctas)
+
+
 def test_fewer_slots_than_the_protocol_needs_is_caught_by_the_model():
     # 2 x buffers slots are needed without the tight rule: with fewer, a fast peer overwrites an unread pair
     cl = Cluster(C=2, H=16, n_q=4, n_buf=4, n_slot=4, tight=0, limit=0.3, jitter={(0, "add"): 0.01})
@@ -63,6 +82,16 @@ FAULTS = [
     (1, "exp", 1, "stats"),     # one CTA's statistics never arrive anywhere
     (0, "add", 3, "tempty"),    # a buffer is never freed
 ]
+EXTRA_FAULTS = FAULTS + [(1, "exp", 4, "xempty")]   # the place of a head's last columns is never given back
+
+
+@pytest.mark.parametrize("geo", [dict(n_buf=3), dict(n_buf=3, n_slot=2, tight=1)], ids=["full", "tight"])
+@pytest.mark.parametrize("fault", EXTRA_FAULTS, ids=lambda f: "cta%d_%s_h%d_%s" % f)
+def test_a_skipped_arrive_times_out_everywhere_with_last_columns_apart(fault, geo):
+    cl = Cluster(C=2, H=12, n_q=2, limit=0.2, fault=fault, extra=True, **geo)
+    assert cl.run(join_limit=10.0), "a role hung instead of giving up"
+    assert cl.errors == [] and cl.kept_cnt == -1
+    assert all(c.status == TIMEOUT for c in cl.ctas)
 
 
 @pytest.mark.parametrize("tight", [0, 2])
