@@ -46,8 +46,9 @@ def test_key_set_at_the_change_overs(B, H, D, M):
         assert np.array_equal(ki.cpu().numpy()[b, :n], np.nonzero(got_a > mu.cpu().numpy()[b])[0])
 
 
-# windows for three, five and seven CTAs, vectors that end in the first and in the second of a lane's pair
-@pytest.mark.parametrize("B,grid,C", [(3, 10, 512), (1, 12, 520), (2, 14, 776), (90, 24, 16)])
+# on a B200, four, five and seven CTAs per image, three and six (the last three; with one vector of a token in flight at
+# 16 channels, two at 264), vectors that end in the first and in the second of a lane's pair
+@pytest.mark.parametrize("B,grid,C", [(3, 10, 512), (1, 12, 520), (2, 14, 776), (90, 24, 16), (111, 12, 264), (64, 24, 264)])
 def test_spatial_merge_with_other_cluster_sizes(B, grid, C):
     bits = synth.make_vit_tokens(23, B, grid, C, merge_frac=0.4)
     n = grid * grid

@@ -10,6 +10,7 @@ from paper_2411_10803_b200 import build as md_build
 from paper_2411_10803_b200 import synth
 
 from parity_util import assert_scores_close, cfg, force, to_dev_bf16
+from test_gpu_layers import run_ragged_layer
 from test_gpu_parity import run_chain_and_check, small
 
 pytestmark = pytest.mark.gpu
@@ -27,8 +28,12 @@ def _built():
 @pytest.mark.parametrize("path", ["filter", "staged"])
 def test_wide_tiles_match_the_oracle(cluster, n_vis, n_txt, n_heads, path, monkeypatch):
     force(monkeypatch, variant="fused", cluster=cluster)
-    run_chain_and_check(small(batch=2, n_vis=n_vis, n_txt=n_txt, n_heads=n_heads, hidden=128 * n_heads, vis_start=0,
-                              key_cnt=5, budget=n_vis // 3), path=path)
+    w = small(batch=2, n_vis=n_vis, n_txt=n_txt, n_heads=n_heads, hidden=128 * n_heads, vis_start=0, key_cnt=5, budget=n_vis // 3)
+    f = md.Filter(cfg(w))
+    tile = (-(-w.seq_len // cluster) + 15) // 16 * 16
+    assert "cluster %d," % cluster in f.description and "%d keys per CTA" % tile in f.description
+    f.close()
+    run_chain_and_check(w, path=path)
 
 
 # every cluster size holds tiles of 176 keys under more than 64 rows, with both readings of Eq. 10: the keys that
@@ -47,6 +52,40 @@ def test_wide_tiles_in_large_clusters(cluster, n_txt, flags):
     assert_scores_close(f.g.cpu().numpy(), G, "G")
     assert_scores_close(f.i.cpu().numpy(), I, "I")
     f.close()
+
+
+@pytest.mark.parametrize("flags", [0, md.MUSTDROP_FLAG_PER_HEAD_MAX])
+@pytest.mark.parametrize("cluster,n_vis,n_txt,tail", [(2, 274, 78, 0), (3, 400, 120, 8), (9, 1484, 100, 0)])
+def test_wide_tiles_without_a_mask(cluster, n_vis, n_txt, tail, flags):
+    """Every row sees every key, those behind the text span among them."""
+    w = small(batch=2, n_vis=n_vis, n_txt=n_txt, n_heads=5, hidden=640, vis_start=0)
+    d = synth.make_batch(w, with_values=False)
+    behind = synth.f32_to_bf16_bits(np.random.default_rng(4).standard_normal((2, 5, tail, 128), dtype=np.float32))
+    k = np.concatenate([d["k"], behind], axis=2)
+    f = md.Filter(cfg(w, flags=flags, causal=0, seq_len=w.seq_len + tail, debug_score_variant=md.MUSTDROP_DEBUG_VARIANT_FUSED,
+                      debug_cluster=cluster))
+    assert "176 keys per CTA" in f.description
+    f.score(to_dev_bf16(d["q_text"]), to_dev_bf16(k))
+    torch.cuda.synchronize()
+    assert f.device_status() == (0, 0)
+    G, I = (oracle.score_per_head if flags else oracle.score)(d["q_text"], k, w.vis_start, w.n_vis, w.txt_start, False)
+    assert_scores_close(f.g.cpu().numpy(), G, "G")
+    assert_scores_close(f.i.cpu().numpy(), I, "I")
+    f.close()
+
+
+@pytest.mark.parametrize("rebuild", [False, True])
+@pytest.mark.parametrize("cluster,n_vis,n_txt,vis_cnt", [
+    (4, 576, 128, [576, 400, 60, 33]),       # sequences that end with the last tile, the third, in the second, in the first's last 16
+    (4, 600, 100, [429, 428, 251, 76]),      # ... one key into the last tile, on its edge, one short of two tiles, on the first's edge
+])
+def test_wide_tiles_that_a_short_sequence_never_reaches(cluster, n_vis, n_txt, vis_cnt, rebuild, monkeypatch):
+    force(monkeypatch, variant="fused", cluster=cluster)
+    w = small(batch=4, n_vis=n_vis, n_txt=n_txt, n_heads=5, hidden=640, vis_start=0, key_cnt=5, budget=30)
+    f = md.Filter(cfg(w))
+    assert "176 keys per CTA" in f.description
+    f.close()
+    run_ragged_layer(w, np.array(vis_cnt, np.int32), rebuild)
 
 
 @pytest.mark.parametrize("flags", [0, md.MUSTDROP_FLAG_PER_HEAD_MAX])
