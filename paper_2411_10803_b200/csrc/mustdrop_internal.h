@@ -145,6 +145,26 @@ cudaError_t launch_compact(const mustdrop_plan& p, const int32_t* kept_idx, cons
 // of more than 8 CTAs.
 cudaError_t ensure_kernel_attributes(const void* kernel, bool nonportable_cluster);
 
+// Clusters of `cluster` CTAs of a kernel that the current device holds at once (processing-cluster boundaries make this
+// less than its SMs would hold); 0 where it cannot be asked or the shape cannot launch.
+inline int ask_resident_clusters(const void* kernel, int cluster, int threads, size_t smem) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(cluster));
+  cfg.blockDim = dim3(static_cast<unsigned>(threads));
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(cluster);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess) return n;
+  (void)cudaGetLastError();
+  return 0;
+}
+
 // Remember the cudaError_t of a failed runtime call for mustdrop_last_cuda_error (per thread).
 void set_last_cuda_error(cudaError_t e);
 

@@ -1642,22 +1642,8 @@ int max_resident_clusters(int cluster) {
     (void)cudaGetLastError();
     return 0;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(cluster));
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kMinSmem;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = static_cast<unsigned>(cluster);
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return 0;
-  }
+  const int n = ask_resident_clusters(reinterpret_cast<const void*>(kernel), cluster, kThreads, kMinSmem);
+  if (n <= 0) return 0;
   known[{dev, cluster}] = n;
   return n;
 }

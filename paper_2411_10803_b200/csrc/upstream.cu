@@ -639,26 +639,12 @@ inline int sm_count(int dev) {
 using MergeKernel = void (*)(MergeParams);
 using KeySetKernel = void (*)(KeySetParams);
 
-// Clusters of `cluster` CTAs of a merge kernel that the current device holds at once (processing-cluster boundaries make
-// this less than its SMs would hold).
 inline int resident_merge_clusters(int dev, MergeKernel kernel, int fly, int cluster) {
   std::atomic<int>& known = facts_of(dev).merge_clusters[fly - 1][cluster];
   int n = known.load(std::memory_order_relaxed);
   if (n > 0) return n;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(cluster));
-  cfg.blockDim = dim3(kThreads);
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = static_cast<unsigned>(cluster);
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
-    (void)cudaGetLastError();
-    return 1;                                              // no answer (the launch will tell): as if one fitted
-  }
+  n = ask_resident_clusters(reinterpret_cast<const void*>(kernel), cluster, kThreads, 0);
+  if (n < 1) return 1;                                     // no answer (the launch will tell): as if one fitted
   if (dev >= 0 && dev < kMaxDevices) known.store(n, std::memory_order_relaxed);
   return n;
 }
