@@ -1811,9 +1811,10 @@ bool plan_score_fused(const Resolved& r, int sm_count, int forced_cluster, Fused
       // Tiles of 176 columns with a third buffer look faster than they are: the chunk that is kept apart takes some of it
       // back (28 requests of 1035 keys, 8 heads, 83 rows: 96.9 us in such tiles, 88.3 in two launches, which looked a
       // few per cent slower).  37 of 862 shapes move to them with this: 1.077 x faster in the mean, 0.965 to 1.35.
-      // (With few slots as well: without it 12 of 3000 shapes - one head of 2500 to 2700 keys - would leave grid plans
-      // for clusters of sixteen, 29.6 -> 34.5 us, and forced cluster plans take 3 % longer in the mean of 290.)
-      if (extra_cols && n_buf > 2) est *= 1.06;
+      // With few slots the exchange takes longer as well: 15 % keep 12 and 6 requests of one head on the grid plans that
+      // are faster (1441 keys: 28.6 us against 31.3 on nine CTAs; 2634: 30.7 against 34.4 on sixteen); without a factor
+      // 290 forced cluster plans take 3 % longer in the mean.
+      if (extra_cols && n_buf > 2) est *= is_tight ? 1.15 : 1.06;
       if (best < 0.0 || est < best - 1e-9) {
         best = est;
         g.halves = halves; g.cluster = c; g.groups = grp; g.tk = tk; g.cpl = cpl; g.n_q = n_q; g.n_k = n_k; g.split = split;

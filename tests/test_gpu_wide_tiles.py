@@ -54,6 +54,15 @@ def test_wide_tiles_in_large_clusters(cluster, n_txt, flags):
     f.close()
 
 
+@pytest.mark.parametrize("batch,n_vis,n_txt", [(6, 2515, 119), (6, 2598, 96), (12, 1327, 114)])
+def test_wide_tiles_with_few_slots_leave_one_head_to_grid_plans(batch, n_vis, n_txt):
+    """(A tenth faster there; the clusters of nine and sixteen looked as fast.)"""
+    w = small(batch=batch, n_vis=n_vis, n_txt=n_txt, n_heads=1, hidden=128, vis_start=0, n_salient=0, key_cnt=0, budget=n_vis // 7)
+    f = md.Filter(cfg(w))
+    assert "grid plan" in f.description
+    f.close()
+
+
 @pytest.mark.parametrize("flags", [0, md.MUSTDROP_FLAG_PER_HEAD_MAX])
 @pytest.mark.parametrize("cluster,n_vis,n_txt,tail", [(2, 274, 78, 0), (3, 400, 120, 8), (9, 1484, 100, 0)])
 def test_wide_tiles_without_a_mask(cluster, n_vis, n_txt, tail, flags):
