@@ -33,7 +33,7 @@ struct FusedGeometry {
   int32_t split;      // 1: split rings
   int32_t n_buf;      // tensor-memory buffers
   int32_t n_slot;     // statistics slots: 2 x n_buf, or 2d (d = 2 or 1) with the exp warps held within d heads of the add warps
-  int32_t ach;        // chunks of 16 columns per accumulating thread (kernel variant: 5 or 10)
+  int32_t ach;        // chunks of 16 columns per accumulating thread (kernel variant: 5, 10 or 11)
   int32_t row0, n_rows;   // the text rows this geometry's launch covers
   int32_t gx;         // 1: grid plan - the request's CTAs are ordinary CTAs of the grid (cluster = their number) and
                       //    exchange their statistics through global memory
